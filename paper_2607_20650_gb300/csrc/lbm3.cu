@@ -53,22 +53,6 @@ __global__ void k3_count(const uint32_t *links, uint32_t N, unsigned long long *
     if ((threadIdx.x & 31) == 0) atomicAdd(out, c);
 }
 
-__global__ void k3_sum3(const double *partials, int nb, double *out) {
-    if (threadIdx.x || blockIdx.x) return;
-    for (int k = 0; k < 3; ++k) {
-        double s = 0.0;
-        for (int b = 0; b < nb; ++b) s += partials[3 * b + k];
-        out[k] = s;
-    }
-}
-
-__global__ void k3_sum(const double *partials, int nb, double *out) {
-    if (threadIdx.x || blockIdx.x) return;
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += partials[b];
-    *out = s;
-}
-
 }  // namespace d3
 }  // namespace lbm
 
@@ -443,16 +427,25 @@ extern "C" lbm_status lbm3_write_populations(lbm3_lattice *L, const void *host, 
     return LBM_OK;
 }
 
+// Second pass of a reduction of `width` components, its result and the error
+// word read in one copy.
+static lbm_status finish_reduction3(lbm3_lattice *L, double *partials, int width, double *out) {
+    double r[4], *sum = partials + 3 * kReduceBlocks;
+    CK3(launch_sum_partials(partials, kReduceBlocks, width, sum, L->err, L->stream));
+    CK3(cudaMemcpyAsync(r, sum, (width + 1) * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
+    CK3(cudaStreamSynchronize(L->stream));
+    for (int w = 0; w < width; ++w) out[w] = r[w];
+    long long flag;
+    memcpy(&flag, &r[width], sizeof(flag));
+    return flag ? lbm3_check(L) : LBM_OK;
+}
+
 extern "C" lbm_status lbm3_mass(lbm3_lattice *L, double *out) {
     if (!L || !out) return lbm_fail(LBM_EINVAL, "NULL argument");
     if (state_readable(L) != LBM_OK) return LBM_EINVAL;
     double *partials = (double *)(L->ws + L->pl.partials);
     CK3(L->ops->mass(L, partials, L->stream));
-    k3_sum<<<1, 32, 0, L->stream>>>(partials, kReduceBlocks, partials + kReduceBlocks);
-    CK3(cudaGetLastError());
-    CK3(cudaMemcpyAsync(out, partials + kReduceBlocks, sizeof(double), cudaMemcpyDeviceToHost, L->stream));
-    CK3(cudaStreamSynchronize(L->stream));
-    return lbm3_check(L);
+    return finish_reduction3(L, partials, 1, out);
 }
 
 extern "C" lbm_status lbm3_force(lbm3_lattice *L, const uint8_t *d_body, double out[3]) {
@@ -460,11 +453,7 @@ extern "C" lbm_status lbm3_force(lbm3_lattice *L, const uint8_t *d_body, double 
     if (state_readable(L) != LBM_OK) return LBM_EINVAL;
     double *partials = (double *)(L->ws + L->pl.partials);
     CK3(L->ops->force(L, d_body, partials, L->stream));
-    k3_sum3<<<1, 32, 0, L->stream>>>(partials, kReduceBlocks, partials + 3 * kReduceBlocks);
-    CK3(cudaGetLastError());
-    CK3(cudaMemcpyAsync(out, partials + 3 * kReduceBlocks, 3 * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
-    CK3(cudaStreamSynchronize(L->stream));
-    return lbm3_check(L);
+    return finish_reduction3(L, partials, 3, out);
 }
 
 extern "C" lbm_status lbm3_get_info(lbm3_lattice *L, lbm_info *out) {

@@ -669,24 +669,31 @@ static lbm_status aa_state_readable(lbm_lattice *L) {
     return LBM_OK;
 }
 
+// Second pass of a reduction of `width` components, its result and the error
+// word read in one copy.
+static lbm_status finish_reduction(lbm_lattice *L, int width, double *out) {
+    double r[4];
+    CK(launch_sum_partials(L->partials, kReduceBlocks, width, L->red_out, L->err, L->stream));
+    CK(cudaMemcpyAsync(r, L->red_out, (width + 1) * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
+    CK(cudaStreamSynchronize(L->stream));
+    for (int w = 0; w < width; ++w) out[w] = r[w];
+    long long flag;
+    memcpy(&flag, &r[width], sizeof(flag));
+    return flag ? check_err(L) : LBM_OK;
+}
+
 extern "C" lbm_status lbm_mass(lbm_lattice *L, double *out) {
     if (!L || !out) return lbm_fail(LBM_EINVAL, "NULL argument");
     if (aa_state_readable(L) != LBM_OK) return LBM_EINVAL;
     CK(L->ops->mass(L->h, L->cur, L->partials, kReduceBlocks, L->stream));
-    CK(launch_sum_partials(L->partials, kReduceBlocks, 1, L->red_out, L->stream));
-    CK(cudaMemcpyAsync(out, L->red_out, sizeof(double), cudaMemcpyDeviceToHost, L->stream));
-    CK(cudaStreamSynchronize(L->stream));
-    return check_err(L);
+    return finish_reduction(L, 1, out);
 }
 
 extern "C" lbm_status lbm_force(lbm_lattice *L, const uint8_t *d_body, double out[2]) {
     if (!L || !out) return lbm_fail(LBM_EINVAL, "NULL argument");
     if (aa_state_readable(L) != LBM_OK) return LBM_EINVAL;
     CK(L->ops->force(L->h, L->cur, d_body, L->partials, kReduceBlocks, L->stream));
-    CK(launch_sum_partials(L->partials, kReduceBlocks, 2, L->red_out, L->stream));
-    CK(cudaMemcpyAsync(out, L->red_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, L->stream));
-    CK(cudaStreamSynchronize(L->stream));
-    return check_err(L);
+    return finish_reduction(L, 2, out);
 }
 
 // Host conversion between raw storage and canonical h[i*N + n].

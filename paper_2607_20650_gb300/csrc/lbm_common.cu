@@ -39,14 +39,32 @@ __global__ void k_count_fluid(const uint8_t *links, uint32_t N, unsigned long lo
     if ((threadIdx.x & 31) == 0) atomicAdd(out, c);
 }
 
-// Fixed-order sum of the per-block partials (one thread: deterministic).
-__global__ void k_sum_partials(const double *partials, int nblocks, int width, double *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Fixed-order sum of the per-block partials: kSumThreads threads add strided
+// partials, then a shuffle tree per warp and one over the warps (the same
+// order on every call, so repeated calls agree bit for bit). out[width] takes
+// the bits of the error word, so the host reads result and flag in one copy.
+// The sum is latency only (1,024 partials, 8-24 KB): on one thread it took
+// 66 us per component, the longest kernel of a force or mass read-out of up to
+// 10M nodes; as a tree it takes about 4 us for all of them.
+constexpr int kSumThreads = 256;
+__global__ void __launch_bounds__(kSumThreads) k_sum_partials(const double *partials, int nblocks, int width,
+                                                              double *out, const unsigned int *err) {
+    __shared__ double red[kSumThreads / 32];
+    const int t = (int)threadIdx.x;
     for (int w = 0; w < width; ++w) {
         double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partials[b * width + w];
-        out[w] = s;
+        for (int b = t; b < nblocks; b += kSumThreads) s += partials[b * width + w];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if ((t & 31) == 0) red[t >> 5] = s;
+        __syncthreads();
+        if (t < 32) {
+            s = t < kSumThreads / 32 ? red[t] : 0.0;
+            for (int o = kSumThreads / 64; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+            if (t == 0) out[w] = s;
+        }
+        __syncthreads();
     }
+    if (t == 0) out[width] = __longlong_as_double((long long)*err);
 }
 
 __global__ void k_bump(long long *ctr, long long by) {
@@ -82,8 +100,8 @@ cudaError_t launch_count_fluid(const uint8_t *links, int64_t N, unsigned long lo
 }
 
 cudaError_t launch_sum_partials(const double *partials, int nblocks, int width, double *out,
-                                cudaStream_t st) {
-    k_sum_partials<<<1, 32, 0, st>>>(partials, nblocks, width, out);
+                                const unsigned int *err, cudaStream_t st) {
+    k_sum_partials<<<1, kSumThreads, 0, st>>>(partials, nblocks, width, out, err);
     return cudaGetLastError();
 }
 

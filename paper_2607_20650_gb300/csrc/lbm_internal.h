@@ -87,8 +87,9 @@ cudaError_t launch_links(int nx, int ny, int bw, int be, int bs, int bn, const u
                          uint8_t *links, cudaStream_t);
 cudaError_t launch_count_fluid(const uint8_t *links, int64_t N, unsigned long long *out,
                                cudaStream_t);
+// out: width sums, then the bits of the error word.
 cudaError_t launch_sum_partials(const double *partials, int nblocks, int width, double *out,
-                                cudaStream_t);
+                                const unsigned int *err, cudaStream_t);
 cudaError_t launch_bump_counter(long long *ctr, long long by, cudaStream_t);
 cudaError_t launch_quantize(int storage, int rounding, uint64_t seed, int64_t t, const float *in,
                             void *out, float *back, int64_t count, cudaStream_t);
