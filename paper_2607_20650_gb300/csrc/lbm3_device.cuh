@@ -43,27 +43,107 @@ __host__ __device__ __forceinline__ int64_t addr(int64_t N, int64_t n, int i) {
     return (int64_t)bundle_first(i) * N + (int64_t)bundle_size(i) * n + (i - bundle_first(i));
 }
 
-template <class C> struct Consts3 {
-    C omega;
-    C hf[3];        // F/2
-    C f[3];         // F
-    C cF[Q];        // c_i . F
-    C w0, w1, w2;   // 1/3, 1/18, 1/36
-    C wl0, wl1, wl2;  // w - (C)w: rounding residuals of the weights (0 in FP64)
-    C kw0, kw1, kw2;  // (1 - omega/2) w
+// Constants of the collision: as in 2-D, one operation order per storage
+// class (FP32, FP64, 16-bit).
+template <class C> struct Relax3;
+template <> struct Relax3<float> {
+    float omega;
+    float hf[3];        // F/2
+    float f[3];         // F
+    float cF[Q];        // c_i . F
+    float w0, w1, w2;   // 1/3, 1/18, 1/36
+    float wl0, wl1, wl2;  // w - (float)w: rounding residuals of the weights
+    float kw0, kw1, kw2;  // (1 - omega/2) w
     int force;
 };
+template <> struct Relax3<double> {
+    double om1, hom;           // 1 - omega, omega/4
+    double hf[3], k[3], c[3];  // F/2, (1 - omega/2) F / 2, (1 - omega/2) F / 6
+    double o6, o18;            // omega/6, omega/18
+};
+// T = float or f2 (each value duplicated).
+template <class T> struct NarrowRelax3 {
+    T nomega;                  // -omega
+    T nw[3], nwl[3];           // -w (rest, axis, diagonal), rounded value and residual
+    T hf[3];                   // F/2
+    T a3[3], a9[3];            // 3 tau F, 9 tau F
+    T e[Q];                    // constants of the even parts, by direction (collide3_narrow)
+    T c15, c45, c3, cm3;       // 1.5, 4.5, 3, -3
+};
+
+template <class C, bool NARROW> struct Consts3 {
+    std::conditional_t<NARROW, NarrowRelax3<C>, Relax3<C>> r;
+};
+
+// Host: FP64 constants rounded once.
+inline void make_relax3(double omega, const double *F, Relax3<float> &k) {
+    const double kf = 1.0 - 0.5 * omega;
+    k.omega = (float)omega;
+    for (int d = 0; d < 3; ++d) {
+        k.hf[d] = (float)(0.5 * F[d]);
+        k.f[d] = (float)F[d];
+    }
+    k.w0 = (float)(1.0 / 3.0);
+    k.w1 = (float)(1.0 / 18.0);
+    k.w2 = (float)(1.0 / 36.0);
+    k.wl0 = (float)(1.0 / 3.0 - (double)k.w0);
+    k.wl1 = (float)(1.0 / 18.0 - (double)k.w1);
+    k.wl2 = (float)(1.0 / 36.0 - (double)k.w2);
+    k.kw0 = (float)(kf / 3.0);
+    k.kw1 = (float)(kf / 18.0);
+    k.kw2 = (float)(kf / 36.0);
+    k.force = (F[0] != 0.0 || F[1] != 0.0 || F[2] != 0.0) ? 1 : 0;
+    for (int i = 0; i < Q; ++i) k.cF[i] = (float)(cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2]);
+}
+inline void make_relax3(double omega, const double *F, Relax3<double> &q) {
+    q.om1 = 1.0 - omega;
+    const double om = 1.0 - q.om1;
+    q.hom = 0.25 * om;
+    for (int a = 0; a < 3; ++a) {
+        q.hf[a] = 0.5 * F[a];
+        q.k[a] = 0.5 * (1.0 - 0.5 * om) * F[a];
+        q.c[a] = q.k[a] / 3.0;
+    }
+    q.o6 = om / 6.0;
+    q.o18 = om / 18.0;
+}
+inline void make_relax3(double omega, const double *F, NarrowRelax3<float> &q) {
+    const double w[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
+    const bool force = F[0] != 0.0 || F[1] != 0.0 || F[2] != 0.0;
+    const double om = omega == 0.0 && force ? 0x1p-60 : omega;   // as in 2-D
+    const double k = force ? (1.0 - 0.5 * omega) / om : 0.0, tau = force ? k + 0.5 : 0.0;
+    q.nomega = (float)-om;
+    for (int s = 0; s < 3; ++s) {
+        q.nw[s] = (float)-w[s];
+        q.nwl[s] = (float)(-w[s] - (double)q.nw[s]);
+    }
+    for (int a = 0; a < 3; ++a) {
+        q.hf[a] = (float)(0.5 * F[a]);
+        q.a3[a] = (float)(3.0 * tau * F[a]);
+        q.a9[a] = (float)(9.0 * tau * F[a]);
+    }
+    const double k0 = (0.375 + 1.5 * k) * (F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
+    for (int i = 0; i < Q; ++i) {
+        const double c = cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2];
+        q.e[i] = (float)((1.125 + 4.5 * k) * c * c - k0 + 3.0 * tau * c);
+    }
+    q.c15 = 1.5f;
+    q.c45 = 4.5f;
+    q.c3 = 3.0f;
+    q.cm3 = -3.0f;
+}
 
 // Moments, Eq. 2 equilibrium (deviation form) and Eq. 1 BGK relaxation with
-// the Guo source in one fixed operation order (shared by every D3Q19 kernel):
+// the Guo source in the fixed operation order of 32-bit storage:
 //   P_i  = drho - 3/2 u^2 + cu_i (3 + 9/2 cu_i),  h*_i = g_i + omega (w_i P_i - g_i)
 //          + (1 - omega/2) w_i [cF_i (3 + 9 cu_i) - 3 u.F]
 // with cu_i formed from the one or two nonzero components of c_i, and in
 // FP32 w_i P_i formed with w_i as the rounded weight plus its residual (the
 // rounded weights alone miss sum_i w_i c_i c_i = 1/3 by ~1e-8, which would
 // make the relaxation a momentum source proportional to u).
-template <class C>
-__device__ __forceinline__ void collide3(const Consts3<C> &k, C *g, C &drho, C &ux, C &uy, C &uz) {
+__device__ __forceinline__ void collide3_ops(const Relax3<float> &k, float *g, float &drho, float &ux, float &uy,
+                                             float &uz) {
+    using C = float;
     using A = Ar<C>;
     C r = g[0];
 #pragma unroll
@@ -108,7 +188,7 @@ __device__ __forceinline__ void collide3(const Consts3<C> &k, C *g, C &drho, C &
         const C w = sq(i) == 0 ? k.w0 : (sq(i) == 1 ? k.w1 : k.w2);
         const C P = any ? A::fma(cu, A::fma(C(4.5), cu, C(3)), base) : base;
         C t = A::fma(w, P, -g[i]);
-        if (sizeof(C) == 4) t = A::fma(sq(i) == 0 ? k.wl0 : (sq(i) == 1 ? k.wl1 : k.wl2), P, t);
+        t = A::fma(sq(i) == 0 ? k.wl0 : (sq(i) == 1 ? k.wl1 : k.wl2), P, t);
         C o = A::fma(k.omega, t, g[i]);
         if (k.force && any) {
             const C kw = sq(i) == 1 ? k.kw1 : k.kw2;
@@ -120,91 +200,147 @@ __device__ __forceinline__ void collide3(const Consts3<C> &k, C *g, C &drho, C &
     }
 }
 
-// The FP32 constants of Consts3<float>, each duplicated into both lanes of a
-// packed pair, with the signs collide3_2 folds in.
-struct Consts3x2 {
-    f2 nomega, nw[3], nwl[3], kw[3];
-    f2 hf[3], f[3], cF[Q];
-    f2 c45, c3, c9, cm3, cm15, cm1;
-};
-
-inline Consts3x2 make_consts3x2(const Consts3<float> &k) {
-    Consts3x2 q;
-    q.nomega = dup2(-k.omega);
-    const float w[3] = {k.w0, k.w1, k.w2}, wl[3] = {k.wl0, k.wl1, k.wl2}, kw[3] = {k.kw0, k.kw1, k.kw2};
-    for (int s = 0; s < 3; ++s) {
-        q.nw[s] = dup2(-w[s]);
-        q.nwl[s] = dup2(-wl[s]);
-        q.kw[s] = dup2(kw[s]);
-        q.hf[s] = dup2(k.hf[s]);
-        q.f[s] = dup2(k.f[s]);
-    }
-    for (int i = 0; i < Q; ++i) q.cF[i] = dup2(k.cF[i]);
-    q.c45 = dup2(4.5f);
-    q.c3 = dup2(3.0f);
-    q.c9 = dup2(9.0f);
-    q.cm3 = dup2(-3.0f);
-    q.cm15 = dup2(-1.5f);
-    q.cm1 = dup2(-1.0f);
-    return q;
-}
-
-// collide3 on two nodes at once (packed FP32 pairs, fma.rn.f32x2 and
-// friends): the same rounded operations lane by lane, so each lane equals
-// the scalar collide3 bit for bit. The relaxation is written without
-// negated operands, t' = fma(-w, P, g) = -fma(w, P, -g) and o =
-// fma(-omega, t'', g), which IEEE rounding makes exact; a negative first
-// term of a sum is an exact product with -1.
-__device__ __forceinline__ void collide3_2(const Consts3x2 &q, int force, f2 *g, f2 &drho, f2 &ux, f2 &uy,
-                                           f2 &uz) {
-    f2 r = g[0];
-#pragma unroll
-    for (int i = 1; i < Q; ++i) r = add2(r, g[i]);
-    drho = r;
-    f2 j[3];
+// Density and momentum of the populations (without the force's half) from the
+// sums and differences of opposite directions: 39 operations instead of 45.
+template <class T>
+__device__ __forceinline__ void moments3(const T *g, T &drho, T *u) {
+    using A = Op<T>;
+    T r = g[REST];
     bool started[3] = {false, false, false};
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
+    for (int i = REST + 1; i < Q; ++i) {
+        r = A::add(r, A::add(g[i], g[opp(i)]));
+        const T d = A::sub(g[i], g[opp(i)]);
         const int c[3] = {cx(i), cy(i), cz(i)};
+        // the first term of each component has c_a = +1 (directions 10, 11, 14)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             if (!c[a]) continue;
-            if (!started[a]) {
-                j[a] = c[a] > 0 ? g[i] : mul2(g[i], q.cm1);
-                started[a] = true;
-            } else {
-                j[a] = c[a] > 0 ? add2(j[a], g[i]) : sub2(j[a], g[i]);
-            }
+            u[a] = !started[a] ? d : (c[a] > 0 ? A::add(u[a], d) : A::sub(u[a], d));
+            started[a] = true;
         }
     }
-    ux = add2(j[0], q.hf[0]);
-    uy = add2(j[1], q.hf[1]);
-    uz = add2(j[2], q.hf[2]);
-    const f2 usq = fma2(ux, ux, fma2(uy, uy, mul2(uz, uz)));
-    const f2 base = fma2(q.cm15, usq, drho);
-    const f2 m3uF = mul2(q.cm3, fma2(ux, q.f[0], fma2(uy, q.f[1], mul2(uz, q.f[2]))));
-    const f2 u[3] = {ux, uy, uz};
+    drho = r;
+}
+
+// 16-bit storage, one node or a packed pair: the 2-D form (collide_narrow) on
+// nine pairs of directions; the force enters as one constant per direction
+// added to the even part. 164 operations with or without a force; direction by
+// direction 157, and 215 with a force.
+template <class T>
+__device__ __forceinline__ void collide3_narrow(const NarrowRelax3<T> &q, T *g, T &drho, T *u) {
+    using A = Op<T>;
+    T m[3];
+    moments3(g, drho, m);
+    const T c15 = A::lit(q.c15, 1.5), c45 = A::lit(q.c45, 4.5), c3 = A::lit(q.c3, 3.0), cm3 = A::lit(q.cm3, -3.0);
+    T a3[3], a9[3];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int c[3] = {cx(i), cy(i), cz(i)};
-        f2 cu = 0;
+    for (int a = 0; a < 3; ++a) {
+        u[a] = A::add(m[a], q.hf[a]);
+        a3[a] = A::fma(c15, m[a], q.a3[a]);
+        a9[a] = A::fma(c45, m[a], q.a9[a]);
+    }
+    const T base = A::sub(drho, A::fma(a3[0], m[0], A::fma(a3[1], m[1], A::mul(a3[2], m[2]))));
+    {
+        const T P = A::add(base, q.e[REST]);
+        const T t = A::fma(q.nwl[0], P, A::fma(q.nw[0], P, g[REST]));   // g - w P
+        g[REST] = A::fma(q.nomega, t, g[REST]);
+    }
+#pragma unroll
+    for (int i = REST + 1; i < Q; ++i) {
+        // direction j of the pair (i, opp(i)) whose first nonzero component (x, y, z) is +1
+        const int j = (cx(i) ? cx(i) : (cy(i) ? cy(i) : cz(i))) > 0 ? i : opp(i);
+        const int c[3] = {cx(j), cy(j), cz(j)};
+        const int s = sq(i);
+        T mc = m[0], Ac = m[0];
         bool any = false;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             if (!c[a]) continue;
-            if (!any) cu = c[a] > 0 ? u[a] : mul2(u[a], q.cm1);
-            else cu = c[a] > 0 ? add2(cu, u[a]) : sub2(cu, u[a]);
+            mc = !any ? m[a] : (c[a] > 0 ? A::add(mc, m[a]) : A::sub(mc, m[a]));
+            Ac = !any ? a9[a] : (c[a] > 0 ? A::add(Ac, a9[a]) : A::sub(Ac, a9[a]));
             any = true;
         }
-        const int s = sq(i);
-        const f2 P = any ? fma2(cu, fma2(q.c45, cu, q.c3), base) : base;
-        f2 t = fma2(q.nw[s], P, g[i]);
-        t = fma2(q.nwl[s], P, t);
-        f2 o = fma2(q.nomega, t, g[i]);
-        if (force && any) o = fma2(q.kw[s], fma2(q.cF[i], fma2(q.c9, cu, q.c3), m3uF), o);
-        else if (force) o = fma2(q.kw[0], m3uF, o);
-        g[i] = o;
+        const T E = A::fma(Ac, mc, base);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int k = e ? opp(j) : j;
+            const T P = A::fma(e ? cm3 : c3, mc, A::add(E, q.e[k]));
+            const T t = A::fma(q.nwl[s], P, A::fma(q.nw[s], P, g[k]));
+            g[k] = A::fma(q.nomega, t, g[k]);
+        }
     }
+}
+
+// FP64: h* = (1 - omega) g + H with omega w folded into the shared parts,
+//   b = omega/4 u + (1 - omega/2) F/2,  B = omega/18 drho - (b.u)/3,
+//   O_a = omega/6 u_a + (1 - omega/2) F_a/6:
+// the axis directions take E_a = B + b_a u_a and +-O_a, the rest direction
+// 6 B, the diagonal ones of the axes a, e the even part
+// (E_a + b_e u_e)/2 +- (b_a u_e + b_e u_a)/2 and (O_a +- O_e)/2: 119
+// operations, where it was 216 with and 160 without a force.
+__device__ __forceinline__ void collide3_ops64(const Relax3<double> &q, double *g, double &drho, double *u) {
+    using A = Ar<double>;
+    moments3(g, drho, u);
+    double b[3], O[3], E[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        u[a] = A::add(u[a], q.hf[a]);
+        b[a] = A::fma(q.hom, u[a], q.k[a]);
+        O[a] = A::fma(q.o6, u[a], q.c[a]);
+    }
+    const double t = A::fma(b[0], u[0], A::fma(b[1], u[1], A::mul(b[2], u[2])));
+    const double B = A::fma(-1.0 / 3.0, t, A::mul(q.o18, drho));
+    g[REST] = A::fma(q.om1, g[REST], A::mul(6.0, B));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) E[a] = A::fma(b[a], u[a], B);
+#pragma unroll
+    for (int i = REST + 1; i < Q; ++i) {   // axis directions: +x = 10, +y = 12, +z = 16
+        if (sq(i) != 1) continue;
+        const int a = cx(i) ? 0 : (cy(i) ? 1 : 2);
+        g[i] = A::fma(q.om1, g[i], A::add(E[a], O[a]));
+        g[opp(i)] = A::fma(q.om1, g[opp(i)], A::sub(E[a], O[a]));
+    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {   // pairs of axes a < e: c = (+1, +1) and (+1, -1)
+        const int a = m == 2 ? 1 : 0, e = m == 0 ? 1 : 2;
+        const double G = A::mul(0.5, A::fma(b[e], u[e], E[a]));
+        const double X = A::fma(b[a], u[e], A::mul(b[e], u[a]));
+        const double Es = A::fma(0.5, X, G), Ed = A::fma(-0.5, X, G);
+        const double os = A::add(O[a], O[e]), od = A::sub(O[a], O[e]);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const int c[3] = {cx(i), cy(i), cz(i)};
+            if (sq(i) != 2 || c[a] != 1 || c[e] == 0) continue;
+            const double Ei = c[e] > 0 ? Es : Ed, Oi = c[e] > 0 ? os : od;
+            g[i] = A::fma(q.om1, g[i], A::fma(0.5, Oi, Ei));
+            g[opp(i)] = A::fma(q.om1, g[opp(i)], A::fma(-0.5, Oi, Ei));
+        }
+    }
+}
+
+// The collision of a storage class.
+template <class C, bool NARROW>
+__device__ __forceinline__ void collide3(const Consts3<C, NARROW> &k, C *g, C &drho, C &ux, C &uy, C &uz) {
+    if constexpr (NARROW || sizeof(C) == 8) {
+        C u[3];
+        if constexpr (NARROW) collide3_narrow(k.r, g, drho, u);
+        else collide3_ops64(k.r, g, drho, u);
+        ux = u[0];
+        uy = u[1];
+        uz = u[2];
+    } else {
+        collide3_ops(k.r, g, drho, ux, uy, uz);
+    }
+}
+
+// Two nodes of 16-bit storage at once: each lane equals the one-node form bit for bit.
+__device__ __forceinline__ void collide3_2(const NarrowRelax3<f2> &q, f2 *g, f2 &drho, f2 &ux, f2 &uy, f2 &uz) {
+    f2 u[3];
+    collide3_narrow(q, g, drho, u);
+    ux = u[0];
+    uy = u[1];
+    uz = u[2];
 }
 
 }  // namespace d3

@@ -59,7 +59,7 @@ struct Step3 {
     using C = typename Codec<S>::C;
     Geo3 g;
     uint32_t N;
-    Consts3<C> k;
+    Consts3<C, Codec<S>::narrow> k;
     const uint32_t *links;
     const S *src;
     S *dst;
@@ -87,7 +87,8 @@ struct Step3 {
     // Zou-He: U_x/3, (U_x + U_y)/6, (U_x - U_y)/6, (U_x + U_z)/6, (U_x - U_z)/6,
     // -U_y/3, -U_z/3, rho_out - 1
     C zh[8];
-    Consts3x2 k2;   // FP32 arithmetic: k duplicated for the packed node pairs
+    // 16-bit storage: k.r duplicated for the packed node pairs
+    std::conditional_t<Codec<S>::narrow, NarrowRelax3<f2>, NoPairs> k2;
 };
 
 // Storage slot of population i in the stored state.
@@ -431,7 +432,7 @@ __device__ __forceinline__ void step3_pair(const Step3<S> &a, uint32_t x, uint32
         for (int i = 0; i < Q; ++i) g[i] = pk2(ga[i], gb[i]);
     }
     f2 drho, ux, uy, uz;
-    collide3_2(a.k2, a.k.force, g, drho, ux, uy, uz);
+    collide3_2(a.k2, g, drho, ux, uy, uz);
     float da, db;
     up2(drho, da, db);
     if ((fa && !isfinite(da)) || (fb && !isfinite(db))) atomicOr(a.err, 1u);

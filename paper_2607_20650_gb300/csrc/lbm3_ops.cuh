@@ -45,24 +45,7 @@ Step3<S> make3(const lbm3_lattice *L, int src, int toff, int mom) {
         }
     }
     a.N = (uint32_t)L->pl.N;
-    const double om = 1.0 / p.tau, kf = 1.0 - 0.5 * om;
-    a.k.omega = (C)om;
-    for (int d = 0; d < 3; ++d) {
-        a.k.hf[d] = (C)(0.5 * p.force[d]);
-        a.k.f[d] = (C)p.force[d];
-    }
-    a.k.w0 = (C)(1.0 / 3.0);
-    a.k.w1 = (C)(1.0 / 18.0);
-    a.k.w2 = (C)(1.0 / 36.0);
-    a.k.wl0 = (C)(1.0 / 3.0 - (double)a.k.w0);
-    a.k.wl1 = (C)(1.0 / 18.0 - (double)a.k.w1);
-    a.k.wl2 = (C)(1.0 / 36.0 - (double)a.k.w2);
-    a.k.kw0 = (C)(kf / 3.0);
-    a.k.kw1 = (C)(kf / 18.0);
-    a.k.kw2 = (C)(kf / 36.0);
-    a.k.force = (p.force[0] != 0.0 || p.force[1] != 0.0 || p.force[2] != 0.0) ? 1 : 0;
-    for (int i = 0; i < Q; ++i)
-        a.k.cF[i] = (C)(d3::cx(i) * p.force[0] + d3::cy(i) * p.force[1] + d3::cz(i) * p.force[2]);
+    make_relax3(1.0 / p.tau, p.force, a.k.r);
     {
         const int64_t N = L->pl.N, nx = p.nx, nxy = (int64_t)p.nx * p.ny;
         for (int i = 0; i < Q; ++i) {
@@ -97,7 +80,7 @@ Step3<S> make3(const lbm3_lattice *L, int src, int toff, int mom) {
     a.nxy_magic = magic3((uint64_t)p.nx * (uint64_t)p.ny);
     // measured: +7 % for the stream layout on a porous box, -3 % for the bundle layout
     a.zero_fill = (p.layout != LBM_LAYOUT_BUNDLE && (p.algo == LBM_LPTL || L->pl.tx % 32 == 0)) ? 1 : 0;
-    if constexpr (std::is_same<C, float>::value) a.k2 = make_consts3x2(a.k);
+    if constexpr (Codec<S>::narrow) a.k2 = duplicate(a.k.r);
     return a;
 }
 

@@ -282,7 +282,6 @@ void lbm_fill_args(const lbm_params *p, const Plan &pl, char *ws, const Ops *ops
     h->storage = p->storage;
     h->rounding = p->rounding;
     h->omega = 1.0 / p->tau;
-    h->kf = 1.0 - 0.5 * h->omega;
     h->fx = p->force[0];
     h->fy = p->force[1];
     h->ux_in = p->u_in[0];

@@ -22,7 +22,7 @@ struct Step {
     using C = typename Codec<S>::C;
     Geo geo;
     uint32_t N;
-    Consts<C> k;
+    Consts<C, Codec<S>::narrow> k;
     const uint8_t *links;
     const S *src;
     S *dst;
@@ -39,7 +39,8 @@ struct Step {
     int off32;  // 9N < 2^32: element offsets fit 32 bits
     int aos16;  // nx % 16 == 0: warp segments of 32 records start on 16-byte boundaries
     uint32_t pf;  // L2 prefetch distance of the two-lattice kernel: nodes (LPTL), rows (NPTL); 0 = off
-    Consts2 k2;   // FP32 arithmetic: k with every constant duplicated for the packed node pairs
+    // 16-bit storage: k.r with every constant duplicated for the packed node pairs
+    std::conditional_t<Codec<S>::narrow, NarrowRelax<f2>, NoPairs> k2;
 };
 
 // Host: FP64 constants rounded once to the compute type.
@@ -49,23 +50,11 @@ Step<S> make_step(const HostArgs &h, const StepCall &c) {
     Step<S> a;
     a.geo = Geo{h.nx, h.ny, h.bw, h.be, h.bs, h.bn};
     a.N = (uint32_t)h.N;
-    Consts<C> &k = a.k;
-    k.omega = (C)h.omega;
-    k.hfx = (C)(0.5 * h.fx);
-    k.hfy = (C)(0.5 * h.fy);
-    k.fx = (C)h.fx;
-    k.fy = (C)h.fy;
-    k.sF = (C)(h.fx + h.fy);
-    k.dF = (C)(h.fx - h.fy);
+    Consts<C, Codec<S>::narrow> &k = a.k;
+    make_relax(h.omega, h.fx, h.fy, k.r);
     k.w0 = (C)(1.0 / 36.0);
     k.w1 = (C)(1.0 / 9.0);
     k.w4 = (C)(4.0 / 9.0);
-    k.wl0 = (C)(1.0 / 36.0 - (double)k.w0);
-    k.wl1 = (C)(1.0 / 9.0 - (double)k.w1);
-    k.wl4 = (C)(4.0 / 9.0 - (double)k.w4);
-    k.kw0 = (C)(h.kf / 36.0);
-    k.kw1 = (C)(h.kf / 9.0);
-    k.kw4 = (C)(4.0 * h.kf / 9.0);
     k.zh5 = (C)(2.0 / 3.0 * h.ux_in);
     k.zh8 = (C)(h.ux_in / 6.0 + h.uy_in / 2.0);
     k.zh2 = (C)(h.ux_in / 6.0 - h.uy_in / 2.0);
@@ -97,8 +86,7 @@ Step<S> make_step(const HostArgs &h, const StepCall &c) {
     a.off32 = (9 * h.N) < (int64_t(1) << 32) ? 1 : 0;
     a.aos16 = (h.nx % 16 == 0) ? 1 : 0;
     a.pf = h.pf;
-    if constexpr (sizeof(C) == 4) a.k2 = make_consts2(a.k);
-    else memset(&a.k2, 0, sizeof(a.k2));
+    if constexpr (Codec<S>::narrow) a.k2 = duplicate(a.k.r);
     return a;
 }
 
@@ -195,7 +183,7 @@ __device__ __forceinline__ void collide_encode(const Step<S> &a, uint32_t x, uin
     using A = Ar<C>;
     if (EDGE) edge_substitute(a, x, g, drho_nb);
     C drho, ux, uy;
-    collide<Codec<S>::narrow>(a.k, g, drho, ux, uy);
+    collide(a.k, g, drho, ux, uy);
     if (!isfinite(drho)) atomicOr(a.err, 1u);
     if (a.mom) {
         a.mom[n] = A::add(C(1), drho);
@@ -1473,8 +1461,8 @@ __global__ void k_state_moments(const Step<S> a, int rev, int post) {
         if (cy(i) != 0) jy = cy(i) > 0 ? A::add(jy, h[i]) : A::sub(jy, h[i]);
     }
     if (post) {
-        jx = A::sub(jx, a.k.hfx);
-        jy = A::sub(jy, a.k.hfy);
+        jx = A::sub(jx, a.k.r.hfx);
+        jy = A::sub(jy, a.k.r.hfy);
     }
     m[n] = A::add(C(1), r);
     m[a.N + n] = jx;
