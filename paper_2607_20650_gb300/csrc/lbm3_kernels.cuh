@@ -562,23 +562,22 @@ __global__ void __launch_bounds__(512, PHASE == 0 ? (sizeof(S) == 8 ? 1 : 2) : (
 }
 
 // ------------------------------------------------------------ NPOL (3-D)
-// Buffer grid: per tile and parity, for each of the six tile faces the five
-// populations that leave each face node through it (c_a = +1 for the high
-// face of axis a, -1 for the low face). Face order x+, x-, y+, y-, z+, z-;
-// a face of axis x holds ty tz slots per direction (position ly + ty lz),
-// of axis y tx tz (lx + tx lz), of axis z tx ty (lx + tx ly).
+// Buffer grid: for each axis, per sign of c and rank among the five
+// directions that cross its tile boundaries, one plane of nodes per tile
+// position along the axis, holding the populations that left the tiles
+// through that face in the previous update (one set per parity). Planes are
+// indexed by the global coordinates of the two other axes (X: z ny + y, Y:
+// z nx + x, Z: y nx + x), so a node finds a crossing value by the same shift
+// from its own position as in the lattice, with no division into source tile
+// and local position. A pull that crosses several tile boundaries reads the
+// plane of the first axis crossed. Boundaries of the box are tile boundaries
+// too: a periodic wrap is read from the planes like any other crossing.
+// Elements: 10 (ntx ny nz + nty nx nz + ntz nx ny), at most the
+// 10 (ty tz + tx tz + tx ty) per tile that are allocated.
 struct Tile3 {
     int tx, ty, tz;
     __host__ __device__ int nodes(int axis) const { return axis == 0 ? ty * tz : (axis == 1 ? tx * tz : tx * ty); }
     __host__ __device__ int64_t per_tile() const { return 10ll * (nodes(0) + nodes(1) + nodes(2)); }
-    __host__ __device__ int64_t face_off(int axis, int sign) const {
-        int64_t o = 0;
-        for (int a = 0; a < axis; ++a) o += 10ll * nodes(a);
-        return o + (sign > 0 ? 0 : 5ll * nodes(axis));
-    }
-    __host__ __device__ int pos(int axis, int lx, int ly, int lz) const {
-        return axis == 0 ? ly + ty * lz : (axis == 1 ? lx + tx * lz : lx + tx * ly);
-    }
 };
 
 // Rank of direction i among the five directions with the same nonzero c_a.
@@ -592,82 +591,98 @@ __host__ __device__ constexpr int face_rank(int i, int axis) {
     return r;
 }
 
-// Publish the outgoing populations e (canonical order) of the node at local
-// (lx, ly, lz) of tile t, whose bounds are lo[] .. hi[] (global).
-template <class S>
-__device__ __forceinline__ void publish3(S *hw, const Tile3 &T, int64_t t, const int *p, const int *lo,
-                                         const int *hi, int lx, int ly, int lz, const S *e) {
-    S *base = hw + t * T.per_tile();
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int pos = T.pos(a, lx, ly, lz);
-        const int fn = T.nodes(a);
-        if (p[a] == hi[a]) {
-            S *f = base + T.face_off(a, 1);
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-                if ((a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i))) > 0) f[face_rank(i, a) * fn + pos] = e[i];
-        }
-        if (p[a] == lo[a]) {
-            S *f = base + T.face_off(a, -1);
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-                if ((a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i))) < 0) f[face_rank(i, a) * fn + pos] = e[i];
-        }
-    }
-}
+// A node's place in the buffer grid. OFF32: elements of the grid fit 32 bits
+// (they are at most 30 N, and the lattice's 19 N fit 31).
+template <bool OFF32>
+struct Halo3 {
+    using I = std::conditional_t<OFF32, uint32_t, uint64_t>;
+    I X, Y, Z;             // planes of the node's own tile position, sign +, rank 0
+    I px, py, pz;          // elements per (sign, rank)
+    I xb, xf, yb, yf, zb, zf;   // to the plane of the tile before / after, which c > 0 / c < 0 pulls read
+    bool lo[3], hi[3];     // the node lies on its tile's low / high face
+    int yl, yh, zl, zh;    // shift of y (z) by a pull with c > 0 / c < 0, periodic
+    int nx, ny;
 
-// Pulls of a fluid node off the box faces with the 32-bit offset tables:
-// every lane runs the interior pull (neighbour value, or the node's own
-// opposite value for a bounced link) and, for a direction whose source lies
-// in another tile, reads the source tile's publication of the previous
-// update instead (the face of the first axis along which the tiles differ).
-// Face nodes therefore run the same code as inner nodes plus a short
-// address computation per crossing direction.
-template <class S, int L>
-__device__ __forceinline__ void npol3_pull(const Step3<S> &a, const S *hr, const Tile3 &T, const int *b,
-                                           const int *nt, const int *tdim, const int *l, const int *p,
-                                           const int *lo, const int *hi, uint32_t n, uint32_t lk,
-                                           typename Codec<S>::C *g) {
+    __device__ __forceinline__ Halo3(const Geo3 &g, const int *nt, const int *b, const int *p, const int *tlo,
+                                     const int *thi) {
+        nx = g.nx;
+        ny = g.ny;
+        const I sx = (I)g.ny * (I)g.nz, sy = (I)g.nx * (I)g.nz, sz = (I)g.nx * (I)g.ny;
+        px = (I)nt[0] * sx;
+        py = (I)nt[1] * sy;
+        pz = (I)nt[2] * sz;
+        X = (I)b[0] * sx + (I)p[2] * (I)ny + (I)p[1];
+        Y = (I)10 * px + (I)b[1] * sy + (I)p[2] * (I)nx + (I)p[0];
+        Z = (I)10 * px + (I)10 * py + (I)b[2] * sz + (I)p[1] * (I)nx + (I)p[0];
+        xb = b[0] == 0 ? px - sx : (I)0 - sx;
+        xf = b[0] == nt[0] - 1 ? sx - px : sx;
+        yb = b[1] == 0 ? py - sy : (I)0 - sy;
+        yf = b[1] == nt[1] - 1 ? sy - py : sy;
+        zb = b[2] == 0 ? pz - sz : (I)0 - sz;
+        zf = b[2] == nt[2] - 1 ? sz - pz : sz;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const S *base = a.src + mult3<L>(i) * n;
-        if (i == REST) {
-            g[i] = Codec<S>::dec(base[a.os[i]]);
-            continue;
+        for (int k = 0; k < 3; ++k) {
+            lo[k] = p[k] == tlo[k];
+            hi[k] = p[k] == thi[k];
         }
-        const bool bounce = (lk >> bit(i)) & 1u;
-        const S *q = base + (bounce ? a.ob[i] : a.op[i]);
-        const int c[3] = {cx(i), cy(i), cz(i)};
-        bool cr[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) cr[k] = (c[k] > 0 && p[k] == lo[k]) || (c[k] < 0 && p[k] == hi[k]);
-        if (!bounce && (cr[0] || cr[1] || cr[2])) {
-            int bs[3], ls[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                bs[k] = cr[k] ? b[k] - c[k] : b[k];
-                ls[k] = cr[k] ? (c[k] > 0 ? tdim[k] - 1 : 0) : l[k] - c[k];
-            }
-            const int ax = cr[0] ? 0 : (cr[1] ? 1 : 2);
-            const int64_t ts = ((int64_t)bs[2] * nt[1] + bs[1]) * nt[0] + bs[0];
-            q = hr + ts * T.per_tile() + T.face_off(ax, c[ax]) + (int64_t)face_rank(i, ax) * T.nodes(ax) +
-                T.pos(ax, ls[0], ls[1], ls[2]);
-        }
-        g[i] = Codec<S>::dec(*q);
+        yl = p[1] == 0 ? g.ny - 1 : -1;
+        yh = p[1] == g.ny - 1 ? 1 - g.ny : 1;
+        zl = p[2] == 0 ? g.nz - 1 : -1;
+        zh = p[2] == g.nz - 1 ? 1 - g.nz : 1;
     }
-}
+    // Does the pull of direction i leave the tile along axis a?
+    __device__ __forceinline__ bool crosses(int i, int a) const {
+        const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
+        return c > 0 ? lo[a] : (c < 0 ? hi[a] : false);
+    }
+    // Element that the pull of direction i, which leaves the tile, reads.
+    __device__ __forceinline__ I at(int i) const {
+        const int dy = cy(i) > 0 ? yl : (cy(i) < 0 ? yh : 0), dz = cz(i) > 0 ? zl : (cz(i) < 0 ? zh : 0);
+        I r = 0;
+        if (cz(i)) r = Z + (cz(i) > 0 ? zb : zf) + (I)((cz(i) < 0 ? 5 : 0) + face_rank(i, 2)) * pz - (I)(cx(i) + cy(i) * nx);
+        if (cy(i)) {
+            const I v = Y + (cy(i) > 0 ? yb : yf) + (I)((cy(i) < 0 ? 5 : 0) + face_rank(i, 1)) * py + (I)(dz * nx - cx(i));
+            r = !cz(i) || crosses(i, 1) ? v : r;
+        }
+        if (cx(i)) {
+            const I v = X + (cx(i) > 0 ? xb : xf) + (I)((cx(i) < 0 ? 5 : 0) + face_rank(i, 0)) * px + (I)(dy + dz * ny);
+            r = !(cy(i) || cz(i)) || crosses(i, 0) ? v : r;
+        }
+        return r;
+    }
+    // Publish the outgoing populations e (canonical order) of the node.
+    template <class S>
+    __device__ __forceinline__ void publish(S *hw, const S *e) const {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const I base = a == 0 ? X : (a == 1 ? Y : Z), plane = a == 0 ? px : (a == 1 ? py : pz);
+#pragma unroll
+            for (int sign = 0; sign < 2; ++sign) {
+                if (!(sign ? lo[a] : hi[a])) continue;
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
+                    if (c == (sign ? -1 : 1)) hw[base + (I)(5 * sign + face_rank(i, a)) * plane] = e[i];
+                }
+            }
+        }
+    }
+};
 
 // One lattice, pull: every node of the tile reads its 19 incoming values
 // (sources in the tile from the lattice, from other tiles out of the buffer
 // grid the previous update wrote), a block barrier separates all reads from
 // the in-place writes, and face nodes publish their outgoing values.
-// Tile b (of nt per axis) of the update.
+// Tile b (of nt per axis) of the update. Every lane runs the same code: with
+// 8 x 8 x 8 tiles 58 % of the nodes lie on a face and every warp holds some,
+// so a separate path for them would run in every warp (as it did: 1,806 warp
+// instructions per 32 nodes, 383 us an update of 200 x 160 x 132 sphere-packing
+// nodes, FP32 stream layout; now 172 us). Bound by instruction issue and the
+// barrier, with two 512-thread blocks per SM.
 template <class S, int L, bool OFF32>
 __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw, const int *b, const int *nt) {
     using C = typename Codec<S>::C;
     using A = Ar<C>;
-    const Tile3 T{a.tx, a.ty, a.tz};
     const int ext[3] = {a.g.nx, a.g.ny, a.g.nz};
     const int tdim[3] = {a.tx, a.ty, a.tz};
     const int l[3] = {(int)threadIdx.x, (int)threadIdx.y, (int)threadIdx.z};
@@ -688,81 +703,26 @@ __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw
         lk = a.links[n];
     }
     const bool fluid = lk != SOLID;
-    const bool inner = p[0] > lo[0] && p[0] < hi[0] && p[1] > lo[1] && p[1] < hi[1] && p[2] > lo[2] && p[2] < hi[2];
-    const int64_t t = ((int64_t)b[2] * nt[1] + b[1]) * nt[0] + b[0];
+    const Halo3<OFF32> H(a.g, nt, b, p, lo, hi);
     C g[Q];
-    const bool box_inner = p[0] > 0 && p[0] < ext[0] - 1 && p[1] > 0 && p[1] < ext[1] - 1 && p[2] > 0 &&
-                           p[2] < ext[2] - 1;
-    if (fluid && inner) {
-        pull3<S, L, OFF32>(a, (uint32_t)p[0], (uint32_t)p[1], (uint32_t)p[2], n, lk, g);
-    } else if (OFF32 && fluid && box_inner) {
-        npol3_pull<S, L>(a, hr, T, b, nt, tdim, l, p, lo, hi, n, lk, g);
-    } else if (fluid) {
-        // Per axis: does a pull with c = +1 (-1) leave the tile (the node is on
-        // the tile's low (high) face)? Where the tile spans the whole axis, such
-        // a pull wraps around the box inside the tile (periodic) or bounces.
-        bool lof[3], hif[3];
-        int wrap_lo[3], wrap_hi[3];   // node-index correction of an in-tile wrap
-        int tprev[3], tnext[3], lprev[3];
-        const int stride[3] = {1, (int)nx, (int)(nx * ny)};
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lof[k] = p[k] == lo[k];
-            hif[k] = p[k] == hi[k];
-            wrap_lo[k] = p[k] == 0 ? ext[k] * stride[k] : 0;
-            wrap_hi[k] = p[k] == ext[k] - 1 ? -ext[k] * stride[k] : 0;
-            tprev[k] = b[k] == 0 ? nt[k] - 1 : b[k] - 1;
-            tnext[k] = b[k] == nt[k] - 1 ? 0 : b[k] + 1;
-            lprev[k] = min(tdim[k], ext[k] - tprev[k] * tdim[k]) - 1;
-        }
+    if (fluid) {
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
             if (i == REST) {
-                g[i] = Codec<S>::dec(lat[addr<L>(a.N, n, i)]);
+                g[i] = Codec<S>::dec(OFF32 ? lat[mult3<L>(i) * n + (uint32_t)a.os[i]] : lat[addr<L>(a.N, n, i)]);
                 continue;
             }
-            if ((lk >> bit(i)) & 1u) {
-                g[i] = Codec<S>::dec(lat[addr<L>(a.N, n, opp(i))]);
-                continue;
-            }
-            const int c[3] = {cx(i), cy(i), cz(i)};
-            bool out = false;   // the source lies in another tile
-            int shift = 0;      // node-index shift of the source (in-tile, wraps included)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                if (c[k] == 0) continue;
-                const bool cross = c[k] > 0 ? lof[k] : hif[k];
-                shift += -c[k] * stride[k];
-                if (cross) {
-                    if (nt[k] == 1) shift += c[k] > 0 ? wrap_lo[k] : wrap_hi[k];
-                    else out = true;
-                }
-            }
-            if (!out) {
-                g[i] = Codec<S>::dec(lat[addr<L>(a.N, (uint32_t)((int64_t)n + shift), i)]);
+            const bool bounce = (lk >> bit(i)) & 1u;
+            const S *q;
+            if (OFF32) {
+                // (out of range only for a pull that wraps, which reads the grid)
+                q = lat + (mult3<L>(i) * n + (uint32_t)(bounce ? a.ob[i] : a.op[i]));
             } else {
-                // the value left the source tile through its face of the first
-                // axis along which the tiles differ
-                int bs[3], ls[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const bool cr = c[k] != 0 && (c[k] > 0 ? lof[k] : hif[k]) && nt[k] > 1;
-                    if (!cr) {
-                        bs[k] = b[k];
-                        int sk = p[k] - c[k];
-                        sk = sk < 0 ? sk + ext[k] : (sk >= ext[k] ? sk - ext[k] : sk);
-                        ls[k] = sk - lo[k];
-                    } else {
-                        bs[k] = c[k] > 0 ? tprev[k] : tnext[k];
-                        ls[k] = c[k] > 0 ? lprev[k] : 0;
-                    }
-                }
-                const int ax = bs[0] != b[0] ? 0 : (bs[1] != b[1] ? 1 : 2);
-                const int64_t ts = ((int64_t)bs[2] * nt[1] + bs[1]) * nt[0] + bs[0];
-                const int64_t slot = ts * T.per_tile() + T.face_off(ax, c[ax]) +
-                                     (int64_t)face_rank(i, ax) * T.nodes(ax) + T.pos(ax, ls[0], ls[1], ls[2]);
-                g[i] = Codec<S>::dec(hr[slot]);
+                const int64_t d = ((int64_t)cz(i) * ny + cy(i)) * (int64_t)nx + cx(i);
+                q = lat + (bounce ? addr<L>(a.N, n, opp(i)) : addr<L>(a.N, (int64_t)n - d, i));
             }
+            if (!bounce && (H.crosses(i, 0) || H.crosses(i, 1) || H.crosses(i, 2))) q = hr + H.at(i);
+            g[i] = Codec<S>::dec(*q);
         }
     }
     __syncthreads();
@@ -783,9 +743,10 @@ __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         e[i] = Codec<S>::enc(g[i], sr, sr ? pop_rand(nk, i) : 0u);
-        lat[addr<L>(a.N, n, i)] = e[i];
+        if (OFF32) lat[mult3<L>(i) * n + (uint32_t)a.os[i]] = e[i];
+        else lat[addr<L>(a.N, n, i)] = e[i];
     }
-    if (!inner) publish3(hw, T, t, p, lo, hi, l[0], l[1], l[2], e);
+    H.publish(hw, e);
 }
 
 template <class S, int L, bool OFF32>
@@ -803,9 +764,8 @@ __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 2) k3_npol(const Ste
 // x + c_i is in the tile and no bounce separates them. After the exchanges
 // slot j of x holds the value x pulls in direction j (a bounced link keeps
 // the node's own value, i.e. bounce-back). Pulls from other tiles come from
-// the buffer grid, in the same format as NPOL's; pulls that wrap around a
-// periodic face inside one tile are read from the staged slots before the
-// exchange. Results are stored back into the opposite slots and face nodes
+// the buffer grid, in the same format as NPOL's (a wrap around a periodic face
+// inside one tile included). Results are stored back into the opposite slots and face nodes
 // publish their outgoing values. Shared memory: 19 planes of the tile's
 // nodes (compute type).
 template <class S>
@@ -819,7 +779,6 @@ __device__ __forceinline__ void nsol3_tile(const Step3<S> &a, const S *hr, S *hw
                                            typename Codec<S>::C *sm) {
     using C = typename Codec<S>::C;
     using A = Ar<C>;
-    const Tile3 T{a.tx, a.ty, a.tz};
     const int TN = a.tx * a.ty * a.tz;
     const int ext[3] = {a.g.nx, a.g.ny, a.g.nz};
     const int tdim[3] = {a.tx, a.ty, a.tz};
@@ -842,74 +801,22 @@ __device__ __forceinline__ void nsol3_tile(const Step3<S> &a, const S *hr, S *hw
         lk = a.links[n];
     }
     const bool fluid = lk != SOLID;
-    const bool inner = p[0] > lo[0] && p[0] < hi[0] && p[1] > lo[1] && p[1] < hi[1] && p[2] > lo[2] && p[2] < hi[2];
-    const int64_t t = ((int64_t)b[2] * nt[1] + b[1]) * nt[0] + b[0];
     if (fluid) {
 #pragma unroll
         for (int s = 0; s < Q; ++s) sm[s * TN + tid] = Codec<S>::dec(lat[addr<L>(a.N, n, s)]);
     }
-    __syncthreads();
-    // Pulls the in-tile exchange does not cover: sources in another tile
-    // (buffer grid) or reached through a periodic face inside this tile.
+    // Pulls the in-tile exchange does not cover: those that leave the tile.
+    const Halo3<false> H(a.g, nt, b, p, lo, hi);
     C fix[Q];
     uint32_t fixmask = 0;
-    if (fluid && !inner) {
-        bool lof[3], hif[3];
-        int tprev[3], tnext[3], lprev[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            lof[k] = p[k] == lo[k];
-            hif[k] = p[k] == hi[k];
-            tprev[k] = b[k] == 0 ? nt[k] - 1 : b[k] - 1;
-            tnext[k] = b[k] == nt[k] - 1 ? 0 : b[k] + 1;
-            lprev[k] = min(tdim[k], ext[k] - tprev[k] * tdim[k]) - 1;
-        }
+    if (fluid) {
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
             fix[j] = C(0);
             if (j == REST || ((lk >> bit(j)) & 1u)) continue;
-            const int c[3] = {cx(j), cy(j), cz(j)};
-            bool cross = false, out = false;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                if (c[k] == 0) continue;
-                if (c[k] > 0 ? lof[k] : hif[k]) {
-                    cross = true;
-                    if (nt[k] > 1) out = true;
-                }
-            }
-            if (!cross) continue;   // adjacent in the tile: the exchange delivers it
-            fixmask |= 1u << j;
-            if (!out) {
-                // wraps around a periodic face of an axis the tile spans whole
-                int q[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    int sk = p[k] - c[k];
-                    sk = sk < 0 ? sk + ext[k] : (sk >= ext[k] ? sk - ext[k] : sk);
-                    q[k] = sk - lo[k];
-                }
-                fix[j] = sm[opp(j) * TN + (q[2] * a.ty + q[1]) * a.tx + q[0]];
-            } else {
-                int bs[3], ls[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const bool cr = c[k] != 0 && (c[k] > 0 ? lof[k] : hif[k]) && nt[k] > 1;
-                    if (!cr) {
-                        bs[k] = b[k];
-                        int sk = p[k] - c[k];
-                        sk = sk < 0 ? sk + ext[k] : (sk >= ext[k] ? sk - ext[k] : sk);
-                        ls[k] = sk - lo[k];
-                    } else {
-                        bs[k] = c[k] > 0 ? tprev[k] : tnext[k];
-                        ls[k] = c[k] > 0 ? lprev[k] : 0;
-                    }
-                }
-                const int ax = bs[0] != b[0] ? 0 : (bs[1] != b[1] ? 1 : 2);
-                const int64_t ts = ((int64_t)bs[2] * nt[1] + bs[1]) * nt[0] + bs[0];
-                const int64_t slot = ts * T.per_tile() + T.face_off(ax, c[ax]) +
-                                     (int64_t)face_rank(j, ax) * T.nodes(ax) + T.pos(ax, ls[0], ls[1], ls[2]);
-                fix[j] = Codec<S>::dec(hr[slot]);
+            if (H.crosses(j, 0) || H.crosses(j, 1) || H.crosses(j, 2)) {
+                fixmask |= 1u << j;
+                fix[j] = Codec<S>::dec(hr[H.at(j)]);
             }
         }
     }
@@ -952,7 +859,7 @@ __device__ __forceinline__ void nsol3_tile(const Step3<S> &a, const S *hr, S *hw
         e[i] = Codec<S>::enc(g[i], sr, sr ? pop_rand(nk, i) : 0u);
         lat[addr<L>(a.N, n, opp(i))] = e[i];
     }
-    if (!inner) publish3(hw, T, t, p, lo, hi, l[0], l[1], l[2], e);
+    H.publish(hw, e);
 }
 
 template <class S, int L>
@@ -966,9 +873,9 @@ __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 2) k3_nsol(const Ste
 // Fill a buffer-grid parity from the stored state (after init or a write).
 template <class S, int L>
 __global__ void k3_publish(const Step3<S> a, S *hw) {
-    const Tile3 T{a.tx, a.ty, a.tz};
     const int ext[3] = {a.g.nx, a.g.ny, a.g.nz};
     const int b[3] = {(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
+    const int nt[3] = {(int)gridDim.x, (int)gridDim.y, (int)gridDim.z};
     const int tdim[3] = {a.tx, a.ty, a.tz};
     const int l[3] = {(int)threadIdx.x, (int)threadIdx.y, (int)threadIdx.z};
     int lo[3], hi[3], p[3];
@@ -981,12 +888,10 @@ __global__ void k3_publish(const Step3<S> a, S *hw) {
     }
     const uint32_t n = (((uint32_t)p[2] * (uint32_t)ext[1]) + (uint32_t)p[1]) * (uint32_t)ext[0] + (uint32_t)p[0];
     if (a.links[n] == SOLID) return;
-    const int64_t ntx = (ext[0] + a.tx - 1) / a.tx, nty = (ext[1] + a.ty - 1) / a.ty;
-    const int64_t t = ((int64_t)b[2] * nty + b[1]) * ntx + b[0];
     S e[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) e[i] = a.dst[addr<L>(a.N, n, slot3(a, i))];
-    publish3(hw, T, t, p, lo, hi, l[0], l[1], l[2], e);
+    Halo3<false>(a.g, nt, b, p, lo, hi).publish(hw, e);
 }
 
 template <class S, int L>
