@@ -34,7 +34,7 @@ struct Step {
     int toff;
     int sr;
     uint64_t seed;
-    int tx, ty, ntx;
+    int tx, ty, ntx, nty;
     uint64_t nx_magic;
     int off32;  // 9N < 2^32: element offsets fit 32 bits
     int aos16;  // nx % 16 == 0: warp segments of 32 records start on 16-byte boundaries
@@ -82,6 +82,7 @@ Step<S> make_step(const HostArgs &h, const StepCall &c) {
     a.tx = h.tile_x;
     a.ty = h.tile_y;
     a.ntx = h.ntx;
+    a.nty = h.nty;
     a.nx_magic = h.nx_magic;
     a.off32 = (9 * h.N) < (int64_t(1) << 32) ? 1 : 0;
     a.aos16 = (h.nx % 16 == 0) ? 1 : 0;
@@ -732,48 +733,94 @@ __global__ void __launch_bounds__(kMaxTileThreads / 2, LBM_PAIR_MINB) k_two_latt
 }
 
 // ------------------------------------------------------------ buffer grid
-// Per tile and parity: east edge 3 x ty values (directions 2,5,8), west
-// 3 x ty (0,3,6), north 3 x tx (6,7,8), south 3 x tx (0,1,2).
-enum Edge { EDGE_E = 0, EDGE_W = 1, EDGE_N = 2, EDGE_S = 3 };
-
-__device__ __forceinline__ int64_t halo_slot(int tx, int ty, int ntx, int bx, int by, int edge,
-                                             int k, int pos) {
-    int64_t base = (int64_t)(by * ntx + bx) * (6 * (tx + ty));
-    switch (edge) {
-        case EDGE_E: return base + k * ty + pos;
-        case EDGE_W: return base + 3 * ty + k * ty + pos;
-        case EDGE_N: return base + 6 * ty + k * tx + pos;
-        default: return base + 6 * ty + 3 * tx + k * tx + pos;
-    }
+// Per parity, in triples of the three populations that leave a tile through
+// one of its edges: for each tile column the column of nodes on its east edge
+// (2, 5, 8), triple bx ny + y; then those of the west edges (0, 3, 6); then for
+// each tile row the row of nodes on its north edge (6, 7, 8), triple
+// by nx + x, and those of the south edges (0, 1, 2). Global coordinates along
+// the edge: a node finds a crossing value by the same shift from its own
+// position as in the lattice, with no division into source tile and local
+// position, and in the bundle layout a row of triples replaces the lattice's
+// own row. 6 (ntx ny + nty nx) elements, at most the 6 (tx + ty) per tile that
+// are allocated.
+template <class S> __device__ __forceinline__ int64_t halo_cols(const Step<S> &a) { return (int64_t)a.ntx * a.geo.ny; }
+template <class S> __device__ __forceinline__ int64_t halo_rows(const Step<S> &a) { return (int64_t)a.nty * a.geo.nx; }
+// First triple elements of node (., y) of tile column bx and of node (x, .) of tile row by.
+template <class S>
+__device__ __forceinline__ int64_t halo_col(const Step<S> &a, bool west, int bx, int y) {
+    return 3 * ((west ? halo_cols(a) : 0) + (int64_t)bx * a.geo.ny + y);
+}
+template <class S>
+__device__ __forceinline__ int64_t halo_row(const Step<S> &a, bool south, int by, int x) {
+    return 6 * halo_cols(a) + 3 * ((south ? halo_rows(a) : 0) + (int64_t)by * a.geo.nx + x);
 }
 
 // Value S[(xs, ys)][j] of a node in another tile, as that tile published it.
 template <class S>
-__device__ __forceinline__ typename Codec<S>::C halo_read(const Step<S> &a, int xs, int ys, int j,
-                                                          int bx) {
-    const int bxs = xs / a.tx, bys = ys / a.ty;
-    int64_t s;
-    if (bxs != bx)
-        s = halo_slot(a.tx, a.ty, a.ntx, bxs, bys, cx(j) > 0 ? EDGE_E : EDGE_W, j / 3, ys - bys * a.ty);
-    else
-        s = halo_slot(a.tx, a.ty, a.ntx, bxs, bys, cy(j) > 0 ? EDGE_N : EDGE_S, j % 3, xs - bxs * a.tx);
+__device__ __forceinline__ typename Codec<S>::C halo_read(const Step<S> &a, int xs, int ys, int j, int bx) {
+    const int bxs = xs / a.tx;
+    const int64_t s = bxs != bx ? halo_col(a, cx(j) < 0, bxs, ys) + j / 3 : halo_row(a, cy(j) < 0, ys / a.ty, xs) + j % 3;
     return Codec<S>::dec(a.halo_rd[s]);
 }
 
 // Publish the populations of an edge node that leave its tile.
 template <class S>
-__device__ __forceinline__ void halo_publish(S *hw, int tx, int ty, int ntx, int bx, int by, int x,
-                                             int y, int x0, int y0, int x1, int y1, const S *e) {
-    S *t = hw + (int64_t)(by * ntx + bx) * (6 * (tx + ty));
-    const int r = y - y0, c = x - x0;
+__device__ __forceinline__ void halo_publish(const Step<S> &a, S *hw, int bx, int by, int x, int y, int x0, int y0,
+                                             int x1, int y1, const S *e) {
+    if (x == x1 || x == x0) {
+        S *p = hw + halo_col(a, false, bx, y);
+        if (x == x1) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        if (x == x1) t[k * ty + r] = e[3 * k + 2];                  // east:  2, 5, 8
-        if (x == x0) t[3 * ty + k * ty + r] = e[3 * k];             // west:  0, 3, 6
-        if (y == y1) t[6 * ty + k * tx + c] = e[6 + k];             // north: 6, 7, 8
-        if (y == y0) t[6 * ty + 3 * tx + k * tx + c] = e[k];        // south: 0, 1, 2
+            for (int k = 0; k < 3; ++k) p[k] = e[3 * k + 2];
+        }
+        if (x == x0) {
+            p += 3 * halo_cols(a);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) p[k] = e[3 * k];
+        }
+    }
+    if (y == y1 || y == y0) {
+        S *p = hw + halo_row(a, false, by, x);
+        if (y == y1) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) p[k] = e[6 + k];
+        }
+        if (y == y0) {
+            p += 3 * halo_rows(a);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) p[k] = e[k];
+        }
     }
 }
+
+// What the pulls of a node (x, y) of tile (bx, by) off the domain edge read
+// where they leave the tile: triples of the adjacent tile columns and rows, at
+// the node's own y and x.
+template <class S>
+struct HaloPull {
+    const S *w, *e, *s, *n;   // east edges of the column before, west edges of the one after; rows alike
+    bool x0, x1, y0, y1;      // the node lies on its tile's west, east, south, north edge
+    __device__ __forceinline__ HaloPull(const Step<S> &a, int bx, int by, int x, int y, int tx0, int tx1, int ty0,
+                                        int ty1) {
+        w = a.halo_rd + halo_col(a, false, bx - 1, y);
+        e = a.halo_rd + halo_col(a, true, bx + 1, y);
+        s = a.halo_rd + halo_row(a, false, by - 1, x);
+        n = a.halo_rd + halo_row(a, true, by + 1, x);
+        x0 = x == tx0;
+        x1 = x == tx1;
+        y0 = y == ty0;
+        y1 = y == ty1;
+    }
+    // Does the pull of direction i cross the south or north edge (crosses_y),
+    // or only the west or east one (crosses_x)? Through a corner it reads the
+    // diagonal tile's row.
+    __device__ __forceinline__ bool crosses_y(int i) const { return cy(i) > 0 ? y0 : (cy(i) < 0 ? y1 : false); }
+    __device__ __forceinline__ bool crosses_x(int i) const {
+        return (cx(i) > 0 ? x0 : (cx(i) < 0 ? x1 : false)) && !crosses_y(i);
+    }
+    __device__ __forceinline__ const S *at_x(int i) const { return (cx(i) > 0 ? w : e) + (i / 3 - 3 * cy(i)); }
+    __device__ __forceinline__ const S *at_y(int i) const { return (cy(i) > 0 ? s : n) + (i % 3 - 3 * cx(i)); }
+};
 
 // ------------------------------------------------------------ NPOL
 // One lattice, pull: every node reads its nine incoming values (in-tile
@@ -781,23 +828,25 @@ __device__ __forceinline__ void halo_publish(S *hw, int tx, int ty, int ntx, int
 // previous update), the block barrier separates all reads from the in-place
 // writes, and edge nodes publish their outgoing values for the next update.
 
-// Pulls of a node off the domain edge (32-bit offsets): every lane runs the
-// interior pull (neighbour value, or the own opposite value of a bounced
-// link) and, where the source lies across a tile edge, reads instead the
-// source tile's publication of the previous update: its east/west edge when
-// the tiles differ in x (the diagonal tile at a corner), else its north/south
-// edge. Tile-edge nodes thus take no separate per-direction path, so a warp
-// holding them does not run two.
+// Pulls of a node off the domain edge (9N < 2^32): every lane runs the same
+// code, the interior pull (neighbour value, or the own opposite value of a
+// bounced link) reading the source tile's publication of the previous update
+// where the source lies across a tile edge. In the bundle layout a row of the
+// buffer grid has the lattice's own format, so crossing the south or north
+// edge only changes the two row pointers (for whole warps, tile_x being a
+// multiple of 32).
 template <class S, int L>
-__device__ __forceinline__ void npol_pull(const Step<S> &a, int bx, int by, int lx, int ly, int x, int y,
-                                          int x0, int x1, int y0, int y1, uint32_t n, uint32_t lk,
+__device__ __forceinline__ void npol_pull(const Step<S> &a, const HaloPull<S> &H, uint32_t n, uint32_t lk,
                                           typename Codec<S>::C *g) {
     const uint32_t nx = (uint32_t)a.geo.nx;
     const S *own = a.dst + lay_mul<L>() * n;
     const S *rs = own + (ptrdiff_t)lay_mul<L>() * nx;  // row y+1: source of c_y = -1
     const S *rn = own - (ptrdiff_t)lay_mul<L>() * nx;  // row y-1: source of c_y = +1
-    const bool ex0 = x == x0, ex1 = x == x1, ey0 = y == y0, ey1 = y == y1;
-    const int per = 6 * (a.tx + a.ty);
+    if (L == BUNDLE) {
+        rn += (ptrdiff_t)lay_base<L>(a.N, 6);
+        if (H.y1) rs = H.n;
+        if (H.y0) rn = H.s;
+    }
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         if (i == 4) {
@@ -805,21 +854,17 @@ __device__ __forceinline__ void npol_pull(const Step<S> &a, int bx, int by, int 
             continue;
         }
         const bool bounce = (lk >> link_bit(i)) & 1u;
-        const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own);
-        const S *p = bounce ? own + (ptrdiff_t)lay_base<L>(a.N, opp(i))
-                            : row + ((ptrdiff_t)lay_base<L>(a.N, i) - (ptrdiff_t)lay_mul<L>() * cx(i));
-        const bool crx = (cx(i) > 0 && ex0) || (cx(i) < 0 && ex1);
-        const bool cry = (cy(i) > 0 && ey0) || (cy(i) < 0 && ey1);
-        if (!bounce && (crx || cry)) {
-            const int bxs = bx - (crx ? cx(i) : 0), bys = by - (cry ? cy(i) : 0);
-            const S *t = a.halo_rd + (int64_t)(bys * a.ntx + bxs) * per;
-            if (crx) {
-                const int r = cry ? (cy(i) > 0 ? a.ty - 1 : 0) : ly - cy(i);
-                p = t + (cx(i) > 0 ? 0 : 3 * a.ty) + (i / 3) * a.ty + r;
-            } else {
-                p = t + 6 * a.ty + (cy(i) > 0 ? 0 : 3 * a.tx) + (i % 3) * a.tx + (lx - cx(i));
-            }
+        const S *p;
+        if (L == BUNDLE) {
+            const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own + (ptrdiff_t)lay_base<L>(a.N, 3));
+            p = row + (i % 3 - 3 * cx(i));
+        } else {
+            const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own);
+            p = row + ((ptrdiff_t)lay_base<L>(a.N, i) - (ptrdiff_t)lay_mul<L>() * cx(i));
+            if (cy(i) != 0 && H.crosses_y(i)) p = H.at_y(i);
         }
+        if (cx(i) != 0 && H.crosses_x(i)) p = H.at_x(i);
+        if (bounce) p = own + (ptrdiff_t)lay_base<L>(a.N, opp(i));
         g[i] = Codec<S>::dec(*p);
     }
 }
@@ -844,9 +889,10 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
     const bool zero_fill = false;   // measured: NPOL is 5 % faster without the sector zero fill
     const bool inner = x > x0 && x < x1 && y > y0 && y < y1;
     const bool dom_inner = x > 0 && x < nx - 1 && y > 0 && y < ny - 1;
+    const HaloPull<S> H(a, bx, by, x, y, x0, x1, y0, y1);
     C g[9];
     if (fluid && dom_inner && a.off32) {
-        npol_pull<S, L>(a, bx, by, lx, ly, x, y, x0, x1, y0, y1, n, lk, g);
+        npol_pull<S, L>(a, H, n, lk, g);
     } else if (fluid) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
@@ -857,22 +903,11 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
             } else if (inner) {
                 g[i] = ldp<S, L>(lat, a.N, n - (uint32_t)(cy(i) * nx + cx(i)), i);
             } else if (dom_inner) {
-                // Tile edge inside the domain: the source is in this tile or in
-                // the adjacent tile's buffer grid; the crossed edge follows from
-                // c_i and the node's place on the tile edge.
-                const int dbx = (cx(i) > 0 && x == x0) ? -1 : ((cx(i) < 0 && x == x1) ? 1 : 0);
-                const int dby = (cy(i) > 0 && y == y0) ? -1 : ((cy(i) < 0 && y == y1) ? 1 : 0);
-                if (dbx == 0 && dby == 0) {
-                    g[i] = ldp<S, L>(lat, a.N, n - (uint32_t)(cy(i) * nx + cx(i)), i);
-                } else {
-                    const int64_t tb = (int64_t)((by + dby) * a.ntx + (bx + dbx)) * (6 * (a.tx + a.ty));
-                    int off;
-                    if (dbx != 0)  // east (c_x > 0) or west edge buffer, row of the source
-                        off = (cx(i) > 0 ? 0 : 3 * a.ty) + (i / 3) * a.ty + (ly - cy(i) - dby * a.ty);
-                    else           // north (c_y > 0) or south edge buffer, column of the source
-                        off = 6 * a.ty + (cy(i) > 0 ? 0 : 3 * a.tx) + (i % 3) * a.tx + (lx - cx(i));
-                    g[i] = Codec<S>::dec(a.halo_rd[tb + off]);
-                }
+                // Tile edge inside the domain: the source is in this tile or
+                // published in the buffer grid.
+                g[i] = H.crosses_y(i)   ? Codec<S>::dec(*H.at_y(i))
+                       : H.crosses_x(i) ? Codec<S>::dec(*H.at_x(i))
+                                        : ldp<S, L>(lat, a.N, n - (uint32_t)(cy(i) * nx + cx(i)), i);
             } else {
                 int xs, ys, j;
                 if (map_pull(a.geo, x, y, i, xs, ys, j) != PULL_NODE)
@@ -890,14 +925,20 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
         S e[9];
         collide_encode(a, (uint32_t)x, n, g, e, dnb);
         store_node<S, L>(lat, n, a.N, a.off32, e);
-        if (!inner) halo_publish(a.halo_wr, a.tx, a.ty, a.ntx, bx, by, x, y, x0, y0, x1, y1, e);
+        if (!inner) halo_publish(a, a.halo_wr, bx, by, x, y, x0, y0, x1, y1, e);
     } else if (zero_fill) {
         store_zero<S, L>(lat, a.N, n, a.off32);  // whole-sector writes, as in two_lattice_node
     }
 }
 
+// Registers: 32 (four 512-thread blocks, spills) for the stream layout and
+// 16-bit storage, 40 (three) where it measured faster: 6000 x 3001 nodes, 16
+// updates, FP32 bundle 64 x 4 3.89 against 3.90 ms and 128 x 4 4.35 against
+// 4.09, collision 5.41 / 4.88, stream 32 x 8 4.11 / 4.29, FP16 3.85 / 3.95.
 template <class S, int L>
-__global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_npol(const Step<S> a) {
+__global__ void __launch_bounds__(kMaxTileThreads,
+                                  sizeof(S) == 8 ? 1 : (sizeof(S) == 4 && L != STREAM) || L == COLLISION ? 3 : 4)
+    k_npol(const Step<S> a) {
     npol_tile<S, L>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
                     (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
 }
@@ -953,19 +994,14 @@ __device__ __forceinline__ void nsol_tile(const Step<S> &a, int bx, int by, int 
     if (fluid && dom_inner && !(x > x0 && x < x1 && y > y0 && y < y1)) {
         // Tile edge inside the domain: values from other tiles come from their
         // buffer grid (same slots as NPOL); in-tile sources are exchanged.
+        const HaloPull<S> H(a, bx, by, x, y, x0, x1, y0, y1);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             fix[i] = C(0);
             if (i == 4 || ((lk >> link_bit(i)) & 1u)) continue;
-            const int dbx = (cx(i) > 0 && x == x0) ? -1 : ((cx(i) < 0 && x == x1) ? 1 : 0);
-            const int dby = (cy(i) > 0 && y == y0) ? -1 : ((cy(i) < 0 && y == y1) ? 1 : 0);
-            if (dbx == 0 && dby == 0) continue;
-            const int64_t tb = (int64_t)((by + dby) * a.ntx + (bx + dbx)) * (6 * (a.tx + a.ty));
-            const int off = dbx != 0
-                ? (cx(i) > 0 ? 0 : 3 * a.ty) + (i / 3) * a.ty + (ly - cy(i) - dby * a.ty)
-                : 6 * a.ty + (cy(i) > 0 ? 0 : 3 * a.tx) + (i % 3) * a.tx + (lx - cx(i));
+            if (!H.crosses_y(i) && !H.crosses_x(i)) continue;
             fixmask |= 1u << i;
-            fix[i] = Codec<S>::dec(a.halo_rd[tb + off]);
+            fix[i] = Codec<S>::dec(H.crosses_y(i) ? *H.at_y(i) : *H.at_x(i));
         }
     } else if (fluid && !(x > x0 && x < x1 && y > y0 && y < y1)) {
 #pragma unroll
@@ -1020,7 +1056,7 @@ __device__ __forceinline__ void nsol_tile(const Step<S> &a, int bx, int by, int 
 #pragma unroll
         for (int i = 0; i < 9; ++i) lat[addr<L>(a.N, n, opp(i))] = e[i];
         if (!(x > x0 && x < x1 && y > y0 && y < y1))
-            halo_publish(a.halo_wr, a.tx, a.ty, a.ntx, bx, by, x, y, x0, y0, x1, y1, e);
+            halo_publish(a, a.halo_wr, bx, by, x, y, x0, y0, x1, y1, e);
     } else if (zero_fill) {
         store_zero<S, L>(lat, a.N, n, a.off32);
     }
@@ -1431,7 +1467,7 @@ __global__ void k_publish(const Step<S> a, S *hw, int rev) {
     S e[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) e[i] = a.src[addr<L>(a.N, n, rev ? opp(i) : i)];
-    halo_publish(hw, a.tx, a.ty, a.ntx, bx, by, x, y, x0, y0, x1, y1, e);
+    halo_publish(a, hw, bx, by, x, y, x0, y0, x1, y1, e);
 }
 
 // Moments from a stored state: rho = 1 + sum h, v = sum h c (- F/2 for a
