@@ -173,7 +173,7 @@ static cudaError_t launch3(lbm3_lattice *L, cudaStream_t st, int64_t count, int 
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
-    return launch_bump_counter(L->tctr, count, st);
+    return lbm_draws(&L->p) ? launch_bump_counter(L->tctr, count, st) : cudaSuccess;
 }
 
 extern "C" lbm_status lbm3_workspace_bytes(const lbm3_params *p, size_t *bytes) {

@@ -90,6 +90,7 @@ struct lbm3_batch {
     cudaStream_t stream, cap;
     unsigned int *err;
     long long *tctr;
+    bool draws;    // some box uses stochastic rounding (the update counter's only reader)
     int cur;
     int64_t steps;
     cudaGraphExec_t graph[2];
@@ -134,6 +135,7 @@ extern "C" lbm_status lbm3_batch_create(int32_t ncases, const lbm3_params *param
     B->ncases = ncases;
     B->p0 = params[0];
     B->ops = ops3_for(params[0].storage);
+    for (int c = 0; c < ncases; ++c) B->draws = B->draws || lbm_draws(&params[c]);
     B->ws = (char *)d_workspace;
     B->stream = (cudaStream_t)cuda_stream;
     B->err = (unsigned int *)(B->ws + B->bl.misc_off);
@@ -208,7 +210,7 @@ static cudaError_t batch3_block(lbm3_batch *B, cudaStream_t st, int64_t count, i
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
-    return lbm::launch_bump_counter(B->tctr, count, st);
+    return B->draws ? lbm::launch_bump_counter(B->tctr, count, st) : cudaSuccess;
 }
 
 extern "C" lbm_status lbm3_batch_step(lbm3_batch *B, int64_t nsteps, uint32_t want_moments) {

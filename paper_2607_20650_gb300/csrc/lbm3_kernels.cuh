@@ -311,6 +311,7 @@ __device__ __forceinline__ void step3_node(const Step3<S> &a, uint32_t x, uint32
     const uint32_t nx = (uint32_t)a.g.nx, ny = (uint32_t)a.g.ny;
     const uint32_t n = (z * ny + y) * nx + x;
     const uint32_t lk = a.links[n];
+    chain_wait();
     const bool f = lk != SOLID;
     if (a.zero_fill) {
         const int lane = (int)(((threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x) & 31u);
@@ -328,6 +329,7 @@ __device__ __forceinline__ void step3_node(const Step3<S> &a, uint32_t x, uint32
 template <class S, int L, bool LINEAR, bool OFF32>
 __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 2 : 3) k3_step(const Step3<S> a) {
     uint32_t x, y, z;
+    chain_next();
     if (LINEAR) {
         const uint64_t n64 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
         if (n64 >= a.N) return;
@@ -415,6 +417,7 @@ __device__ __forceinline__ void pull3_pair(const Step3<S> &a, uint32_t x, uint32
 template <class S, int L>
 __device__ __forceinline__ void step3_pair(const Step3<S> &a, uint32_t x, uint32_t y, uint32_t z, uint32_t n) {
     const uint2 lk2 = *reinterpret_cast<const uint2 *>(a.links + n);   // n even: 8-byte aligned
+    chain_wait();
     const bool fa = lk2.x != SOLID, fb = lk2.y != SOLID;
     if (!fa && !fb) return;
     f2 g[Q];
@@ -485,6 +488,7 @@ __device__ __forceinline__ void step3_pair(const Step3<S> &a, uint32_t x, uint32
 template <class S, int L, bool LINEAR>
 __global__ void __launch_bounds__(256, LBM3_PAIR_MINB) k3_step_pair(const Step3<S> a) {
     uint32_t x, y, z, n;
+    chain_next();
     if (LINEAR) {
         const uint64_t n64 = 2ull * ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x);
         if (n64 >= a.N) return;
@@ -516,9 +520,11 @@ __global__ void __launch_bounds__(512, PHASE == 0 ? (sizeof(S) == 8 ? 1 : 2) : (
     const uint32_t x = blockIdx.x * a.tx + threadIdx.x;
     const uint32_t y = blockIdx.y * a.ty + threadIdx.y;
     const uint32_t z = blockIdx.z * a.tz + threadIdx.z;
+    chain_next();
     if (x >= nx || y >= ny || z >= nz) return;
     const uint32_t n = (z * ny + y) * nx + x;
     const uint32_t lk = a.links[n];
+    chain_wait();
     if (lk == SOLID) return;
     S *lat = a.dst;
     C g[Q];
@@ -702,6 +708,7 @@ __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw
         n = ((uint32_t)p[2] * ny + (uint32_t)p[1]) * nx + (uint32_t)p[0];
         lk = a.links[n];
     }
+    chain_wait();
     const bool fluid = lk != SOLID;
     const Halo3<OFF32> H(a.g, nt, b, p, lo, hi);
     C g[Q];
@@ -751,6 +758,7 @@ __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw
 
 template <class S, int L, bool OFF32>
 __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 2) k3_npol(const Step3<S> a, const S *hr, S *hw) {
+    chain_next();
     const int b[3] = {(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
     const int nt[3] = {(int)gridDim.x, (int)gridDim.y, (int)gridDim.z};
     npol3_tile<S, L, OFF32>(a, hr, hw, b, nt);
@@ -800,6 +808,7 @@ __device__ __forceinline__ void nsol3_tile(const Step3<S> &a, const S *hr, S *hw
         n = ((uint32_t)p[2] * ny + (uint32_t)p[1]) * nx + (uint32_t)p[0];
         lk = a.links[n];
     }
+    chain_wait();
     const bool fluid = lk != SOLID;
     if (fluid) {
 #pragma unroll
@@ -865,6 +874,7 @@ __device__ __forceinline__ void nsol3_tile(const Step3<S> &a, const S *hr, S *hw
 template <class S, int L>
 __global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 2) k3_nsol(const Step3<S> a, const S *hr, S *hw) {
     extern __shared__ __align__(16) unsigned char smem_nsol3[];
+    chain_next();
     const int b[3] = {(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
     const int nt[3] = {(int)gridDim.x, (int)gridDim.y, (int)gridDim.z};
     nsol3_tile<S, L>(a, hr, hw, b, nt, reinterpret_cast<typename Codec<S>::C *>(smem_nsol3));
@@ -1057,6 +1067,7 @@ __global__ void __launch_bounds__(batch3_threads(ALGO), batch3_min_blocks(ALGO, 
     k3_batch(const Case3<S> *cases, const uint2 *items, int src, int toff, int mom) {
     __shared__ __align__(16) unsigned char raw[sizeof(Step3<S>)];
     Step3<S> &a = *reinterpret_cast<Step3<S> *>(raw);
+    chain_next();
     const uint2 it = items[blockIdx.x];
     const Case3<S> &cs = cases[it.x];
     const int tid = (int)((threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x);

@@ -99,6 +99,7 @@ struct lbm_batch {
     unsigned int *err;
     long long *tctr;
     int grid;
+    bool draws;    // some case uses stochastic rounding (the update counter's only reader)
     int kind;      // layout * 4 + algo shared by every case, -1 if mixed
     int cur;
     int64_t steps;
@@ -186,6 +187,7 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
         lbm_batch_destroy(B);
         return lbm_cuda_fail(e, "batch upload");
     }
+    for (int c = 0; c < ncases; ++c) B->draws = B->draws || lbm_draws(&params[c]);
     B->kind = params[0].layout * 4 + params[0].algo;
     for (int c = 1; c < ncases; ++c)
         if (params[c].layout * 4 + params[c].algo != B->kind) B->kind = -1;
@@ -214,7 +216,7 @@ static cudaError_t batch_block(lbm_batch *B, cudaStream_t st, int64_t count, int
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
-    return launch_bump_counter(B->tctr, count, st);
+    return B->draws ? launch_bump_counter(B->tctr, count, st) : cudaSuccess;
 }
 
 extern "C" lbm_status lbm_batch_step(lbm_batch *B, int64_t nsteps, uint32_t want_moments) {

@@ -293,7 +293,14 @@ void lbm_fill_args(const lbm_params *p, const Plan &pl, char *ws, const Ops *ops
     h->ntx = pl.ntx;
     h->nty = pl.nty;
     ops->prepare();
+    int dev = 0;
+    h->sms = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        (void)cudaGetLastError();
     h->block_1d = p->algo == LBM_LPTL ? ops->lptl_block(p->layout) : 0;
+    // a lattice of few blocks is cut into smaller ones that spread over all SMs
+    while (h->block_1d > 64 && (pl.N + h->block_1d - 1) / h->block_1d < 4 * (int64_t)h->sms) h->block_1d /= 2;
     h->flags = p->flags;
     h->nx_magic = p->nx == 1 ? 0ull : (~0ull / (uint64_t)p->nx) + 1ull;
     h->pf = prefetch_distance(p, pl.N, ops->elem, pl.tx);
@@ -435,7 +442,8 @@ static cudaError_t launch_block(lbm_lattice *L, cudaStream_t st, int64_t count, 
         if (two) cur ^= 1;
         ++steps;
     }
-    return launch_bump_counter(L->h.tctr, count, st);
+    // the update counter only keys stochastic rounding
+    return lbm_draws(&L->p) ? launch_bump_counter(L->h.tctr, count, st) : cudaSuccess;
 }
 
 static lbm_status get_graph(lbm_lattice *L, cudaGraphExec_t *out) {

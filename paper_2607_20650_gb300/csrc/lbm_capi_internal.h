@@ -44,6 +44,11 @@ struct lbm_lattice {
     cudaEvent_t stage_ev[2];
 };
 
+// Whether the updates of a lattice or box draw random numbers.
+template <class P> inline bool lbm_draws(const P *p) {
+    return p->rounding == LBM_ROUND_SR && (p->storage == LBM_F16S || p->storage == LBM_BF16S);
+}
+
 lbm_status lbm_fail(lbm_status s, const char *fmt, ...);
 // Tensor map (TMA descriptor) of an FP32 tensor of `rank` dimensions (dims
 // innermost first, byte strides of dimensions 1 .. rank-1, copy box); false

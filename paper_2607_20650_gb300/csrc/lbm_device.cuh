@@ -56,6 +56,17 @@ template <> struct Ar<double> {
     static __device__ __forceinline__ double fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 };
 
+// ------------------------------------------------------------ chained launches
+// Update kernels are launched so that the next update's blocks may become
+// resident, and load what no update writes (node indices, link bytes, case
+// records), while the last blocks of this one still run (programmatic
+// dependent launch). chain_next() lets the next grid start once every block
+// of this one has; chain_wait() returns when the previous grid has completed
+// and its stores are visible, and comes before the first access to the
+// lattice, the buffer grid, the moments or the update counter.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------ hashing
 // 32-bit integer finaliser "lowbias32" (C. Wellons, hash-prospector).
 __host__ __device__ __forceinline__ uint32_t mix32(uint32_t x) {

@@ -14,6 +14,24 @@ struct alignas(64) TmaDesc {
     unsigned char bytes[128];
 };
 
+// Launch of an update kernel (one that calls chain_wait before it touches what
+// updates write): its blocks may start before the previous kernel on the
+// stream has ended.
+template <class... P, class... A>
+inline cudaError_t launch_update(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...a) {
+    cudaLaunchConfig_t c = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(a)...);
+}
+
 // Everything a kernel launch needs, in host types.
 struct HostArgs {
     int nx, ny;
@@ -24,6 +42,7 @@ struct HostArgs {
     uint64_t seed;
     int tile_x, tile_y, ntx, nty;
     int block_1d;              // LPTL block size
+    int sms;                   // SMs of the device
     uint32_t flags;            // lbm_params.flags
     uint64_t nx_magic;         // ceil(2^64 / nx) for n -> (x, y); 0 when nx == 1
     uint32_t pf;               // L2 prefetch distance: nodes (LPTL) or rows (NPTL); 0 = off

@@ -317,10 +317,11 @@ __device__ __forceinline__ void two_lattice_fluid(const Step<S> &a, uint32_t x, 
 
 // One node of the two-lattice pull update (LPTL and NPTL). lane: the
 // thread's lane (the zero fill below votes over the warp).
-template <class S, int L>
+template <class S, int L, bool CHAIN = true>
 __device__ __forceinline__ void two_lattice_node(const Step<S> &a, uint32_t x, uint32_t y, int lane) {
     const uint32_t n = y * (uint32_t)a.geo.nx + x;
     const uint32_t lk = a.links[n];
+    if (CHAIN) chain_wait();
     const bool fluid = lk != SOLID_LINKS;
     const unsigned F = __ballot_sync(__activemask(), fluid);
     if (!fluid) {
@@ -341,6 +342,7 @@ __global__ void __launch_bounds__(kMaxTileThreads) k_two_lattice2(const Step<S> 
     using C = typename Codec<S>::C;
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     const uint32_t x = blockIdx.x * a.tx + threadIdx.x;
+    chain_next();
     const uint32_t ya = blockIdx.y * a.ty + threadIdx.y, yb = ya + (uint32_t)(a.ty >> 1);
     if (x >= nx || ya >= ny) return;
     const int lane = (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u);
@@ -348,6 +350,7 @@ __global__ void __launch_bounds__(kMaxTileThreads) k_two_lattice2(const Step<S> 
     const uint32_t na = ya * nx + x, nb = yb * nx + x;
     const uint32_t lka = a.links[na];
     const uint32_t lkb = hb ? (uint32_t)a.links[nb] : SOLID_LINKS;
+    chain_wait();
     const bool fa = lka != SOLID_LINKS, fb = lkb != SOLID_LINKS;
     const unsigned act = __activemask();
     const unsigned Fa = __ballot_sync(act, fa), Fb = __ballot_sync(act, hb && fb);
@@ -397,9 +400,11 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two
     const int lane = tid & 31, warp = tid >> 5;
     const uint32_t x = blockIdx.x * a.tx + threadIdx.x;
     const uint32_t y = blockIdx.y * a.ty + threadIdx.y;
+    chain_next();
     if (x >= nx || y >= ny) return;
     const uint32_t n = y * nx + x;
     const uint32_t lk = a.links[n];
+    chain_wait();
     const bool fluid = lk != SOLID_LINKS;
     const unsigned act = __activemask();
     const unsigned F = __ballot_sync(act, fluid);
@@ -489,12 +494,17 @@ __device__ __forceinline__ void prefetch_record(const S *src, uint32_t N, uint32
 // by instruction issue (the prefetch cost 3 %), and the collision layout's
 // LPTL form spills at 32 registers with it (its NPTL form is the staged
 // kernel above).
-template <class S, int L, bool LINEAR>
+// CHAIN: a chained launch (launch_update). Off for large lattices, where the
+// gap between updates is nothing and the wait between the loads costs 0.9 %
+// (134M nodes, FP32 bundle: 1.199 against 1.210 ms).
+constexpr int64_t kChainNodes = 4 << 20;
+template <class S, int L, bool LINEAR, bool CHAIN = true>
 __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two_lattice(const Step<S> a) {
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     constexpr bool PF = sizeof(S) == 4 && L != COLLISION;
     uint32_t x, y, np = 0;
     bool ahead;
+    if (CHAIN) chain_next();
     if (LINEAR) {
         const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
         if (n >= a.N) return;
@@ -510,7 +520,7 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two
         np = (y + a.pf) * nx + x;
     }
     const uint32_t lkp = ahead ? (uint32_t)a.links[np] : SOLID_LINKS;
-    two_lattice_node<S, L>(a, x, y, (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
+    two_lattice_node<S, L, CHAIN>(a, x, y, (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
     if (PF && lkp != SOLID_LINKS) prefetch_record<S, L>(a.src, a.N, np);
 }
 
@@ -711,6 +721,7 @@ __global__ void __launch_bounds__(kMaxTileThreads / 2, LBM_PAIR_MINB) k_two_latt
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     uint32_t x, y, n, np;
     bool ahead;
+    chain_next();
     if (LINEAR) {
         n = 2u * (blockIdx.x * blockDim.x + threadIdx.x);
         if (n >= a.N) return;
@@ -728,6 +739,7 @@ __global__ void __launch_bounds__(kMaxTileThreads / 2, LBM_PAIR_MINB) k_two_latt
     }
     const uint32_t lkp = ahead ? (uint32_t)*reinterpret_cast<const unsigned short *>(a.links + np) : 0xFFFFu;
     const uint32_t lk2 = *reinterpret_cast<const unsigned short *>(a.links + n);
+    chain_wait();
     pair_update<S, L>(a, x, y, n, lk2, (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
     if (lkp != 0xFFFFu) prefetch_pair<S, L>(a.src, a.N, np);
 }
@@ -883,6 +895,7 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
         n = (uint32_t)y * (uint32_t)nx + (uint32_t)x;
         lk = a.links[n];
     }
+    chain_wait();
     const bool fluid = lk != SOLID_LINKS;
     const unsigned F = __ballot_sync(__activemask(), fluid);
     (void)F;
@@ -933,12 +946,13 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
 
 // Registers: 32 (four 512-thread blocks, spills) for the stream layout and
 // 16-bit storage, 40 (three) where it measured faster: 6000 x 3001 nodes, 16
-// updates, FP32 bundle 64 x 4 3.89 against 3.90 ms and 128 x 4 4.35 against
-// 4.09, collision 5.41 / 4.88, stream 32 x 8 4.11 / 4.29, FP16 3.85 / 3.95.
+// updates, 32 / 40 registers: FP32 bundle 64 x 4 3.89 / 3.90 ms and 128 x 4
+// 4.35 / 4.09, collision 5.41 / 4.88, stream 32 x 8 4.11 / 4.29, FP16 3.85 / 3.95.
 template <class S, int L>
 __global__ void __launch_bounds__(kMaxTileThreads,
                                   sizeof(S) == 8 ? 1 : (sizeof(S) == 4 && L != STREAM) || L == COLLISION ? 3 : 4)
     k_npol(const Step<S> a) {
+    chain_next();
     npol_tile<S, L>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
                     (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
 }
@@ -956,6 +970,7 @@ __device__ __forceinline__ void nsol_tile(const Step<S> &a, int bx, int by, int 
     // slot of direction s of tile node t among the staged values
     auto si = [T](int s, int t) { return (TMA && L == BUNDLE) ? (s / 3) * 3 * T + 3 * t + s % 3 : s * T + t; };
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem_raw + sizeof(C) * 9 * T);
+    chain_wait();
     if constexpr (TMA) {
         if (lx == 0 && ly == 0)
             tma_issue_3d(tm, sm, bar, L == BUNDLE ? 3 * bx * a.tx : bx * a.tx, by * a.ty, 0,
@@ -1068,6 +1083,7 @@ __device__ __forceinline__ void nsol_tile(const Step<S> &a, int bx, int by, int 
 template <class S, int L>
 __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : LBM_NSOL_MINB) k_nsol(const Step<S> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_next();
     nsol_tile<S, L>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
                     (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u), smem_raw);
 }
@@ -1078,6 +1094,7 @@ template <class S, int L>
 __global__ void __launch_bounds__(kMaxTileThreads, LBM_NSOL_MINB)
     k_nsol_tma(const Step<S> a, const __grid_constant__ TmaDesc tm) {
     extern __shared__ __align__(128) unsigned char smem_tma[];
+    chain_next();
     nsol_tile<S, L, true>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
                           (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u), smem_tma, &tm);
 }
@@ -1102,6 +1119,7 @@ __device__ __forceinline__ void aa_node(const Step<S> &a, uint32_t x, uint32_t y
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     const uint32_t n = y * nx + x;
     const uint32_t lk = a.links[n];
+    chain_wait();
     S *lat = a.dst;
     const bool fluid = lk != SOLID_LINKS;
     const unsigned F = __ballot_sync(__activemask(), fluid);
@@ -1238,6 +1256,7 @@ __device__ __forceinline__ void aa_node(const Step<S> &a, uint32_t x, uint32_t y
 
 template <class S, int L, int PHASE>
 __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : (PHASE == 0 || L == STREAM ? 3 : 4)) k_aa(const Step<S> a) {
+    chain_next();
     const uint32_t x = blockIdx.x * a.tx + threadIdx.x;
     const uint32_t y = blockIdx.y * a.ty + threadIdx.y;
     if (x >= (uint32_t)a.geo.nx || y >= (uint32_t)a.geo.ny) return;
@@ -1285,7 +1304,7 @@ __device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uin
             const uint32_t n = (t * kBatchSuper + k) * (uint32_t)kBatchThreads + (uint32_t)tid;
             if (n < a.N) {
                 const uint32_t y = a.nx_magic ? (uint32_t)__umul64hi((unsigned long long)n, a.nx_magic) : n;
-                two_lattice_node<S, L>(a, n - y * (uint32_t)a.geo.nx, y, lane);
+                two_lattice_node<S, L, false>(a, n - y * (uint32_t)a.geo.nx, y, lane);
             }
         }
         return;
@@ -1300,7 +1319,7 @@ __device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uin
             const uint32_t by = bc.ntx_magic ? (uint32_t)__umul64hi((unsigned long long)tt, bc.ntx_magic) : tt;
             const uint32_t bx = tt - by * (uint32_t)a.ntx;
             const int x = (int)bx * a.tx + lx, y = (int)by * a.ty + ly;
-            if (ly < a.ty && x < a.geo.nx && y < a.geo.ny) two_lattice_node<S, L>(a, x, y, lane);
+            if (ly < a.ty && x < a.geo.nx && y < a.geo.ny) two_lattice_node<S, L, false>(a, x, y, lane);
         }
         return;
     }
@@ -1604,65 +1623,73 @@ bool pairs_ok(const HostArgs &h) {
            !(h.flags & 0x20u);
 }
 
+// Rows of a tile that one block of the per-node kernels (no exchange within a
+// tile) updates: a lattice of few tiles is cut into smaller blocks, so that
+// its nodes spread over all SMs. 256 x 64 nodes in 32 x 8 tiles are 64 blocks on
+// 152 SMs, and the FP64 lanes of 88 SMs are idle; in blocks of 32 x 1, chained, an
+// FP64 update takes 6.5 instead of 6.95 us.
+inline int rows_per_block(const HostArgs &h) {
+    int ty = h.tile_y;
+    int64_t blocks = (int64_t)h.ntx * h.nty;
+    while (blocks < 4 * (int64_t)h.sms && ty % 2 == 0 && h.tile_x * ty >= 64) {
+        ty /= 2;
+        blocks = (int64_t)h.ntx * ((h.ny + ty - 1) / ty);
+    }
+    return ty;
+}
+
 template <class S, int L>
-cudaError_t step_layout(const HostArgs &h, const Step<S> &a, int phase, cudaStream_t st) {
+cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStream_t st) {
     using C = typename Codec<S>::C;
     const dim3 tile(h.tile_x, h.tile_y), grid(h.ntx, h.nty);
-    switch (h.algo) {
-        case LPTL: {
-            if constexpr (sizeof(S) == 2 && L == BUNDLE) {
-                if (pairs_ok<S, L>(h)) {
-                    const int b = 128;
-                    const unsigned g = (unsigned)((h.N / 2 + b - 1) / b);
-                    k_two_lattice_pair<S, L, true><<<g, b, 0, st>>>(a);
-                    break;
-                }
+    Step<S> a = a0;
+    if (h.algo == LPTL) {
+        if constexpr (sizeof(S) == 2 && L == BUNDLE) {
+            if (pairs_ok<S, L>(h)) {
+                const int b = 128;
+                return launch_update(k_two_lattice_pair<S, L, true>, dim3((unsigned)((h.N / 2 + b - 1) / b)), dim3(b), 0,
+                                     st, a);
             }
-            const int b = h.block_1d;
-            const unsigned g = (unsigned)((h.N + b - 1) / b);
-            k_two_lattice<S, L, true><<<g, b, 0, st>>>(a);
-            break;
         }
-        case NPTL:
-            if (L == COLLISION && h.tile_x % 32 == 0 && !(h.flags & 4u)) {
-                const size_t sm = (size_t)AosSpan<S>::WARP_BYTES * ((h.tile_x * h.tile_y + 31) / 32);
-                k_two_lattice_aos<S><<<grid, tile, sm, st>>>(a);
-                break;
-            }
-            if constexpr (sizeof(S) == 2 && L == BUNDLE) {
-                if (pairs_ok<S, L>(h) && !(h.tile_x & 1)) {
-                    k_two_lattice_pair<S, L, false><<<grid, dim3(h.tile_x / 2, h.tile_y), 0, st>>>(a);
-                    break;
-                }
-            }
-            // Two nodes per thread on request (4- and 8-byte storage): one node
-            // per thread at 32 registers keeps full occupancy and measured faster.
-            if (sizeof(S) >= 4 && h.tile_y >= 2 && !(h.tile_y & 1) && (h.flags & 2u))
-                k_two_lattice2<S, L><<<grid, dim3(h.tile_x, h.tile_y / 2), 0, st>>>(a);
-            else
-                k_two_lattice<S, L, false><<<grid, tile, 0, st>>>(a);
-            break;
-        case NPOL: k_npol<S, L><<<grid, tile, 0, st>>>(a); break;
-        case NSOL: {
-            const size_t sm = sizeof(C) * 9 * h.tile_x * h.tile_y;
-            if constexpr (std::is_same<S, float>::value && L != COLLISION) {
-                if (h.tma) {
-                    k_nsol_tma<S, L><<<grid, tile, sm + 16, st>>>(a, h.tmap);
-                    break;
-                }
-            }
-            k_nsol<S, L><<<grid, tile, sm, st>>>(a);
-            break;
+        const int b = h.block_1d;
+        const dim3 blocks((unsigned)((h.N + b - 1) / b));
+        if (h.N > kChainNodes) {
+            k_two_lattice<S, L, true, false><<<blocks, b, 0, st>>>(a);
+            return cudaGetLastError();
         }
-        case AA:
-            if (phase)
-                k_aa<S, L, 1><<<grid, tile, 0, st>>>(a);
-            else
-                k_aa<S, L, 0><<<grid, tile, 0, st>>>(a);
-            break;
-        default: return cudaErrorInvalidValue;
+        return launch_update(k_two_lattice<S, L, true>, blocks, dim3(b), 0, st, a);
     }
-    return cudaGetLastError();
+    if (h.algo == NPOL) return launch_update(k_npol<S, L>, grid, tile, 0, st, a);
+    if (h.algo == NSOL) {
+        const size_t sm = sizeof(C) * 9 * h.tile_x * h.tile_y;
+        if constexpr (std::is_same<S, float>::value && L != COLLISION) {
+            if (h.tma) return launch_update(k_nsol_tma<S, L>, grid, tile, sm + 16, st, a, h.tmap);
+        }
+        return launch_update(k_nsol<S, L>, grid, tile, sm, st, a);
+    }
+    if (h.algo == NPTL) {
+        if (L == COLLISION && h.tile_x % 32 == 0 && !(h.flags & 4u)) {
+            const size_t sm = (size_t)AosSpan<S>::WARP_BYTES * ((h.tile_x * h.tile_y + 31) / 32);
+            return launch_update(k_two_lattice_aos<S>, grid, tile, sm, st, a);
+        }
+        if constexpr (sizeof(S) == 2 && L == BUNDLE) {
+            if (pairs_ok<S, L>(h) && !(h.tile_x & 1))
+                return launch_update(k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st, a);
+        }
+        // Two nodes per thread on request (4- and 8-byte storage): one node
+        // per thread at 32 registers keeps full occupancy and measured faster.
+        if (sizeof(S) >= 4 && h.tile_y >= 2 && !(h.tile_y & 1) && (h.flags & 2u))
+            return launch_update(k_two_lattice2<S, L>, grid, dim3(h.tile_x, h.tile_y / 2), 0, st, a);
+    }
+    if (h.algo == NPTL && h.N > kChainNodes) {
+        k_two_lattice<S, L, false, false><<<grid, tile, 0, st>>>(a);
+        return cudaGetLastError();
+    }
+    a.ty = rows_per_block(h);
+    const dim3 cut(h.tile_x, a.ty), cuts(h.ntx, (h.ny + a.ty - 1) / a.ty);
+    if (h.algo == NPTL) return launch_update(k_two_lattice<S, L, false>, cuts, cut, 0, st, a);
+    if (h.algo != AA) return cudaErrorInvalidValue;
+    return phase ? launch_update(k_aa<S, L, 1>, cuts, cut, 0, st, a) : launch_update(k_aa<S, L, 0>, cuts, cut, 0, st, a);
 }
 
 template <class S>
