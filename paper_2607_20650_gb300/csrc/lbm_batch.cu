@@ -70,7 +70,7 @@ lbm_status batch_layout(int32_t ncases, const lbm_params *params, BatchLayout *b
     const Ops *ops = ops_for_storage(storage);
     bl->ntiles = (uint32_t)tiles;
     bl->cases_off = 0;
-    bl->tiles_off = align256(ops->batch_case_bytes * ncases);
+    bl->tiles_off = align256(4 * ops->batch_case_bytes * ncases);   // parities, without and with moments
     bl->misc_off = bl->tiles_off + align256(sizeof(uint32_t) * 2 * (size_t)tiles);
     bl->header = bl->misc_off + 256;
     size_t off = bl->header;
@@ -101,6 +101,7 @@ struct lbm_batch {
     int grid;
     bool draws;    // some case uses stochastic rounding (the update counter's only reader)
     int kind;      // layout * 4 + algo shared by every case, -1 if mixed
+    int pf;        // L2 prefetch within the work items: the lattices exceed the L2 cache
     int cur;
     int64_t steps;
     cudaGraphExec_t graph[2];
@@ -157,7 +158,8 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
         delete B;
         return lbm_cuda_fail(e, "cudaStreamCreateWithFlags");
     }
-    std::vector<unsigned char> recs(B->ops->batch_case_bytes * ncases);
+    const size_t rec = B->ops->batch_case_bytes;
+    std::vector<unsigned char> recs(4 * rec * ncases);
     std::vector<uint32_t> tiles;
     tiles.reserve(2 * (size_t)B->bl.ntiles);
     for (int c = 0; c < ncases; ++c) {
@@ -170,7 +172,7 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
         B->cases.push_back(L);
         L->h.err = B->err;        // one divergence flag and update counter for the batch
         L->h.tctr = B->tctr;
-        B->ops->batch_case(L->h, recs.data() + (size_t)c * B->ops->batch_case_bytes);
+        for (int m = 0; m < 4; ++m) B->ops->batch_case(L->h, m & 1, m >> 1, recs.data() + ((size_t)m * ncases + c) * rec);
         const int64_t nt = case_tiles(params[c], B->bl.plans[c]);
         for (int64_t t = 0; t < nt; ++t) {
             tiles.push_back((uint32_t)c);
@@ -191,6 +193,12 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
     B->kind = params[0].layout * 4 + params[0].algo;
     for (int c = 1; c < ncases; ++c)
         if (params[c].layout * 4 + params[c].algo != B->kind) B->kind = -1;
+    double lattices = 0.0;   // bytes of the source lattices
+    for (int c = 0; c < ncases; ++c) lattices += 9.0 * (double)B->bl.plans[c].N * (double)B->ops->elem;
+    int dev = 0, l2 = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+        (void)cudaGetLastError();
+    B->pf = l2 > 0 && lattices > (double)l2 && !(params[0].flags & LBM_FLAG_NO_PREFETCH) ? 1 : 0;
     const int g = B->ops->batch_grid(B->kind);
     B->grid = (int)std::max<int64_t>(1, std::min<int64_t>(g > 0 ? g : 152, B->bl.ntiles));
     *out = B;
@@ -211,8 +219,8 @@ extern "C" lbm_status lbm_batch_init(lbm_batch *B, int32_t c, const double *rho,
 static cudaError_t batch_block(lbm_batch *B, cudaStream_t st, int64_t count, int want_moments) {
     int cur = B->cur;
     for (int64_t k = 0; k < count; ++k) {
-        cudaError_t e = B->ops->batch_step(B->kind, B->d_cases, B->d_tiles, B->bl.ntiles, B->grid, cur, (int)k,
-                                           (want_moments && k == count - 1) ? 1 : 0, st);
+        cudaError_t e = B->ops->batch_step(B->kind, B->d_cases, B->ncases, B->d_tiles, B->bl.ntiles, B->grid, cur,
+                                           (int)k, (want_moments && k == count - 1) ? 1 : 0, B->pf, st);
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
