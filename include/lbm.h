@@ -179,10 +179,10 @@ lbm_status lbm_wait(lbm_lattice *L, double timeout_s);
 
 /* Moments of the last update that stored them (or of lbm_init), as host
  * doubles, N each (solid nodes: rho = 1, v = 0); a NULL array is skipped.
- * Synchronous. Page-locked destinations (cudaHostAlloc, cudaHostRegister)
- * are written by the device directly; pageable ones of more than 64 MB per
- * field go through page-locked staging the lattice allocates on first use
- * (128 MB of host memory, freed by lbm_destroy). */
+ * Synchronous. FP32 moments are widened by the device straight into
+ * page-locked destinations (cudaHostAlloc, cudaHostRegister) and into
+ * pageable ones of 8 MB and more, which are page-locked during the call;
+ * smaller ones, and memory that cannot be locked, on the host. */
 lbm_status lbm_read_moments(lbm_lattice *L, double *rho, double *ux, double *uy);
 
 /* Same moments as FP32 device arrays (N each), enqueued on the stream. */
@@ -200,7 +200,9 @@ lbm_status lbm_force(lbm_lattice *L, const uint8_t *d_body, double out[2]);
 
 /* Copy the state to / from host memory in canonical order h[i*N + n],
  * as = LBM_F64 (double) or LBM_F32 (float). Writes round to the storage
- * type (via FP32 for F16S/BF16S, nearest-even). Synchronous. */
+ * type (via FP32 for F16S/BF16S, nearest-even). Synchronous. The device
+ * converts; pageable buffers of 1 MB and more are page-locked during the
+ * call (memory that cannot be locked is copied and converted on the host). */
 lbm_status lbm_read_populations(lbm_lattice *L, void *host, int32_t as);
 lbm_status lbm_write_populations(lbm_lattice *L, const void *host, int32_t as);
 

@@ -345,18 +345,17 @@ extern "C" lbm_status lbm3_sync(lbm3_lattice *L) {
 extern "C" lbm_status lbm3_read_moments(lbm3_lattice *L, double *rho, double *ux, double *uy, double *uz) {
     if (!L) return lbm_fail(LBM_EINVAL, "lattice is NULL");
     const int64_t N = L->pl.N;
-    std::vector<unsigned char> buf(4 * (size_t)N * L->pl.comp);
-    CK3(cudaStreamSynchronize(L->stream));
-    CK3(cudaMemcpy(buf.data(), L->ws + L->pl.mom, buf.size(), cudaMemcpyDeviceToHost));
+    const char *mom = L->ws + L->pl.mom;
     double *dst[4] = {rho, ux, uy, uz};
-    for (int k = 0; k < 4; ++k) {
-        if (!dst[k]) continue;
-        if (L->pl.comp == 8) {
-            memcpy(dst[k], buf.data() + (size_t)k * N * 8, (size_t)N * 8);
-        } else {
-            const float *f = (const float *)(buf.data() + (size_t)k * N * 4);
-            for (int64_t n = 0; n < N; ++n) dst[k][n] = f[n];
-        }
+    if (L->pl.comp == 8) {
+        for (int k = 0; k < 4; ++k)
+            if (dst[k])
+                CK3(cudaMemcpyAsync(dst[k], (const double *)mom + (size_t)k * N, (size_t)N * 8, cudaMemcpyDeviceToHost,
+                                    L->stream));
+        CK3(cudaStreamSynchronize(L->stream));
+    } else {
+        const lbm_status s = lbm_widen_to_host((const float *)mom, N, 4, dst, L->stream);
+        if (s != LBM_OK) return s;
     }
     return lbm3_check(L);
 }
@@ -392,6 +391,14 @@ extern "C" lbm_status lbm3_read_populations(lbm3_lattice *L, void *host, int32_t
     if (state_readable(L) != LBM_OK) return LBM_EINVAL;
     if (as != LBM_F64 && as != LBM_F32) return lbm_fail(LBM_EINVAL, "as must be LBM_F64 or LBM_F32");
     const int64_t N = L->pl.N;
+    {
+        HostView v(host, 19 * (size_t)N * (as == LBM_F64 ? 8 : 4), true);
+        if (v.ok()) {
+            CK3(L->ops->transfer(L, v.dev(), nullptr, as == LBM_F64, L->stream));
+            CK3(cudaStreamSynchronize(L->stream));
+            return lbm3_check(L);
+        }
+    }
     std::vector<unsigned char> raw(19 * (size_t)N * L->pl.elem);
     CK3(cudaStreamSynchronize(L->stream));
     CK3(cudaMemcpy(raw.data(), L->ws + L->pl.pop[L->cur], raw.size(), cudaMemcpyDeviceToHost));
@@ -410,6 +417,15 @@ extern "C" lbm_status lbm3_write_populations(lbm3_lattice *L, const void *host, 
     if (state_readable(L) != LBM_OK) return LBM_EINVAL;
     if (as != LBM_F64 && as != LBM_F32) return lbm_fail(LBM_EINVAL, "as must be LBM_F64 or LBM_F32");
     const int64_t N = L->pl.N;
+    {
+        HostView v((void *)host, 19 * (size_t)N * (as == LBM_F64 ? 8 : 4), false);
+        if (v.ok()) {
+            CK3(L->ops->transfer(L, nullptr, v.dev(), as == LBM_F64, L->stream));
+            if (L->pl.halo_parity) CK3(L->ops->publish(L, L->cur, L->stream));
+            CK3(cudaStreamSynchronize(L->stream));
+            return LBM_OK;
+        }
+    }
     std::vector<unsigned char> raw(19 * (size_t)N * L->pl.elem);
     for (int i = 0; i < 19; ++i)
         for (int64_t n = 0; n < N; ++n) {

@@ -58,6 +58,9 @@ struct Ops3 {
                         cudaStream_t st);
     // rho, u of the stored state into the moments array.
     cudaError_t (*state_moments)(const lbm3_lattice *L, cudaStream_t st);
+    // The current state to `out` or from `in` (one of them null), canonical
+    // order in mapped host memory, doubles or floats.
+    cudaError_t (*transfer)(const lbm3_lattice *L, void *out, const void *in, bool f64, cudaStream_t st);
     // Fill buffer-grid parity `parity` from the stored state (NPOL, NSOL).
     cudaError_t (*publish)(const lbm3_lattice *L, int parity, cudaStream_t st);
     // FP64 block partial sums of the mass (one per block) and force (three).

@@ -923,6 +923,26 @@ __global__ void k3_init(const Step3<S> a, const double *rho, const double *ux, c
     }
 }
 
+// The stored state to / from canonical order in mapped host memory (as the 2-D
+// k_export / k_import; values of solid nodes are stored as given).
+template <class S, int L, class H>
+__global__ void __launch_bounds__(256) k3_export(const Step3<S> a, H *out) {
+    const uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= a.N) return;
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+        out[(uint64_t)i * a.N + n] = (H)Codec<S>::dec(a.src[addr<L>(a.N, (int64_t)n, slot3(a, i))]);
+}
+template <class S, int L, class H>
+__global__ void __launch_bounds__(256) k3_import(const Step3<S> a, const H *in) {
+    using C = typename Codec<S>::C;
+    const uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (n >= a.N) return;
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+        a.dst[addr<L>(a.N, (int64_t)n, slot3(a, i))] = Codec<S>::enc((C)in[(uint64_t)i * a.N + n], false, 0u);
+}
+
 template <class S, int L>
 __global__ void k3_state_moments(const Step3<S> a) {
     using C = typename Codec<S>::C;

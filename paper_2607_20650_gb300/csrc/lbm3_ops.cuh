@@ -230,6 +230,25 @@ cudaError_t init3(const lbm3_lattice *L, const double *const dv[4], uint32_t n0,
     return init_k<S, COLLISION>(L, dv, n0, c, st);
 }
 
+template <class S, int L>
+cudaError_t transfer_k(const lbm3_lattice *L_, void *out, const void *in, bool f64, cudaStream_t st) {
+    // current lattice as the source of an export and the destination of an import
+    const Step3<S> a = make3<S>(L_, in ? L_->cur ^ 1 : L_->cur, 0, 0);
+    const unsigned g = (unsigned)((L_->pl.N + 255) / 256);
+    if (out && f64) k3_export<S, L, double><<<g, 256, 0, st>>>(a, (double *)out);
+    else if (out) k3_export<S, L, float><<<g, 256, 0, st>>>(a, (float *)out);
+    else if (f64) k3_import<S, L, double><<<g, 256, 0, st>>>(a, (const double *)in);
+    else k3_import<S, L, float><<<g, 256, 0, st>>>(a, (const float *)in);
+    return cudaGetLastError();
+}
+
+template <class S>
+cudaError_t transfer3(const lbm3_lattice *L, void *out, const void *in, bool f64, cudaStream_t st) {
+    if (L->p.layout == LBM_LAYOUT_STREAM) return transfer_k<S, STREAM>(L, out, in, f64, st);
+    if (L->p.layout == LBM_LAYOUT_BUNDLE) return transfer_k<S, BUNDLE>(L, out, in, f64, st);
+    return transfer_k<S, COLLISION>(L, out, in, f64, st);
+}
+
 template <class S>
 cudaError_t state_moments3(const lbm3_lattice *L, cudaStream_t st) {
     const Step3<S> a = make3<S>(L, 0, 0, 1);
@@ -329,6 +348,7 @@ Ops3 make_ops3() {
     o.step = step3<S>;
     o.init = init3<S>;
     o.state_moments = state_moments3<S>;
+    o.transfer = transfer3<S>;
     o.publish = publish_state<S>;
     o.mass = mass3<S>;
     o.force = force3<S>;

@@ -40,14 +40,35 @@ struct lbm_lattice {
     unsigned long long *count;
     cudaGraphExec_t graph[4];
     int graph_steps;
-    char *stage;                // page-locked read-back staging (lazy), two chunks
-    cudaEvent_t stage_ev[2];
 };
 
 // Whether the updates of a lattice or box draw random numbers.
 template <class P> inline bool lbm_draws(const P *p) {
     return p->rounding == LBM_ROUND_SR && (p->storage == LBM_F16S || p->storage == LBM_BF16S);
 }
+
+// Device address of a host buffer for the duration of one synchronous call:
+// page-locked memory as it is, pageable memory of at least kRegisterBytes
+// page-locked for the call (released by the destructor, after the caller has
+// waited for its kernels). ok() is false where neither works (small buffers,
+// memory that cannot be locked): the caller then copies through the host.
+class HostView {
+  public:
+    HostView() = default;
+    HostView(void *p, size_t bytes, bool write) { open(p, bytes, write); }
+    ~HostView();
+    void open(void *p, size_t bytes, bool write);   // once
+    HostView(const HostView &) = delete;
+    HostView &operator=(const HostView &) = delete;
+    bool ok() const { return dev_ != nullptr; }
+    void *dev() const { return dev_; }
+
+  private:
+    void *dev_ = nullptr, *locked_ = nullptr;
+};
+
+// Up to four FP32 moments fields on the device to host doubles (lbm_capi.cu).
+lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *const *dst, cudaStream_t st);
 
 lbm_status lbm_fail(lbm_status s, const char *fmt, ...);
 // Tensor map (TMA descriptor) of an FP32 tensor of `rank` dimensions (dims

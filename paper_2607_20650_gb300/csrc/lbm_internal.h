@@ -75,6 +75,9 @@ struct Ops {
     cudaError_t (*publish)(const HostArgs &, int src, int parity, cudaStream_t);
     // Store h = 0 at every solid node of lattice `src`.
     cudaError_t (*zero_solid)(const HostArgs &, int src, cudaStream_t);
+    // Lattice src / dst to / from canonical order in mapped host memory (doubles or floats).
+    cudaError_t (*export_state)(const HostArgs &, int src, void *out, bool f64, cudaStream_t);
+    cudaError_t (*import_state)(const HostArgs &, int dst, const void *in, bool f64, cudaStream_t);
     // rho = 1 + sum h, v = sum h c (- F/2 if post_collision) into mom.
     cudaError_t (*state_moments)(const HostArgs &, int src, int post_collision, cudaStream_t);
     // FP64 block partial sums: mass (1 value) or force (2 values) per block.
