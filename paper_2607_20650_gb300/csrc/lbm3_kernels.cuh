@@ -195,7 +195,7 @@ template <class S, int L, bool OFF32>
 __device__ __forceinline__ void pull3(const Step3<S> &a, uint32_t x, uint32_t y, uint32_t z, uint32_t n,
                                       uint32_t lk, typename Codec<S>::C *g) {
     const uint32_t nx = (uint32_t)a.g.nx, ny = (uint32_t)a.g.ny, nz = (uint32_t)a.g.nz;
-    const S *__restrict__ src = a.src;
+    const S *src = a.src;
     const bool interior = (x - 1u < nx - 2u) && (y - 1u < ny - 2u) && (z - 1u < nz - 2u);
     if (OFF32) {
         // Node-index corrections of a pull that leaves the box through a
@@ -391,7 +391,7 @@ template <class S, int L>
 __device__ __forceinline__ void pull3_pair(const Step3<S> &a, uint32_t x, uint32_t y, uint32_t z, uint32_t n,
                                            uint32_t lka, uint32_t lkb, bool fa, bool fb, f2 *g) {
     const uint32_t nx = (uint32_t)a.g.nx, ny = (uint32_t)a.g.ny, nz = (uint32_t)a.g.nz;
-    const S *__restrict__ src = a.src;
+    const S *src = a.src;
     const int N = (int)a.N, nxy = (int)(nx * ny);
     const int xlo = x == 0 ? a.xlo_corr : 0, xhi = x + 1u == nx - 1 ? a.xhi_corr : 0;
     const int ylo = y == 0 ? nxy : 0, yhi = y == ny - 1 ? -nxy : 0;

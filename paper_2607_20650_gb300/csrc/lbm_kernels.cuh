@@ -96,26 +96,18 @@ __device__ __forceinline__ typename Codec<S>::C ldp(const S *base, uint32_t N, u
     return Codec<S>::dec(base[addr<L>(N, n, i)]);
 }
 
-#ifndef LBM_LDG_HINT
-#define LBM_LDG_HINT 0
-#endif
 #ifndef LBM_ST_HINT
 #define LBM_ST_HINT 0
 #endif
-// Loads of the read-only source lattice and stores of the destination
-// lattice of the two-lattice update. Stores default to plain stores, which
-// measured 1 % faster than evict-first (st.global.cs) for the bundle layout
-// at 32 registers; LBM_ST_HINT=1 makes every store evict-first, 2 only the
-// bundle layout's; LBM_LDG_HINT=1 loads through the read-only path (no
-// measured difference).
-template <class S>
-__device__ __forceinline__ S ld_src(const S *p) {
-#if LBM_LDG_HINT == 1
-    return __ldg(p);
-#else
-    return *p;
-#endif
-}
+// Loads of the source lattice are plain loads, never read-only (non-coherent)
+// ones, and its pointer is not __restrict__: in a chained launch the previous
+// update may still be writing it when this grid starts, and only a plain load
+// is sure to stay behind chain_wait(). (The read-only path made no difference
+// in time.)
+// Stores of the destination lattice of the two-lattice update default to plain
+// stores, which measured 1 % faster than evict-first (st.global.cs) for the
+// bundle layout at 32 registers; LBM_ST_HINT=1 makes every store evict-first, 2
+// only the bundle layout's.
 template <class S, int L>
 __device__ __forceinline__ void st_dst(S *p, S v) {
 #if LBM_ST_HINT == 1
@@ -251,13 +243,13 @@ __device__ __forceinline__ void pull_interior(const S *src, uint32_t n, uint32_t
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         if (i == 4) {
-            g[i] = Codec<S>::dec(ld_src(own + (ptrdiff_t)lay_base<L>(N, 4)));
+            g[i] = Codec<S>::dec(own[(ptrdiff_t)lay_base<L>(N, 4)]);
             continue;
         }
         const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own);
         const S *pp = row + ((ptrdiff_t)lay_base<L>(N, i) - (ptrdiff_t)lay_mul<L>() * cx(i));
         const S *pb = own + (ptrdiff_t)lay_base<L>(N, opp(i));
-        g[i] = Codec<S>::dec(ld_src(((lk >> link_bit(i)) & 1u) ? pb : pp));
+        g[i] = Codec<S>::dec(*(((lk >> link_bit(i)) & 1u) ? pb : pp));
     }
 }
 
@@ -282,8 +274,8 @@ __device__ __forceinline__ void two_lattice_fluid(const Step<S> &a, uint32_t x, 
                                                   uint32_t lk) {
     using C = typename Codec<S>::C;
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
-    S *__restrict__ dst = a.dst;
-    const S *__restrict__ src = a.src;
+    S *dst = a.dst;
+    const S *src = a.src;
     const bool interior = (x - 1u < nx - 2u) && (y - 1u < ny - 2u);
     C g[9];
     if (interior && a.off32) {
@@ -433,7 +425,7 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two
         const uint4 *g4 = reinterpret_cast<const uint4 *>(srcb + base);
         uint4 *s4 = reinterpret_cast<uint4 *>(wbuf + r * SP::ROW_BYTES);
 #pragma unroll
-        for (int k = lane; k < SP::CHUNKS; k += 32) s4[k] = __ldg(g4 + k);
+        for (int k = lane; k < SP::CHUNKS; k += 32) s4[k] = g4[k];
     }
     __syncwarp();
     C g[9];
