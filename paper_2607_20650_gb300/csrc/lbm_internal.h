@@ -15,10 +15,18 @@ struct alignas(64) TmaDesc {
 };
 
 // Launch of an update kernel (one that calls chain_wait before it touches what
-// updates write): its blocks may start before the previous kernel on the
-// stream has ended.
+// updates write). chained: its blocks may start before the previous kernel on
+// the stream has ended.
+// Small FP64 lattices are not chained: blocks placed beside the previous grid's
+// end up unevenly over the SMs, and where FP64 arithmetic is the bound the
+// fullest SM sets the time. Porous nodes, us an update, unchained / chained:
+// FP64 431 x 77 5.7 / 12.1, 512 x 300 17.7 / 21.1, 1024 x 512 48.6 / 48.3; FP32
+// 3.1 / 1.9, 3.8 / 2.6, 6.5 / 5.2.
+inline bool chained_updates(size_t elem, int64_t nodes) { return elem < 8 || nodes >= (int64_t)1 << 19; }
+
 template <class... P, class... A>
-inline cudaError_t launch_update(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...a) {
+inline cudaError_t launch_update(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t st, A &&...a) {
     cudaLaunchConfig_t c = {};
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -28,7 +36,7 @@ inline cudaError_t launch_update(void (*kernel)(P...), dim3 grid, dim3 block, si
     c.dynamicSmemBytes = smem;
     c.stream = st;
     c.attrs = at;
-    c.numAttrs = 1;
+    c.numAttrs = chained ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(a)...);
 }
 

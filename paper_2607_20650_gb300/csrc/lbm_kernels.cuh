@@ -1498,7 +1498,7 @@ cudaError_t op_batch_step(int kind, const void *recs, int ncases, const void *ti
     const auto *t = (const BatchTile *)tiles;
 #define LBM_BATCH_LAUNCH(S_, L_, A_)                                                       \
     if (kind == ((L_) < 0 ? -1 : (L_) * 4 + (A_)))                                        \
-        return launch_update(k_batch<S_, L_, A_>, dim3(grid), dim3(kBatchThreads), sm, st, c, t, ntiles, toff, pf);
+        return launch_update(sizeof(S) < 8, k_batch<S_, L_, A_>, dim3(grid), dim3(kBatchThreads), sm, st, c, t, ntiles, toff, pf);
     LBM_BATCH_KINDS(LBM_BATCH_LAUNCH, S)
 #undef LBM_BATCH_LAUNCH
     return cudaErrorInvalidValue;
@@ -1747,8 +1747,8 @@ bool pairs_ok(const HostArgs &h) {
 // Rows of a tile that one block of the per-node kernels (no exchange within a
 // tile) updates: a lattice of few tiles is cut into smaller blocks, so that
 // its nodes spread over all SMs. 256 x 64 nodes in 32 x 8 tiles are 64 blocks on
-// 152 SMs, and the FP64 lanes of 88 SMs are idle; in blocks of 32 x 1, chained, an
-// FP64 update takes 6.5 instead of 6.95 us.
+// 152 SMs, and the FP64 lanes of 88 SMs are idle; in blocks of 32 x 1 an FP64
+// update takes 3.9 instead of 6.6 us, an FP32 one (chained) 1.65 instead of 1.87.
 inline int rows_per_block(const HostArgs &h) {
     int ty = h.tile_y;
     int64_t blocks = (int64_t)h.ntx * h.nty;
@@ -1763,13 +1763,14 @@ template <class S, int L>
 cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStream_t st) {
     using C = typename Codec<S>::C;
     const dim3 tile(h.tile_x, h.tile_y), grid(h.ntx, h.nty);
+    const bool chain = chained_updates(sizeof(S), h.N);
     Step<S> a = a0;
     if (h.algo == LPTL) {
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h)) {
                 const int b = 128;
-                return launch_update(k_two_lattice_pair<S, L, true>, dim3((unsigned)((h.N / 2 + b - 1) / b)), dim3(b), 0,
-                                     st, a);
+                return launch_update(chain, k_two_lattice_pair<S, L, true>, dim3((unsigned)((h.N / 2 + b - 1) / b)),
+                                     dim3(b), 0, st, a);
             }
         }
         const int b = h.block_1d;
@@ -1778,29 +1779,30 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
             k_two_lattice<S, L, true, false><<<blocks, b, 0, st>>>(a);
             return cudaGetLastError();
         }
-        return launch_update(k_two_lattice<S, L, true>, blocks, dim3(b), 0, st, a);
+        return launch_update(chain, k_two_lattice<S, L, true>, blocks, dim3(b), 0, st, a);
     }
-    if (h.algo == NPOL) return launch_update(k_npol<S, L>, grid, tile, 0, st, a);
+    if (h.algo == NPOL) return launch_update(chain, k_npol<S, L>, grid, tile, 0, st, a);
     if (h.algo == NSOL) {
         const size_t sm = sizeof(C) * 9 * h.tile_x * h.tile_y;
         if constexpr (std::is_same<S, float>::value && L != COLLISION) {
-            if (h.tma) return launch_update(k_nsol_tma<S, L>, grid, tile, sm + 16, st, a, h.tmap);
+            if (h.tma) return launch_update(chain, k_nsol_tma<S, L>, grid, tile, sm + 16, st, a, h.tmap);
         }
-        return launch_update(k_nsol<S, L>, grid, tile, sm, st, a);
+        return launch_update(chain, k_nsol<S, L>, grid, tile, sm, st, a);
     }
     if (h.algo == NPTL) {
         if (L == COLLISION && h.tile_x % 32 == 0 && !(h.flags & 4u)) {
             const size_t sm = (size_t)AosSpan<S>::WARP_BYTES * ((h.tile_x * h.tile_y + 31) / 32);
-            return launch_update(k_two_lattice_aos<S>, grid, tile, sm, st, a);
+            return launch_update(chain, k_two_lattice_aos<S>, grid, tile, sm, st, a);
         }
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h) && !(h.tile_x & 1))
-                return launch_update(k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st, a);
+                return launch_update(chain, k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st,
+                                     a);
         }
         // Two nodes per thread on request (4- and 8-byte storage): one node
         // per thread at 32 registers keeps full occupancy and measured faster.
         if (sizeof(S) >= 4 && h.tile_y >= 2 && !(h.tile_y & 1) && (h.flags & 2u))
-            return launch_update(k_two_lattice2<S, L>, grid, dim3(h.tile_x, h.tile_y / 2), 0, st, a);
+            return launch_update(chain, k_two_lattice2<S, L>, grid, dim3(h.tile_x, h.tile_y / 2), 0, st, a);
     }
     if (h.algo == NPTL && h.N > kChainNodes) {
         k_two_lattice<S, L, false, false><<<grid, tile, 0, st>>>(a);
@@ -1808,9 +1810,10 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
     }
     a.ty = rows_per_block(h);
     const dim3 cut(h.tile_x, a.ty), cuts(h.ntx, (h.ny + a.ty - 1) / a.ty);
-    if (h.algo == NPTL) return launch_update(k_two_lattice<S, L, false>, cuts, cut, 0, st, a);
+    if (h.algo == NPTL) return launch_update(chain, k_two_lattice<S, L, false>, cuts, cut, 0, st, a);
     if (h.algo != AA) return cudaErrorInvalidValue;
-    return phase ? launch_update(k_aa<S, L, 1>, cuts, cut, 0, st, a) : launch_update(k_aa<S, L, 0>, cuts, cut, 0, st, a);
+    return phase ? launch_update(chain, k_aa<S, L, 1>, cuts, cut, 0, st, a)
+                 : launch_update(chain, k_aa<S, L, 0>, cuts, cut, 0, st, a);
 }
 
 template <class S>
