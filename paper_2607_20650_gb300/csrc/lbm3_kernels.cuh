@@ -683,8 +683,8 @@ struct Halo3 {
 // 8 x 8 x 8 tiles 58 % of the nodes lie on a face and every warp holds some,
 // so a separate path for them would run in every warp (as it did: 1,806 warp
 // instructions per 32 nodes, 383 us an update of 200 x 160 x 132 sphere-packing
-// nodes, FP32 stream layout; now 172 us). Bound by instruction issue and the
-// barrier, with two 512-thread blocks per SM.
+// nodes, FP32 stream layout; now 663 and 160 us). Bound by memory latency and
+// the barrier.
 template <class S, int L, bool OFF32>
 __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw, const int *b, const int *nt) {
     using C = typename Codec<S>::C;
@@ -756,8 +756,11 @@ __device__ __forceinline__ void npol3_tile(const Step3<S> &a, const S *hr, S *hw
     H.publish(hw, e);
 }
 
+// Three 512-thread blocks per SM (40 registers, a few spilled bytes): while one
+// waits at its barrier two load. 8 updates of the sphere packing above 1.366 ms
+// at two blocks (64 registers), 1.283 at three.
 template <class S, int L, bool OFF32>
-__global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 2) k3_npol(const Step3<S> a, const S *hr, S *hw) {
+__global__ void __launch_bounds__(512, sizeof(S) == 8 ? 1 : 3) k3_npol(const Step3<S> a, const S *hr, S *hw) {
     chain_next();
     const int b[3] = {(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z};
     const int nt[3] = {(int)gridDim.x, (int)gridDim.y, (int)gridDim.z};
