@@ -347,16 +347,9 @@ extern "C" lbm_status lbm3_read_moments(lbm3_lattice *L, double *rho, double *ux
     const int64_t N = L->pl.N;
     const char *mom = L->ws + L->pl.mom;
     double *dst[4] = {rho, ux, uy, uz};
-    if (L->pl.comp == 8) {
-        for (int k = 0; k < 4; ++k)
-            if (dst[k])
-                CK3(cudaMemcpyAsync(dst[k], (const double *)mom + (size_t)k * N, (size_t)N * 8, cudaMemcpyDeviceToHost,
-                                    L->stream));
-        CK3(cudaStreamSynchronize(L->stream));
-    } else {
-        const lbm_status s = lbm_widen_to_host((const float *)mom, N, 4, dst, L->stream);
-        if (s != LBM_OK) return s;
-    }
+    const lbm_status s = L->pl.comp == 8 ? lbm_fields_to_host((const double *)mom, N, 4, dst, L->stream)
+                                         : lbm_widen_to_host((const float *)mom, N, 4, dst, L->stream);
+    if (s != LBM_OK) return s;
     return lbm3_check(L);
 }
 

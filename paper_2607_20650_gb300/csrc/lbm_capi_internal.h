@@ -67,7 +67,8 @@ class HostView {
     void *dev_ = nullptr, *locked_ = nullptr;
 };
 
-// Up to four FP32 moments fields on the device to host doubles (lbm_capi.cu).
+// Up to four moments fields on the device, FP64 or FP32, to host doubles (lbm_capi.cu).
+lbm_status lbm_fields_to_host(const double *src, int64_t N, int fields, double *const *dst, cudaStream_t st);
 lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *const *dst, cudaStream_t st);
 
 lbm_status lbm_fail(lbm_status s, const char *fmt, ...);

@@ -111,3 +111,17 @@ def test_moments_around_the_thresholds(N):
     got = box.moments()
     for a, b in zip(got, (1 + ux, ux, uy, -ux)):
         assert np.abs(a - b).max() <= 2.0 ** -20   # FP32 sums of values below 1
+
+
+@pytest.mark.parametrize("N", [1, 1000, 32768, 32769, 43690, 43691])   # scratch: 2^20 bytes of three or four fields
+def test_fp64_moments_around_the_scratch_buffer(N):
+    r = np.random.default_rng(N)
+    ux, uy = 1e-2 * r.standard_normal((2, N))
+    lat = lbm.Lattice(N, 1, 0.8, storage="f64").init(1 + ux, ux, uy)
+    box = lbm.Lattice3(N, 1, 1, 0.8, storage="f64").init(1 + ux, ux, uy, -ux)
+    for got, want in ((lat.moments(), (1 + ux, ux, uy)), (box.moments(), (1 + ux, ux, uy, -ux))):
+        for a, b in zip(got, want):
+            assert np.abs(a.reshape(-1) - b).max() <= 2.0 ** -49   # FP64 sums of values below 2
+    only = np.empty(N)
+    assert lbm.load().lbm_read_moments(lat.h, None, only.ctypes.data, None) == 0
+    assert np.array_equal(only, lat.moments()[1].reshape(-1))
