@@ -324,7 +324,12 @@ template <class S, int L, int ALGO, bool OFF32>
 void batch_k(const Batch3Launch &b, cudaStream_t st) {
     const dim3 block = ALGO == LBM_LPTL ? dim3((unsigned)b.block_1d) : dim3(b.tx, b.ty, b.tz);
     const size_t sm = ALGO == LBM_NSOL ? nsol3_smem_bytes<S>(b.tx, b.ty, b.tz) : 0;
-    launch_update(sizeof(S) < 8, k3_batch<S, L, ALGO, OFF32>, dim3(b.nitems), block, sm, st, (const Case3<S> *)b.cases,
+    // Chained from ten blocks per SM on: with fewer, the next grid's blocks are
+    // placed unevenly over the SMs (as for small FP64 lattices). us an update,
+    // chained / not: 16 boxes of edge 12-20 (about 200 blocks) 6.9 / 4.9; 100 updates
+    // and the read-out of 48 of edge 12-48: 11.3 / 11.7 ms.
+    const bool chain = sizeof(S) < 8 && b.nitems >= 10 * 152;
+    launch_update(chain, k3_batch<S, L, ALGO, OFF32>, dim3(b.nitems), block, sm, st, (const Case3<S> *)b.cases,
                   (const uint2 *)b.items, b.src, b.toff, b.mom);
 }
 
