@@ -112,12 +112,13 @@ typedef enum {
                                                one node per thread) */
 #define LBM_FLAG_NO_STAGING 0x4u  /* NPTL, collision layout: no shared-memory staging of
                                      row spans (default when tile_x % 32 == 0) */
-#define LBM_FLAG_WIDE_OFFSETS 0x8u  /* D3Q19: 64-bit addressing for every pull, the path
-                                       lattices too large for 32-bit offset tables take */
-#define LBM_FLAG_NO_PREFETCH 0x10u  /* LPTL/NPTL/AA: no L2 prefetch of the records pulled
-                                       by the blocks launched next (default: on for 32-bit
-                                       storage in the stream and bundle layouts when a
-                                       lattice exceeds the L2 cache) */
+#define LBM_FLAG_WIDE_OFFSETS 0x8u  /* D3Q19, D2Q9 NPOL: 64-bit addressing for every pull,
+                                       the path lattices too large for 32-bit offsets take */
+#define LBM_FLAG_NO_PREFETCH 0x10u  /* LPTL/NPTL/NPOL/AA: no L2 prefetch of the records
+                                       pulled by the blocks launched next (default: on for
+                                       32-bit storage in the stream and bundle layouts,
+                                       NPOL in the bundle layout, when a lattice exceeds the
+                                       L2 cache) */
 #define LBM_FLAG_NO_PAIRS 0x20u  /* LPTL/NPTL, F16S/BF16S storage: one node per thread
                                     with scalar FP32 arithmetic (default when nx is even,
                                     the layout is bundle and tile_x is even: two
@@ -248,8 +249,8 @@ typedef struct lbm_info {
     int64_t cells, fluid_cells;
     int64_t steps;                 /* updates done since lbm_init */
     int32_t tile_x, tile_y;        /* tile used (LPTL: block size, 1) */
-    int32_t aux;                   /* lbm_get_info: L2 prefetch distance (LPTL: nodes, NPTL
-                                      and AA: rows; 0 = off); NSOL: 1 when tiles are staged
+    int32_t aux;                   /* lbm_get_info: L2 prefetch distance (LPTL: nodes, NPTL,
+                                      NPOL and AA: rows; 0 = off); NSOL: 1 when tiles are staged
                                       by tensor copies (LBM_FLAG_NO_TMA); lbm3_get_info: see
                                       there */
     double bytes_per_update;       /* algorithmic DRAM bytes of one update */

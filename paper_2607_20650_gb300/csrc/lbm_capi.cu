@@ -167,9 +167,9 @@ extern "C" lbm_status lbm_workspace_bytes(const lbm_params *p, size_t *bytes) {
     return LBM_OK;
 }
 
-// L2 prefetch distance of the two-lattice and AA kernels (LPTL: nodes, NPTL
-// and AA: rows), 0 = off. On for 32-bit storage in the stream and bundle
-// layouts when the lattice exceeds the L2 cache (the FP64 update is bound by
+// L2 prefetch distance of the two-lattice, AA and NPOL kernels (LPTL: nodes, the
+// others: rows), 0 = off. On for 32-bit storage in the stream and bundle
+// layouts (NPOL: bundle) when the lattice exceeds the L2 cache (the FP64 update is bound by
 // FP64 arithmetic, the 16-bit one by instruction issue). The distance is
 // 5/4 of the threads resident on the device: far enough that the prefetch
 // lands before the block that pulls it starts, near enough that it is still
@@ -191,8 +191,8 @@ static uint32_t prefetch_distance(const lbm_params *p, int64_t N, size_t elem, i
                        !(p->flags & LBM_FLAG_NO_PAIRS) && 9 * N < (int64_t(1) << 32) &&
                        (p->algo == LBM_LPTL || tile_x % 2 == 0);
     if (elem != 4 && !pairs) return 0;
-    if ((p->algo != LBM_LPTL && p->algo != LBM_NPTL && p->algo != LBM_AA) || p->layout == LBM_LAYOUT_COLLISION)
-        return 0;
+    if (p->algo == LBM_NSOL || p->layout == LBM_LAYOUT_COLLISION) return 0;
+    if (p->algo == LBM_NPOL && p->layout != LBM_LAYOUT_BUNDLE) return 0;
     int dev = 0, sms = 0, threads = 0, l2 = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -634,7 +634,7 @@ static float *host_scratch() {
 
 // The same for FP64 fields. Few values go through the thread's scratch buffer
 // in one copy, as above; a copy per field straight to the caller's fresh pages
-// took 53 instead of 38 us for the four fields of a box of 4,000 nodes.
+// took 53 instead of 35 us for the four fields of a box of 4,000 nodes.
 lbm_status lbm_fields_to_host(const double *src, int64_t N, int fields, double *const *dst, cudaStream_t st) {
     double *f = (size_t)fields * N * sizeof(double) <= kScratch * sizeof(float) ? (double *)host_scratch() : nullptr;
     if (f) CK(cudaMemcpyAsync(f, src, (size_t)fields * N * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -37,6 +37,7 @@ struct Step {
     int tx, ty, ntx, nty;
     uint64_t nx_magic;
     int off32;  // 9N < 2^32: element offsets fit 32 bits
+    int near32; // NPOL: and so do the buffer grid's, from the lattice's start
     int aos16;  // nx % 16 == 0: warp segments of 32 records start on 16-byte boundaries
     uint32_t pf;  // L2 prefetch distance of the two-lattice kernel: nodes (LPTL), rows (NPTL); 0 = off
     // 16-bit storage: k.r with every constant duplicated for the packed node pairs
@@ -85,6 +86,8 @@ Step<S> make_step(const HostArgs &h, const StepCall &c) {
     a.nty = h.nty;
     a.nx_magic = h.nx_magic;
     a.off32 = (9 * h.N) < (int64_t(1) << 32) ? 1 : 0;
+    // (flag 8: LBM_FLAG_WIDE_OFFSETS)
+    a.near32 = halo && !(h.flags & 8u) && halo + 2 * h.halo_parity_elems - a.dst < (int64_t(1) << 32) ? 1 : 0;
     a.aos16 = (h.nx % 16 == 0) ? 1 : 0;
     a.pf = h.pf;
     if constexpr (Codec<S>::narrow) a.k2 = duplicate(a.k.r);
@@ -915,48 +918,67 @@ struct HaloPull {
 // previous update), the block barrier separates all reads from the in-place
 // writes, and edge nodes publish their outgoing values for the next update.
 
-// Pulls of a node off the domain edge (9N < 2^32): every lane runs the same
-// code, the interior pull (neighbour value, or the own opposite value of a
-// bounced link) reading the source tile's publication of the previous update
-// where the source lies across a tile edge. In the bundle layout a row of the
-// buffer grid has the lattice's own format, so crossing the south or north
-// edge only changes the two row pointers (for whole warps, tile_x being a
-// multiple of 32).
-template <class S, int L>
-__device__ __forceinline__ void npol_pull(const Step<S> &a, const HaloPull<S> &H, uint32_t n, uint32_t lk,
-                                          typename Codec<S>::C *g) {
-    const uint32_t nx = (uint32_t)a.geo.nx;
-    const S *own = a.dst + lay_mul<L>() * n;
-    const S *rs = own + (ptrdiff_t)lay_mul<L>() * nx;  // row y+1: source of c_y = -1
-    const S *rn = own - (ptrdiff_t)lay_mul<L>() * nx;  // row y-1: source of c_y = +1
+// Pulls of a node off the domain edge: every lane runs the same code, the
+// interior pull (neighbour value, or the own opposite value of a bounced link)
+// reading the source tile's publication of the previous update where the source
+// lies across a tile edge. In the bundle layout a row of the buffer grid has the
+// lattice's own format, so crossing the south or north edge only changes the
+// two rows (for whole warps, tile_x being a multiple of 32).
+// Lattice and buffer grid lie in one workspace, and I is an element's index from
+// the lattice's start: 32 bits where that reaches the grid's end (Step::near32),
+// so that choosing a source is one select, 64 otherwise. 6000 x 3001 porous nodes,
+// us an update, pointers before / 32-bit indices: FP32 stream 32 x 8 242 / 233,
+// collision 64 x 4 294 / 277, bundle 64 x 4 230 / 226 (220 with the prefetch
+// below), FP16 bundle 64 x 4 229 / 190. (A select avoided by issuing the pulled
+// and the bounced load, each under its own predicate, costs 9 %.)
+template <class S, int L, class I>
+__device__ __forceinline__ void npol_pull(const Step<S> &a, int bx, int by, int x, int y, int x0, int x1, int y0,
+                                          int y1, uint32_t n, uint32_t lk, typename Codec<S>::C *g) {
+    constexpr I m = lay_mul<L>();
+    // direction i from the lattice's start
+    auto base = [N = (I)a.N](int i) -> I {
+        return L == STREAM ? (I)i * N : (L == BUNDLE ? (I)(i / 3) * 3 * N + (I)(i % 3) : (I)i);
+    };
+    const I nx = (I)a.geo.nx, ny = (I)a.geo.ny;
+    const I ncol = (I)a.ntx * ny, nrow = (I)a.nty * nx, grid = (I)(a.halo_rd - a.dst);
+    const I w = grid + 3 * ((I)(bx - 1) * ny + (I)y);                     // east edges of the column before
+    const I e = grid + 3 * (ncol + (I)(bx + 1) * ny + (I)y);              // west edges of the column after
+    const I s = grid + 6 * ncol + 3 * ((I)(by - 1) * nx + (I)x);          // rows alike
+    const I t = grid + 6 * ncol + 3 * (nrow + (I)(by + 1) * nx + (I)x);
+    const bool xl = x == x0, xh = x == x1, yl = y == y0, yh = y == y1;
+    const I own = m * (I)n;
+    I rs = own + m * nx, rn = own - m * nx;   // rows y + 1 and y - 1: sources of c_y = -1 and +1
     if (L == BUNDLE) {
-        rn += (ptrdiff_t)lay_base<L>(a.N, 6);
-        if (H.y1) rs = H.n;
-        if (H.y0) rn = H.s;
+        rn += base(6);
+        if (yh) rs = t;
+        if (yl) rn = s;
     }
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         if (i == 4) {
-            g[i] = Codec<S>::dec(own[(ptrdiff_t)lay_base<L>(a.N, 4)]);
+            g[i] = Codec<S>::dec(a.dst[own + base(4)]);
             continue;
         }
-        const bool bounce = (lk >> link_bit(i)) & 1u;
-        const S *p;
+        const bool cross_y = cy(i) > 0 ? yl : (cy(i) < 0 ? yh : false);
+        I p;
         if (L == BUNDLE) {
-            const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own + (ptrdiff_t)lay_base<L>(a.N, 3));
-            p = row + (i % 3 - 3 * cx(i));
+            p = (cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own + base(3))) + (I)(i % 3 - 3 * cx(i));
         } else {
-            const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own);
-            p = row + ((ptrdiff_t)lay_base<L>(a.N, i) - (ptrdiff_t)lay_mul<L>() * cx(i));
-            if (cy(i) != 0 && H.crosses_y(i)) p = H.at_y(i);
+            p = (cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own)) + (base(i) - m * (I)cx(i));
+            if (cross_y) p = (cy(i) > 0 ? s : t) + (I)(i % 3 - 3 * cx(i));
         }
-        if (cx(i) != 0 && H.crosses_x(i)) p = H.at_x(i);
-        if (bounce) p = own + (ptrdiff_t)lay_base<L>(a.N, opp(i));
-        g[i] = Codec<S>::dec(*p);
+        if ((cx(i) > 0 ? xl : (cx(i) < 0 ? xh : false)) && !cross_y)
+            p = (cx(i) > 0 ? w : e) + (I)(i / 3 - 3 * cy(i));
+        if ((lk >> link_bit(i)) & 1u) p = own + base(opp(i));
+        g[i] = Codec<S>::dec(a.dst[p]);
     }
 }
 
-template <class S, int L>
+// PF: L2 prefetch of the record a.pf rows ahead, as in the two-lattice kernel.
+// FP32 in the bundle layout: 3 % (in the stream layout, nine addresses a node, 2 %,
+// left out); a kernel of its own, as the test for it costs a lattice that fits
+// the L2 cache 5 %.
+template <class S, int L, bool PF = false>
 __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int lx, int ly, int lane) {
     using C = typename Codec<S>::C;
     const int nx = a.geo.nx, ny = a.geo.ny;
@@ -970,6 +992,9 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
         n = (uint32_t)y * (uint32_t)nx + (uint32_t)x;
         lk = a.links[n];
     }
+    const bool ahead = PF && valid && (uint32_t)(ny - y) > a.pf;
+    const uint32_t np = n + a.pf * (uint32_t)nx;
+    const uint32_t lkp = ahead ? (uint32_t)a.links[np] : SOLID_LINKS;
     chain_wait();
     const bool fluid = lk != SOLID_LINKS;
     const unsigned F = __ballot_sync(__activemask(), fluid);
@@ -977,10 +1002,11 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
     const bool zero_fill = false;   // measured: NPOL is 5 % faster without the sector zero fill
     const bool inner = x > x0 && x < x1 && y > y0 && y < y1;
     const bool dom_inner = x > 0 && x < nx - 1 && y > 0 && y < ny - 1;
-    const HaloPull<S> H(a, bx, by, x, y, x0, x1, y0, y1);
     C g[9];
-    if (fluid && dom_inner && a.off32) {
-        npol_pull<S, L>(a, H, n, lk, g);
+    if (fluid && dom_inner && a.near32) {
+        npol_pull<S, L, uint32_t>(a, bx, by, x, y, x0, x1, y0, y1, n, lk, g);
+    } else if (fluid && dom_inner) {
+        npol_pull<S, L, int64_t>(a, bx, by, x, y, x0, x1, y0, y1, n, lk, g);
     } else if (fluid) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
@@ -988,14 +1014,6 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
                 g[i] = ldp<S, L>(lat, a.N, n, 4);
             } else if ((lk >> link_bit(i)) & 1u) {
                 g[i] = ldp<S, L>(lat, a.N, n, opp(i));
-            } else if (inner) {
-                g[i] = ldp<S, L>(lat, a.N, n - (uint32_t)(cy(i) * nx + cx(i)), i);
-            } else if (dom_inner) {
-                // Tile edge inside the domain: the source is in this tile or
-                // published in the buffer grid.
-                g[i] = H.crosses_y(i)   ? Codec<S>::dec(*H.at_y(i))
-                       : H.crosses_x(i) ? Codec<S>::dec(*H.at_x(i))
-                                        : ldp<S, L>(lat, a.N, n - (uint32_t)(cy(i) * nx + cx(i)), i);
             } else {
                 int xs, ys, j;
                 if (map_pull(a.geo, x, y, i, xs, ys, j) != PULL_NODE)
@@ -1008,6 +1026,7 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
         }
     }
     const C dnb = (fluid && x == 0 && a.geo.bw == INLET_EQ_NEUMANN) ? neighbour_drho<S, L>(a, lat, n, 0) : C(0);
+    if (PF && lkp != SOLID_LINKS) prefetch_record<S, L>(lat, a.N, np);
     __syncthreads();
     if (fluid) {
         S e[9];
@@ -1020,16 +1039,17 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
 }
 
 // Registers: 32 (four 512-thread blocks, spills) for the stream layout and
-// 16-bit storage, 40 (three) where it measured faster: 6000 x 3001 nodes, 16
-// updates, 32 / 40 registers: FP32 bundle 64 x 4 3.89 / 3.90 ms and 128 x 4
-// 4.35 / 4.09, collision 5.41 / 4.88, stream 32 x 8 4.11 / 4.29, FP16 3.85 / 3.95.
-template <class S, int L>
+// 16-bit storage, 40 (three) where it measured faster: 6000 x 3001 nodes, us an
+// update, 32 / 40 registers: stream 32 x 8 233 / 251; with the pulls by pointers
+// FP32 bundle 64 x 4 243 / 244 and 128 x 4 272 / 256, collision 338 / 305, FP16
+// 241 / 247.
+template <class S, int L, bool PF>
 __global__ void __launch_bounds__(kMaxTileThreads,
                                   sizeof(S) == 8 ? 1 : (sizeof(S) == 4 && L != STREAM) || L == COLLISION ? 3 : 4)
     k_npol(const Step<S> a) {
     chain_next();
-    npol_tile<S, L>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
-                    (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
+    npol_tile<S, L, PF>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
+                        (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
 }
 
 // TMA: the tile's populations arrive by one tensor copy (FP32 storage, stream
@@ -1781,7 +1801,11 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         }
         return launch_update(chain, k_two_lattice<S, L, true>, blocks, dim3(b), 0, st, a);
     }
-    if (h.algo == NPOL) return launch_update(chain, k_npol<S, L>, grid, tile, 0, st, a);
+    if (h.algo == NPOL) {
+        if constexpr (sizeof(S) == 4 && L == BUNDLE)
+            if (h.pf) return launch_update(chain, k_npol<S, L, true>, grid, tile, 0, st, a);
+        return launch_update(chain, k_npol<S, L, false>, grid, tile, 0, st, a);
+    }
     if (h.algo == NSOL) {
         const size_t sm = sizeof(C) * 9 * h.tile_x * h.tile_y;
         if constexpr (std::is_same<S, float>::value && L != COLLISION) {
