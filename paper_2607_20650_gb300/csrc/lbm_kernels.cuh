@@ -233,27 +233,46 @@ __device__ __forceinline__ void store_zero(S *dst, uint32_t N, uint32_t n, int o
     }
 }
 
-// Pulls of an interior node (requires 9N < 2^32): pointers to the node's
-// own record and to the rows above and below, plus per-direction constant
-// offsets (immediates for the bundle and collision layouts); each pull picks
-// the pulled neighbour or, for a bounced link, the node's opposite slot.
-template <class S, int L>
+// Pulls of an interior node (requires 9N < 2^32); each picks the pulled
+// neighbour or, for a bounced link, the node's opposite slot. IDX: by 32-bit
+// indices, one select a pull, else by pointers with constant offsets. us an update
+// of FP32 lattices, pointers / indices: 2048 x 512 stream 9.63 / 9.22, bundle
+// 9.81 / 9.97 (porous 9.31 / 9.10), 16384 x 8192 porous bundle 1192 / 1186.
+template <class S, int L, bool IDX>
 __device__ __forceinline__ void pull_interior(const S *src, uint32_t n, uint32_t nx, uint32_t N, uint32_t lk,
                                               typename Codec<S>::C *g) {
-    const S *own = src + lay_mul<L>() * n;
-    const S *rs = own + (ptrdiff_t)lay_mul<L>() * nx;  // row y+1: source of c_y = -1
-    const S *rn = own - (ptrdiff_t)lay_mul<L>() * nx;  // row y-1: source of c_y = +1
+    constexpr uint32_t m = lay_mul<L>();
+    if constexpr (IDX) {
+        const uint32_t own = m * n;
+        const uint32_t row[3] = {own + m * nx, own, own - m * nx};   // of c_y = -1, 0, +1
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        if (i == 4) {
-            g[i] = Codec<S>::dec(own[(ptrdiff_t)lay_base<L>(N, 4)]);
-            continue;
+        for (int i = 0; i < 9; ++i) {
+            uint32_t p = row[cy(i) + 1] + (lay_base<L>(N, i) - m * (uint32_t)cx(i));
+            if (i != 4 && ((lk >> link_bit(i)) & 1u)) p = own + lay_base<L>(N, opp(i));
+            g[i] = Codec<S>::dec(src[p]);
         }
-        const S *row = cy(i) < 0 ? rs : (cy(i) > 0 ? rn : own);
-        const S *pp = row + ((ptrdiff_t)lay_base<L>(N, i) - (ptrdiff_t)lay_mul<L>() * cx(i));
-        const S *pb = own + (ptrdiff_t)lay_base<L>(N, opp(i));
-        g[i] = Codec<S>::dec(*(((lk >> link_bit(i)) & 1u) ? pb : pp));
+    } else {
+        const S *own = src + m * n;
+        const S *row[3] = {own + (ptrdiff_t)m * nx, own, own - (ptrdiff_t)m * nx};
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const S *p = row[cy(i) + 1] + ((ptrdiff_t)lay_base<L>(N, i) - (ptrdiff_t)m * cx(i));
+            if (i != 4 && ((lk >> link_bit(i)) & 1u)) p = own + (ptrdiff_t)lay_base<L>(N, opp(i));
+            g[i] = Codec<S>::dec(*p);
+        }
     }
+}
+
+// The same for warps without a bounced link.
+template <class S, int L>
+__device__ __forceinline__ void pull_inner(const S *src, uint32_t n, uint32_t nx, uint32_t N,
+                                           typename Codec<S>::C *g) {
+    constexpr uint32_t m = lay_mul<L>();
+    const S *own = src + m * n;
+    const S *row[3] = {own + (ptrdiff_t)m * nx, own, own - (ptrdiff_t)m * nx};
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+        g[i] = Codec<S>::dec(row[cy(i) + 1][(ptrdiff_t)lay_base<L>(N, i) - (ptrdiff_t)m * cx(i)]);
 }
 
 template <class S, int L>
@@ -302,12 +321,13 @@ __device__ __forceinline__ void pull_edge(const Step<S> &a, uint32_t x, uint32_t
 }
 
 // Pull, collide and store one fluid node of the two-lattice update. Interior
-// nodes take a path with 32-bit element offsets where each pull is one select
-// between two uniform offsets (pulled neighbour or own opposite slot). EDGES:
-// warps that hold a node on the domain edge take pull_edge for all their
+// nodes take a path with 32-bit element offsets. EDGES: warps that hold a node on the domain edge take pull_edge for all their
 // lanes; without it (large lattices, where such warps are rare and the vote
 // costs 0.3 %) and beyond 32-bit offsets, edge nodes take the general mapping.
-template <class S, int L, bool EDGES = true>
+// BATCH (arguments in shared memory): warps of inner nodes without a bounced link
+// choose no source at all. 48 channels, us an update: FP32 124.3 -> 120.6, FP16
+// 125.3 -> 115.4; single lattices gained nothing by it.
+template <class S, int L, bool EDGES = true, bool BATCH = false>
 __device__ __forceinline__ void two_lattice_fluid(const Step<S> &a, uint32_t x, uint32_t y, uint32_t n,
                                                   uint32_t lk) {
     using C = typename Codec<S>::C;
@@ -316,8 +336,10 @@ __device__ __forceinline__ void two_lattice_fluid(const Step<S> &a, uint32_t x, 
     const S *src = a.src;
     const bool interior = (x - 1u < nx - 2u) && (y - 1u < ny - 2u);
     C g[9];
-    if (a.off32 && (EDGES ? __all_sync(__activemask(), interior) != 0 : interior)) {
-        pull_interior<S, L>(src, n, nx, a.N, lk, g);
+    if (BATCH && a.off32 && __all_sync(__activemask(), interior && lk == 0u)) {
+        pull_inner<S, L>(src, n, nx, a.N, g);
+    } else if (a.off32 && (EDGES ? __all_sync(__activemask(), interior) != 0 : interior)) {
+        pull_interior<S, L, BATCH || L == STREAM || (L == BUNDLE && !EDGES)>(src, n, nx, a.N, lk, g);
     } else {
         if (EDGES && a.off32) {
             pull_edge<S, L>(a, x, y, n, lk, g);
@@ -351,11 +373,9 @@ __device__ __forceinline__ void two_lattice_fluid(const Step<S> &a, uint32_t x, 
 
 // One node of the two-lattice pull update (LPTL and NPTL). lane: the
 // thread's lane (the zero fill below votes over the warp).
-template <class S, int L, bool CHAIN = true>
-__device__ __forceinline__ void two_lattice_node(const Step<S> &a, uint32_t x, uint32_t y, int lane) {
-    const uint32_t n = y * (uint32_t)a.geo.nx + x;
-    const uint32_t lk = a.links[n];
-    if (CHAIN) chain_wait();
+template <class S, int L, bool CHAIN, bool BATCH>
+__device__ __forceinline__ void two_lattice_known(const Step<S> &a, uint32_t x, uint32_t y, uint32_t n, uint32_t lk,
+                                                  int lane) {
     const bool fluid = lk != SOLID_LINKS;
     const unsigned F = __ballot_sync(__activemask(), fluid);
     if (!fluid) {
@@ -365,7 +385,14 @@ __device__ __forceinline__ void two_lattice_node(const Step<S> &a, uint32_t x, u
         if (shares_sector<S, L>(F, lane)) store_zero<S, L>(a.dst, a.N, n, a.off32);
         return;
     }
-    two_lattice_fluid<S, L, CHAIN>(a, x, y, n, lk);
+    two_lattice_fluid<S, L, CHAIN, BATCH>(a, x, y, n, lk);
+}
+template <class S, int L, bool CHAIN = true, bool BATCH = false>
+__device__ __forceinline__ void two_lattice_node(const Step<S> &a, uint32_t x, uint32_t y, int lane) {
+    const uint32_t n = y * (uint32_t)a.geo.nx + x;
+    const uint32_t lk = a.links[n];
+    if (CHAIN) chain_wait();
+    two_lattice_known<S, L, CHAIN, BATCH>(a, x, y, n, lk, lane);
 }
 
 // NPTL with two nodes per thread, rows y and y + ty/2 of a tx x ty tile:
@@ -393,8 +420,8 @@ __global__ void __launch_bounds__(kMaxTileThreads) k_two_lattice2(const Step<S> 
     const bool fast_a = fa && a.off32 && (x - 1u < nx - 2u) && (ya - 1u < ny - 2u);
     const bool fast_b = fb && a.off32 && (x - 1u < nx - 2u) && (yb - 1u < ny - 2u);
     C ga[9], gb[9];
-    if (fast_a) pull_interior<S, L>(a.src, na, nx, a.N, lka, ga);
-    if (fast_b) pull_interior<S, L>(a.src, nb, nx, a.N, lkb, gb);
+    if (fast_a) pull_interior<S, L, false>(a.src, na, nx, a.N, lka, ga);
+    if (fast_b) pull_interior<S, L, false>(a.src, nb, nx, a.N, lkb, gb);
     S e[9];
     if (fast_a) {
         collide_encode<S, false>(a, x, na, ga, e);
@@ -1403,15 +1430,24 @@ __device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uin
     const int lane = tid & 31;
     const bool ahead = sizeof(S) == 4 && L != COLLISION && pf != 0;
     if (algo == LPTL) {
+        // each tile's link bytes are loaded one tile ahead (256 channels 74.3 ->
+        // 77.7 GLUPS, 71.8 before the pulls above)
+        constexpr uint32_t T = kBatchThreads;
+        uint32_t n = t * kBatchSuper * T + (uint32_t)tid;
+        bool in = n < a.N;
+        uint32_t lk = in ? (uint32_t)a.links[n] : SOLID_LINKS;
+        chain_wait();
 #pragma unroll 1
-        for (int k = 0; k < kBatchSuper; ++k) {
-            const uint32_t n = (t * kBatchSuper + k) * (uint32_t)kBatchThreads + (uint32_t)tid;
-            if (n < a.N) {
-                if (ahead && k + 1 < kBatchSuper && a.N - n > (uint32_t)kBatchThreads)
-                    prefetch_record<S, L>(a.src, a.N, n + (uint32_t)kBatchThreads);
+        for (int k = 0; k < kBatchSuper; ++k, n += T) {
+            const bool more = k + 1 < kBatchSuper && in && a.N - n > T;
+            const uint32_t lkn = more ? (uint32_t)a.links[n + T] : SOLID_LINKS;
+            if (in) {
+                if (ahead && more) prefetch_record<S, L>(a.src, a.N, n + T);
                 const uint32_t y = a.nx_magic ? (uint32_t)__umul64hi((unsigned long long)n, a.nx_magic) : n;
-                two_lattice_node<S, L>(a, n - y * (uint32_t)a.geo.nx, y, lane);
+                two_lattice_known<S, L, true, true>(a, n - y * (uint32_t)a.geo.nx, y, n, lk, lane);
             }
+            in = more;
+            lk = lkn;
             if (k == 0) stage();
         }
         return;
@@ -1428,7 +1464,7 @@ __device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uin
                 const int x = (int)bx * a.tx + lx, y = (int)by * a.ty + ly;
                 if (ahead && k + 1 < kBatchSuper && ly < a.ty && y < a.geo.ny && x + a.tx < a.geo.nx)
                     prefetch_record<S, L>(a.src, a.N, (uint32_t)y * (uint32_t)a.geo.nx + (uint32_t)(x + a.tx));
-                if (ly < a.ty && x < a.geo.nx && y < a.geo.ny) two_lattice_node<S, L>(a, x, y, lane);
+                if (ly < a.ty && x < a.geo.nx && y < a.geo.ny) two_lattice_node<S, L, true, true>(a, x, y, lane);
             }
             if (k == 0) stage();
         }
