@@ -95,8 +95,8 @@ bool pairs3_ok(const lbm3_lattice *L) {
 }
 
 template <class S>
-bool chained3(const lbm3_lattice *L) {
-    return chained_updates(sizeof(S), L->pl.N);
+bool chained3(const lbm3_lattice *L, dim3 grid, dim3 block) {
+    return chained_updates(sizeof(S), L->pl.N) && spread_evenly(grid, block);
 }
 
 template <class S, bool LINEAR>
@@ -109,25 +109,28 @@ void launch_pair3(const lbm3_lattice *L, const Step3<S> &a, cudaStream_t st) {
         b = dim3(L->pl.tx / 2, L->pl.ty, L->pl.tz);
         g = dim3(L->pl.ntx, L->pl.nty, L->pl.ntz);
     }
-    if (L->p.layout == LBM_LAYOUT_STREAM) launch_update(chained3<S>(L), k3_step_pair<S, STREAM, LINEAR>, g, b, 0, st, a);
-    else launch_update(chained3<S>(L), k3_step_pair<S, BUNDLE, LINEAR>, g, b, 0, st, a);
+    const bool chain = chained3<S>(L, g, b);
+    if (L->p.layout == LBM_LAYOUT_STREAM) launch_update(chain, k3_step_pair<S, STREAM, LINEAR>, g, b, 0, st, a);
+    else launch_update(chain, k3_step_pair<S, BUNDLE, LINEAR>, g, b, 0, st, a);
 }
 
 template <class S, bool LINEAR, bool OFF32>
 void launch3k(const lbm3_lattice *L, const Step3<S> &a, dim3 grid, dim3 block, cudaStream_t st) {
     const int lay = L->p.layout;
-    if (lay == LBM_LAYOUT_STREAM) launch_update(chained3<S>(L), k3_step<S, STREAM, LINEAR, OFF32>, grid, block, 0, st, a);
-    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chained3<S>(L), k3_step<S, BUNDLE, LINEAR, OFF32>, grid, block, 0, st, a);
-    else launch_update(chained3<S>(L), k3_step<S, COLLISION, LINEAR, OFF32>, grid, block, 0, st, a);
+    const bool chain = chained3<S>(L, grid, block);
+    if (lay == LBM_LAYOUT_STREAM) launch_update(chain, k3_step<S, STREAM, LINEAR, OFF32>, grid, block, 0, st, a);
+    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chain, k3_step<S, BUNDLE, LINEAR, OFF32>, grid, block, 0, st, a);
+    else launch_update(chain, k3_step<S, COLLISION, LINEAR, OFF32>, grid, block, 0, st, a);
 }
 
 template <class S, int PHASE>
 void launch_aa(const lbm3_lattice *L, const Step3<S> &a, cudaStream_t st) {
     const dim3 g(L->pl.ntx, L->pl.nty, L->pl.ntz), b(L->pl.tx, L->pl.ty, L->pl.tz);
     const int lay = L->p.layout;
-    if (lay == LBM_LAYOUT_STREAM) launch_update(chained3<S>(L), k3_aa<S, STREAM, PHASE>, g, b, 0, st, a);
-    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chained3<S>(L), k3_aa<S, BUNDLE, PHASE>, g, b, 0, st, a);
-    else launch_update(chained3<S>(L), k3_aa<S, COLLISION, PHASE>, g, b, 0, st, a);
+    const bool chain = chained3<S>(L, g, b);
+    if (lay == LBM_LAYOUT_STREAM) launch_update(chain, k3_aa<S, STREAM, PHASE>, g, b, 0, st, a);
+    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chain, k3_aa<S, BUNDLE, PHASE>, g, b, 0, st, a);
+    else launch_update(chain, k3_aa<S, COLLISION, PHASE>, g, b, 0, st, a);
 }
 
 template <class S>
@@ -141,9 +144,10 @@ void launch_npol(const lbm3_lattice *L, const Step3<S> &a, int parity, cudaStrea
     const S *hr = halo_parity<S>(L, parity);
     S *hw = halo_parity<S>(L, parity ^ 1);
     const int lay = L->p.layout;
-    if (lay == LBM_LAYOUT_STREAM) launch_update(chained3<S>(L), k3_npol<S, STREAM, OFF32>, g, b, 0, st, a, hr, hw);
-    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chained3<S>(L), k3_npol<S, BUNDLE, OFF32>, g, b, 0, st, a, hr, hw);
-    else launch_update(chained3<S>(L), k3_npol<S, COLLISION, OFF32>, g, b, 0, st, a, hr, hw);
+    const bool chain = chained3<S>(L, g, b);
+    if (lay == LBM_LAYOUT_STREAM) launch_update(chain, k3_npol<S, STREAM, OFF32>, g, b, 0, st, a, hr, hw);
+    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chain, k3_npol<S, BUNDLE, OFF32>, g, b, 0, st, a, hr, hw);
+    else launch_update(chain, k3_npol<S, COLLISION, OFF32>, g, b, 0, st, a, hr, hw);
 }
 
 template <class S>
@@ -153,9 +157,10 @@ void launch_nsol(const lbm3_lattice *L, const Step3<S> &a, int parity, cudaStrea
     const S *hr = halo_parity<S>(L, parity);
     S *hw = halo_parity<S>(L, parity ^ 1);
     const int lay = L->p.layout;
-    if (lay == LBM_LAYOUT_STREAM) launch_update(chained3<S>(L), k3_nsol<S, STREAM>, g, b, sm, st, a, hr, hw);
-    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chained3<S>(L), k3_nsol<S, BUNDLE>, g, b, sm, st, a, hr, hw);
-    else launch_update(chained3<S>(L), k3_nsol<S, COLLISION>, g, b, sm, st, a, hr, hw);
+    const bool chain = chained3<S>(L, g, b);
+    if (lay == LBM_LAYOUT_STREAM) launch_update(chain, k3_nsol<S, STREAM>, g, b, sm, st, a, hr, hw);
+    else if (lay == LBM_LAYOUT_BUNDLE) launch_update(chain, k3_nsol<S, BUNDLE>, g, b, sm, st, a, hr, hw);
+    else launch_update(chain, k3_nsol<S, COLLISION>, g, b, sm, st, a, hr, hw);
 }
 
 // Largest staged tile of the 3-D NSOL kernels (512 nodes) beyond the default
@@ -324,11 +329,9 @@ template <class S, int L, int ALGO, bool OFF32>
 void batch_k(const Batch3Launch &b, cudaStream_t st) {
     const dim3 block = ALGO == LBM_LPTL ? dim3((unsigned)b.block_1d) : dim3(b.tx, b.ty, b.tz);
     const size_t sm = ALGO == LBM_NSOL ? nsol3_smem_bytes<S>(b.tx, b.ty, b.tz) : 0;
-    // Chained from ten blocks per SM on: with fewer, the next grid's blocks are
-    // placed unevenly over the SMs (as for small FP64 lattices). us an update,
-    // chained / not: 16 boxes of edge 12-20 (about 200 blocks) 6.9 / 4.9; 100 updates
-    // and the read-out of 48 of edge 12-48: 11.3 / 11.7 ms.
-    const bool chain = sizeof(S) < 8 && b.nitems >= 10 * 152;
+    // (100 updates and the read-out of 48 boxes of edge 12-48: 11.3 ms chained, 11.7
+    // not; 16 of edge 12-20, 200 blocks, 6.9 and 4.9 us an update)
+    const bool chain = sizeof(S) < 8 && spread_evenly(dim3(b.nitems), block);
     launch_update(chain, k3_batch<S, L, ALGO, OFF32>, dim3(b.nitems), block, sm, st, (const Case3<S> *)b.cases,
                   (const uint2 *)b.items, b.src, b.toff, b.mom);
 }

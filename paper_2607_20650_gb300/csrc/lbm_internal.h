@@ -23,6 +23,16 @@ struct alignas(64) TmaDesc {
 // FP64 431 x 77 5.7 / 12.1, 512 x 300 17.7 / 21.1, 1024 x 512 48.6 / 48.3; FP32
 // 3.1 / 1.9, 3.8 / 2.6, 6.5 / 5.2.
 inline bool chained_updates(size_t elem, int64_t nodes) { return elem < 8 || nodes >= (int64_t)1 << 19; }
+// Nor are kernels with blocks of a tile's size, or of one node a thread in three
+// dimensions, while their blocks neither fill the SMs (152 of 1,536 threads) nor
+// leave most of them empty, for the same reason. D3Q19 FP32, us an update,
+// unchained / chained: NPOL 8 x 8 x 8, 30 x 28 x 33 nodes (80 blocks) 4.7 / 8.1, 48 x
+// 40 x 44 (180) 5.4 / 8.4, 64 x 64 x 64 (512) 11.1 / 10.7; LPTL (256 nodes a block)
+// 4.0 / 4.9, 5.9 / 6.5 and 8.9 / 8.4; 12 x 12 x 12 (7 blocks) 3.7 / 3.2.
+inline bool spread_evenly(dim3 grid, dim3 block) {
+    const int64_t blocks = (int64_t)grid.x * grid.y * grid.z;
+    return blocks * block.x * block.y * block.z >= 152 * 1536 || blocks <= 152 / 4;
+}
 
 template <class... P, class... A>
 inline cudaError_t launch_update(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,

@@ -451,7 +451,7 @@ struct AosSpan {
     static constexpr int WARP_BYTES = 3 * ROW_BYTES;
 };
 
-template <class S>
+template <class S, bool CHAIN = true>
 __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two_lattice_aos(const Step<S> a) {
     using C = typename Codec<S>::C;
     using SP = AosSpan<S>;
@@ -461,11 +461,11 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two
     const int lane = tid & 31, warp = tid >> 5;
     const uint32_t x = blockIdx.x * a.tx + threadIdx.x;
     const uint32_t y = blockIdx.y * a.ty + threadIdx.y;
-    chain_next();
+    if (CHAIN) chain_next();
     if (x >= nx || y >= ny) return;
     const uint32_t n = y * nx + x;
     const uint32_t lk = a.links[n];
-    chain_wait();
+    if (CHAIN) chain_wait();
     const bool fluid = lk != SOLID_LINKS;
     const unsigned act = __activemask();
     const unsigned F = __ballot_sync(act, fluid);
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two
             if (shares_sector<S, COLLISION>(F, lane)) store_zero<S, COLLISION>(a.dst, a.N, n, a.off32);
             return;
         }
-        two_lattice_fluid<S, COLLISION>(a, x, y, n, lk);
+        two_lattice_fluid<S, COLLISION, CHAIN>(a, x, y, n, lk);
         return;
     }
     unsigned char *wbuf = smem_aos + (size_t)warp * SP::WARP_BYTES;
@@ -1234,14 +1234,14 @@ __global__ void __launch_bounds__(kMaxTileThreads, LBM_NSOL_MINB)
 // Each slot is read and written by the same node within a phase, so no
 // synchronisation is needed. Zero-gradient outflow reads one slot from two
 // nodes and is not supported here.
-template <class S, int L, int PHASE>
+template <class S, int L, int PHASE, bool CHAIN>
 __device__ __forceinline__ void aa_node(const Step<S> &a, uint32_t x, uint32_t y, int lane) {
     constexpr int phase = PHASE;
     using C = typename Codec<S>::C;
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     const uint32_t n = y * nx + x;
     const uint32_t lk = a.links[n];
-    chain_wait();
+    if (CHAIN) chain_wait();
     S *lat = a.dst;
     const bool fluid = lk != SOLID_LINKS;
     const unsigned F = __ballot_sync(__activemask(), fluid);
@@ -1376,9 +1376,11 @@ __device__ __forceinline__ void aa_node(const Step<S> &a, uint32_t x, uint32_t y
     }
 }
 
-template <class S, int L, int PHASE>
+// CHAIN: as for k_two_lattice (134M nodes, bundle 64 x 2: 1.158 ms an update with
+// the wait).
+template <class S, int L, int PHASE, bool CHAIN = true>
 __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : (PHASE == 0 || L == STREAM ? 3 : 4)) k_aa(const Step<S> a) {
-    chain_next();
+    if (CHAIN) chain_next();
     const uint32_t x = blockIdx.x * a.tx + threadIdx.x;
     const uint32_t y = blockIdx.y * a.ty + threadIdx.y;
     if (x >= (uint32_t)a.geo.nx || y >= (uint32_t)a.geo.ny) return;
@@ -1387,7 +1389,7 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : (PHASE =
     const bool ahead = PF && a.pf != 0u && (uint32_t)a.geo.ny - y > a.pf;
     const uint32_t np = (y + a.pf) * (uint32_t)a.geo.nx + x;
     const uint32_t lkp = ahead ? (uint32_t)a.links[np] : SOLID_LINKS;
-    aa_node<S, L, PHASE>(a, x, y, (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
+    aa_node<S, L, PHASE, CHAIN>(a, x, y, (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
     if (PF && lkp != SOLID_LINKS) prefetch_record<S, L>(a.dst, a.N, np);
 }
 
@@ -1824,9 +1826,8 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
     if (h.algo == LPTL) {
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h)) {
-                const int b = 128;
-                return launch_update(chain, k_two_lattice_pair<S, L, true>, dim3((unsigned)((h.N / 2 + b - 1) / b)),
-                                     dim3(b), 0, st, a);
+                const dim3 b(128), g((unsigned)((h.N / 2 + 127) / 128));
+                return launch_update(chain && spread_evenly(g, b), k_two_lattice_pair<S, L, true>, g, b, 0, st, a);
             }
         }
         const int b = h.block_1d;
@@ -1837,32 +1838,37 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         }
         return launch_update(chain, k_two_lattice<S, L, true>, blocks, dim3(b), 0, st, a);
     }
+    const bool chain_tiles = chain && spread_evenly(grid, tile);
     if (h.algo == NPOL) {
         if constexpr (sizeof(S) == 4 && L == BUNDLE)
-            if (h.pf) return launch_update(chain, k_npol<S, L, true>, grid, tile, 0, st, a);
-        return launch_update(chain, k_npol<S, L, false>, grid, tile, 0, st, a);
+            if (h.pf) return launch_update(chain_tiles, k_npol<S, L, true>, grid, tile, 0, st, a);
+        return launch_update(chain_tiles, k_npol<S, L, false>, grid, tile, 0, st, a);
     }
     if (h.algo == NSOL) {
         const size_t sm = sizeof(C) * 9 * h.tile_x * h.tile_y;
         if constexpr (std::is_same<S, float>::value && L != COLLISION) {
-            if (h.tma) return launch_update(chain, k_nsol_tma<S, L>, grid, tile, sm + 16, st, a, h.tmap);
+            if (h.tma) return launch_update(chain_tiles, k_nsol_tma<S, L>, grid, tile, sm + 16, st, a, h.tmap);
         }
-        return launch_update(chain, k_nsol<S, L>, grid, tile, sm, st, a);
+        return launch_update(chain_tiles, k_nsol<S, L>, grid, tile, sm, st, a);
     }
     if (h.algo == NPTL) {
         if (L == COLLISION && h.tile_x % 32 == 0 && !(h.flags & 4u)) {
             const size_t sm = (size_t)AosSpan<S>::WARP_BYTES * ((h.tile_x * h.tile_y + 31) / 32);
-            return launch_update(chain, k_two_lattice_aos<S>, grid, tile, sm, st, a);
+            if (h.N > kChainNodes) {
+                k_two_lattice_aos<S, false><<<grid, tile, sm, st>>>(a);
+                return cudaGetLastError();
+            }
+            return launch_update(chain_tiles, k_two_lattice_aos<S>, grid, tile, sm, st, a);
         }
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h) && !(h.tile_x & 1))
-                return launch_update(chain, k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st,
-                                     a);
+                return launch_update(chain && spread_evenly(grid, dim3(h.tile_x / 2, h.tile_y)),
+                                     k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st, a);
         }
         // Two nodes per thread on request (4- and 8-byte storage): one node
         // per thread at 32 registers keeps full occupancy and measured faster.
         if (sizeof(S) >= 4 && h.tile_y >= 2 && !(h.tile_y & 1) && (h.flags & 2u))
-            return launch_update(chain, k_two_lattice2<S, L>, grid, dim3(h.tile_x, h.tile_y / 2), 0, st, a);
+            return launch_update(chain_tiles, k_two_lattice2<S, L>, grid, dim3(h.tile_x, h.tile_y / 2), 0, st, a);
     }
     if (h.algo == NPTL && h.N > kChainNodes) {
         k_two_lattice<S, L, false, false><<<grid, tile, 0, st>>>(a);
@@ -1872,6 +1878,13 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
     const dim3 cut(h.tile_x, a.ty), cuts(h.ntx, (h.ny + a.ty - 1) / a.ty);
     if (h.algo == NPTL) return launch_update(chain, k_two_lattice<S, L, false>, cuts, cut, 0, st, a);
     if (h.algo != AA) return cudaErrorInvalidValue;
+    // (bundle: 256 x 64 3.0 unchained / 2.8 chained, 500 x 333 3.9 / 4.1, 1501 x 777
+    // 11.0 / 11.4 us an update; stream 3.2 / 2.9, 4.9 / 4.9, 18.1 / 17.4)
+    if (h.N > (L == BUNDLE ? kChainNodes >> 5 : kChainNodes)) {
+        if (phase) k_aa<S, L, 1, false><<<cuts, cut, 0, st>>>(a);
+        else k_aa<S, L, 0, false><<<cuts, cut, 0, st>>>(a);
+        return cudaGetLastError();
+    }
     return phase ? launch_update(chain, k_aa<S, L, 1>, cuts, cut, 0, st, a)
                  : launch_update(chain, k_aa<S, L, 0>, cuts, cut, 0, st, a);
 }
@@ -1996,7 +2009,9 @@ int op_lptl_block(int layout) {
 template <class S>
 void op_prepare() {
     static const bool done = [] {
-        cudaFuncSetAttribute(k_two_lattice_aos<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_two_lattice_aos<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             AosSpan<S>::WARP_BYTES * (kMaxTileThreads / 32));
+        cudaFuncSetAttribute(k_two_lattice_aos<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              AosSpan<S>::WARP_BYTES * (kMaxTileThreads / 32));
         cudaGetLastError();
         return true;
