@@ -1065,18 +1065,20 @@ __device__ __forceinline__ void npol_tile(const Step<S> &a, int bx, int by, int 
     }
 }
 
-// Registers: 32 (four 512-thread blocks, spills) for the stream layout and
-// 16-bit storage, 40 (three) where it measured faster: 6000 x 3001 nodes, us an
-// update, 32 / 40 registers: stream 32 x 8 233 / 251; with the pulls by pointers
-// FP32 bundle 64 x 4 243 / 244 and 128 x 4 272 / 256, collision 338 / 305, FP16
-// 241 / 247.
-template <class S, int L, bool PF>
-__global__ void __launch_bounds__(kMaxTileThreads,
-                                  sizeof(S) == 8 ? 1 : (sizeof(S) == 4 && L != STREAM) || L == COLLISION ? 3 : 4)
+// LARGE: the lattice exceeds the L2 cache. Registers: 40 (three 512-thread
+// blocks), 32 (four, spills) for 16-bit storage and large lattices in the stream
+// layout, where that measured faster; us an update, 32 / 40 registers: stream 32 x 8
+// 6000 x 3001 nodes 233 / 251, 1501 x 777 17.0 / 16.0; with the pulls by pointers
+// 6000 x 3001 FP32 bundle 64 x 4 243 / 244 and 128 x 4 272 / 256, collision
+// 338 / 305, FP16 241 / 247.
+template <class S, int L, bool LARGE>
+__global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1
+                                                   : L == COLLISION || (sizeof(S) == 4 && !(L == STREAM && LARGE)) ? 3 : 4)
     k_npol(const Step<S> a) {
     chain_next();
-    npol_tile<S, L, PF>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
-                        (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
+    npol_tile<S, L, LARGE && sizeof(S) == 4 && L == BUNDLE>(
+        a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
+        (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
 }
 
 // TMA: the tile's populations arrive by one tensor copy (FP32 storage, stream
@@ -1199,11 +1201,12 @@ __device__ __forceinline__ void nsol_tile(const Step<S> &a, int bx, int by, int 
     }
 }
 
-#ifndef LBM_NSOL_MINB
-#define LBM_NSOL_MINB 4
-#endif
+// Registers: 40 (three 512-thread blocks), 32 (four) where the tile is staged by
+// a tensor copy and in the collision layout. us an update of 8192 x 4096 porous
+// nodes, 32 / 40 registers: FP32 bundle 64 x 4 without the copy 553 / 522, with it
+// 443 / 477, stream 32 x 8 558 / 540, collision 608 / 731, FP16 bundle 575 / 574.
 template <class S, int L>
-__global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : LBM_NSOL_MINB) k_nsol(const Step<S> a) {
+__global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : (L == COLLISION ? 4 : 3)) k_nsol(const Step<S> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     chain_next();
     nsol_tile<S, L>(a, blockIdx.x, blockIdx.y, threadIdx.x, threadIdx.y,
@@ -1213,7 +1216,7 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : LBM_NSOL
 // NSOL with the tile staged by a tensor copy; shared memory: the tile's
 // 9 T values, then the copy's mbarrier.
 template <class S, int L>
-__global__ void __launch_bounds__(kMaxTileThreads, LBM_NSOL_MINB)
+__global__ void __launch_bounds__(kMaxTileThreads, 4)
     k_nsol_tma(const Step<S> a, const __grid_constant__ TmaDesc tm) {
     extern __shared__ __align__(128) unsigned char smem_tma[];
     chain_next();
@@ -1840,8 +1843,10 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
     }
     const bool chain_tiles = chain && spread_evenly(grid, tile);
     if (h.algo == NPOL) {
-        if constexpr (sizeof(S) == 4 && L == BUNDLE)
-            if (h.pf) return launch_update(chain_tiles, k_npol<S, L, true>, grid, tile, 0, st, a);
+        if constexpr (sizeof(S) == 4 && L != COLLISION) {
+            const bool large = L == BUNDLE ? h.pf != 0 : 9 * h.N * (int64_t)sizeof(S) > (int64_t)126 << 20;
+            if (large) return launch_update(chain_tiles, k_npol<S, L, true>, grid, tile, 0, st, a);
+        }
         return launch_update(chain_tiles, k_npol<S, L, false>, grid, tile, 0, st, a);
     }
     if (h.algo == NSOL) {
