@@ -625,6 +625,9 @@ __global__ void k_widen(const float *__restrict__ s, double *__restrict__ d, int
 //    scratch buffer would add as many again.
 static constexpr size_t kWideLock = (size_t)8 << 20;
 static constexpr int64_t kScratch = 1 << 18;
+// Up to here a field takes the host's loop whatever its memory: asking what the
+// memory is costs 0.4 us, a launch more than the loop.
+static constexpr size_t kSmallField = (size_t)64 << 10;
 
 static float *host_scratch() {
     static thread_local std::unique_ptr<float[]> scratch;
@@ -652,7 +655,7 @@ lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *co
     for (int k = 0; k < fields; ++k) {
         if (!dst[k]) continue;
         const size_t bytes = (size_t)N * sizeof(double);
-        if (bytes >= kWideLock || mapped_host(dst[k])) views[k].open(dst[k], bytes, true);
+        if (bytes >= kWideLock || (bytes > kSmallField && mapped_host(dst[k]))) views[k].open(dst[k], bytes, true);
         small[k] = !views[k].ok();
         if (small[k]) continue;
         k_widen<<<kWidenBlocks, 256, 0, st>>>(src + (size_t)k * N, (double *)views[k].dev(), N);

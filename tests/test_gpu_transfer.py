@@ -125,3 +125,16 @@ def test_fp64_moments_around_the_scratch_buffer(N):
     only = np.empty(N)
     assert lbm.load().lbm_read_moments(lat.h, None, only.ctypes.data, None) == 0
     assert np.array_equal(only, lat.moments()[1].reshape(-1))
+
+
+@pytest.mark.parametrize("N", [8192, 8193])   # fields of 64 KB and one value more
+@pytest.mark.parametrize("storage", ["f32", "f64"])
+def test_moments_into_locked_memory_around_64_kb(N, storage):
+    r = np.random.default_rng(N)
+    ux, uy = 1e-2 * r.standard_normal((2, N))
+    lat = lbm.Lattice(N, 1, 0.8, storage=storage).init(1 + ux, ux, uy)
+    want = [np.array(f).reshape(-1) for f in lat.moments()]
+    got = [torch.full((N,), -1.0, dtype=torch.float64, pin_memory=True).numpy() for _ in range(3)]
+    assert lbm.load().lbm_read_moments(lat.h, *(g.ctypes.data for g in got)) == 0
+    for a, b in zip(got, want):
+        assert np.array_equal(a, b)
