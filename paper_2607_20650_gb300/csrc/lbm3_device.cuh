@@ -54,7 +54,6 @@ template <> struct Relax3<float> {
     float w0, w1, w2;   // 1/3, 1/18, 1/36
     float wl0, wl1, wl2;  // w - (float)w: rounding residuals of the weights
     float kw0, kw1, kw2;  // (1 - omega/2) w
-    int force;
 };
 template <> struct Relax3<double> {
     double om1, hom;           // 1 - omega, omega/4
@@ -64,15 +63,14 @@ template <> struct Relax3<double> {
 // T = float or f2 (each value duplicated).
 template <class T> struct NarrowRelax3 {
     T nomega;                  // -omega
-    T nw[3], nwl[3];           // -w (rest, axis, diagonal), rounded value and residual
-    T hf[3];                   // F/2
-    T a3[3], a9[3];            // 3 tau F, 9 tau F
-    T e[Q];                    // constants of the even parts, by direction (collide3_narrow)
-    T c15, c45, c3, cm3;       // 1.5, 4.5, 3, -3
+    T nw[3], nwl[3], kw[3];    // by weight (rest, axis, diagonal): -w, rounded value and residual; (1 - omega/2) w
+    T hf[3], f[3], cF[Q];      // F/2, F, c_i . F
+    T c45, c9, c3, cm3, cm15, cm1;   // 4.5, 9, 3, -3, -1.5, -1
 };
 
 template <class C, bool NARROW> struct Consts3 {
     std::conditional_t<NARROW, NarrowRelax3<C>, Relax3<C>> r;
+    int force;            // F != 0
 };
 
 // Host: FP64 constants rounded once.
@@ -92,7 +90,6 @@ inline void make_relax3(double omega, const double *F, Relax3<float> &k) {
     k.kw0 = (float)(kf / 3.0);
     k.kw1 = (float)(kf / 18.0);
     k.kw2 = (float)(kf / 36.0);
-    k.force = (F[0] != 0.0 || F[1] != 0.0 || F[2] != 0.0) ? 1 : 0;
     for (int i = 0; i < Q; ++i) k.cF[i] = (float)(cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2]);
 }
 inline void make_relax3(double omega, const double *F, Relax3<double> &q) {
@@ -108,29 +105,22 @@ inline void make_relax3(double omega, const double *F, Relax3<double> &q) {
     q.o18 = om / 18.0;
 }
 inline void make_relax3(double omega, const double *F, NarrowRelax3<float> &q) {
-    const double w[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
-    const bool force = F[0] != 0.0 || F[1] != 0.0 || F[2] != 0.0;
-    const double om = omega == 0.0 && force ? 0x1p-60 : omega;   // as in 2-D
-    const double k = force ? (1.0 - 0.5 * omega) / om : 0.0, tau = force ? k + 0.5 : 0.0;
-    q.nomega = (float)-om;
+    const double w[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0}, per[3] = {3.0, 18.0, 36.0}, kf = 1.0 - 0.5 * omega;
+    q.nomega = (float)-omega;
     for (int s = 0; s < 3; ++s) {
         q.nw[s] = (float)-w[s];
         q.nwl[s] = (float)(-w[s] - (double)q.nw[s]);
+        q.kw[s] = (float)(kf / per[s]);
+        q.hf[s] = (float)(0.5 * F[s]);
+        q.f[s] = (float)F[s];
     }
-    for (int a = 0; a < 3; ++a) {
-        q.hf[a] = (float)(0.5 * F[a]);
-        q.a3[a] = (float)(3.0 * tau * F[a]);
-        q.a9[a] = (float)(9.0 * tau * F[a]);
-    }
-    const double k0 = (0.375 + 1.5 * k) * (F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
-    for (int i = 0; i < Q; ++i) {
-        const double c = cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2];
-        q.e[i] = (float)((1.125 + 4.5 * k) * c * c - k0 + 3.0 * tau * c);
-    }
-    q.c15 = 1.5f;
+    for (int i = 0; i < Q; ++i) q.cF[i] = (float)(cx(i) * F[0] + cy(i) * F[1] + cz(i) * F[2]);
     q.c45 = 4.5f;
+    q.c9 = 9.0f;
     q.c3 = 3.0f;
     q.cm3 = -3.0f;
+    q.cm15 = -1.5f;
+    q.cm1 = -1.0f;
 }
 
 // Moments, Eq. 2 equilibrium (deviation form) and Eq. 1 BGK relaxation with
@@ -141,8 +131,8 @@ inline void make_relax3(double omega, const double *F, NarrowRelax3<float> &q) {
 // FP32 w_i P_i formed with w_i as the rounded weight plus its residual (the
 // rounded weights alone miss sum_i w_i c_i c_i = 1/3 by ~1e-8, which would
 // make the relaxation a momentum source proportional to u).
-__device__ __forceinline__ void collide3_ops(const Relax3<float> &k, float *g, float &drho, float &ux, float &uy,
-                                             float &uz) {
+__device__ __forceinline__ void collide3_ops(const Relax3<float> &k, int force, float *g, float &drho, float &ux,
+                                             float &uy, float &uz) {
     using C = float;
     using A = Ar<C>;
     C r = g[0];
@@ -190,27 +180,78 @@ __device__ __forceinline__ void collide3_ops(const Relax3<float> &k, float *g, f
         C t = A::fma(w, P, -g[i]);
         t = A::fma(sq(i) == 0 ? k.wl0 : (sq(i) == 1 ? k.wl1 : k.wl2), P, t);
         C o = A::fma(k.omega, t, g[i]);
-        if (k.force && any) {
+        if (force && any) {
             const C kw = sq(i) == 1 ? k.kw1 : k.kw2;
             o = A::fma(kw, A::fma(k.cF[i], A::fma(C(9), cu, C(3)), m3uF), o);
-        } else if (k.force) {
+        } else if (force) {
             o = A::fma(k.kw0, m3uF, o);
         }
         g[i] = o;
     }
 }
 
+// 16-bit storage, one node or a packed pair: the update above, written without
+// run-time negations as h* = g - omega (g - w P) + ... (t = g - w P), a
+// negative first term of a sum being an exact product with -1. 157 operations
+// without a force (NF), 215 with one.
+template <bool NF, class T>
+__device__ __forceinline__ void collide3_narrow(const NarrowRelax3<T> &q, T *g, T &drho, T *u) {
+    using A = Op<T>;
+    const T cm1 = A::lit(q.cm1, -1.0), cm15 = A::lit(q.cm15, -1.5), c45 = A::lit(q.c45, 4.5), c9 = A::lit(q.c9, 9.0),
+            c3 = A::lit(q.c3, 3.0), cm3 = A::lit(q.cm3, -3.0);
+    T r = g[0];
+#pragma unroll
+    for (int i = 1; i < Q; ++i) r = A::add(r, g[i]);
+    drho = r;
+    // momentum: signed sums in direction order, starting from the first term
+    bool started[3] = {false, false, false};
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int c[3] = {cx(i), cy(i), cz(i)};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (!c[a]) continue;
+            if (!started[a]) u[a] = c[a] > 0 ? g[i] : A::mul(g[i], cm1);
+            else u[a] = c[a] > 0 ? A::add(u[a], g[i]) : A::sub(u[a], g[i]);
+            started[a] = true;
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a] = A::add(u[a], q.hf[a]);
+    const T base = A::fma(cm15, A::fma(u[0], u[0], A::fma(u[1], u[1], A::mul(u[2], u[2]))), drho);
+    T m3uF = cm3;
+    if constexpr (!NF) m3uF = A::mul(cm3, A::fma(u[0], q.f[0], A::fma(u[1], q.f[1], A::mul(u[2], q.f[2]))));
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const int c[3] = {cx(i), cy(i), cz(i)};
+        T cu = base;
+        bool any = false;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (!c[a]) continue;
+            if (!any) cu = c[a] > 0 ? u[a] : A::mul(u[a], cm1);
+            else cu = c[a] > 0 ? A::add(cu, u[a]) : A::sub(cu, u[a]);
+            any = true;
+        }
+        const int s = sq(i);
+        const T P = any ? A::fma(cu, A::fma(c45, cu, c3), base) : base;
+        const T t = A::fma(q.nwl[s], P, A::fma(q.nw[s], P, g[i]));   // g - w P
+        T o = A::fma(q.nomega, t, g[i]);
+        if constexpr (!NF) o = A::fma(q.kw[s], any ? A::fma(q.cF[i], A::fma(c9, cu, c3), m3uF) : m3uF, o);
+        g[i] = o;
+    }
+}
+
 // Density and momentum of the populations (without the force's half) from the
 // sums and differences of opposite directions: 39 operations instead of 45.
-template <class T>
-__device__ __forceinline__ void moments3(const T *g, T &drho, T *u) {
-    using A = Op<T>;
-    T r = g[REST];
+__device__ __forceinline__ void moments3(const double *g, double &drho, double *u) {
+    using A = Ar<double>;
+    double r = g[REST];
     bool started[3] = {false, false, false};
 #pragma unroll
     for (int i = REST + 1; i < Q; ++i) {
         r = A::add(r, A::add(g[i], g[opp(i)]));
-        const T d = A::sub(g[i], g[opp(i)]);
+        const double d = A::sub(g[i], g[opp(i)]);
         const int c[3] = {cx(i), cy(i), cz(i)};
         // the first term of each component has c_a = +1 (directions 10, 11, 14)
 #pragma unroll
@@ -221,55 +262,6 @@ __device__ __forceinline__ void moments3(const T *g, T &drho, T *u) {
         }
     }
     drho = r;
-}
-
-// 16-bit storage, one node or a packed pair: the 2-D form (collide_narrow) on
-// nine pairs of directions; the force enters as one constant per direction
-// added to the even part. 164 operations with or without a force; direction by
-// direction 157, and 215 with a force.
-template <class T>
-__device__ __forceinline__ void collide3_narrow(const NarrowRelax3<T> &q, T *g, T &drho, T *u) {
-    using A = Op<T>;
-    T m[3];
-    moments3(g, drho, m);
-    const T c15 = A::lit(q.c15, 1.5), c45 = A::lit(q.c45, 4.5), c3 = A::lit(q.c3, 3.0), cm3 = A::lit(q.cm3, -3.0);
-    T a3[3], a9[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        u[a] = A::add(m[a], q.hf[a]);
-        a3[a] = A::fma(c15, m[a], q.a3[a]);
-        a9[a] = A::fma(c45, m[a], q.a9[a]);
-    }
-    const T base = A::sub(drho, A::fma(a3[0], m[0], A::fma(a3[1], m[1], A::mul(a3[2], m[2]))));
-    {
-        const T P = A::add(base, q.e[REST]);
-        const T t = A::fma(q.nwl[0], P, A::fma(q.nw[0], P, g[REST]));   // g - w P
-        g[REST] = A::fma(q.nomega, t, g[REST]);
-    }
-#pragma unroll
-    for (int i = REST + 1; i < Q; ++i) {
-        // direction j of the pair (i, opp(i)) whose first nonzero component (x, y, z) is +1
-        const int j = (cx(i) ? cx(i) : (cy(i) ? cy(i) : cz(i))) > 0 ? i : opp(i);
-        const int c[3] = {cx(j), cy(j), cz(j)};
-        const int s = sq(i);
-        T mc = m[0], Ac = m[0];
-        bool any = false;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!c[a]) continue;
-            mc = !any ? m[a] : (c[a] > 0 ? A::add(mc, m[a]) : A::sub(mc, m[a]));
-            Ac = !any ? a9[a] : (c[a] > 0 ? A::add(Ac, a9[a]) : A::sub(Ac, a9[a]));
-            any = true;
-        }
-        const T E = A::fma(Ac, mc, base);
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int k = e ? opp(j) : j;
-            const T P = A::fma(e ? cm3 : c3, mc, A::add(E, q.e[k]));
-            const T t = A::fma(q.nwl[s], P, A::fma(q.nw[s], P, g[k]));
-            g[k] = A::fma(q.nomega, t, g[k]);
-        }
-    }
 }
 
 // FP64: h* = (1 - omega) g + H with omega w folded into the shared parts,
@@ -324,20 +316,23 @@ template <class C, bool NARROW>
 __device__ __forceinline__ void collide3(const Consts3<C, NARROW> &k, C *g, C &drho, C &ux, C &uy, C &uz) {
     if constexpr (NARROW || sizeof(C) == 8) {
         C u[3];
-        if constexpr (NARROW) collide3_narrow(k.r, g, drho, u);
-        else collide3_ops64(k.r, g, drho, u);
+        if constexpr (!NARROW) collide3_ops64(k.r, g, drho, u);
+        else if (k.force) collide3_narrow<false>(k.r, g, drho, u);
+        else collide3_narrow<true>(k.r, g, drho, u);
         ux = u[0];
         uy = u[1];
         uz = u[2];
     } else {
-        collide3_ops(k.r, g, drho, ux, uy, uz);
+        collide3_ops(k.r, k.force, g, drho, ux, uy, uz);
     }
 }
 
 // Two nodes of 16-bit storage at once: each lane equals the one-node form bit for bit.
-__device__ __forceinline__ void collide3_2(const NarrowRelax3<f2> &q, f2 *g, f2 &drho, f2 &ux, f2 &uy, f2 &uz) {
+__device__ __forceinline__ void collide3_2(const NarrowRelax3<f2> &q, int force, f2 *g, f2 &drho, f2 &ux, f2 &uy,
+                                           f2 &uz) {
     f2 u[3];
-    collide3_narrow(q, g, drho, u);
+    if (force) collide3_narrow<false>(q, g, drho, u);
+    else collide3_narrow<true>(q, g, drho, u);
     ux = u[0];
     uy = u[1];
     uz = u[2];

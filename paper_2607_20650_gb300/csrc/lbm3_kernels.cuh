@@ -435,7 +435,7 @@ __device__ __forceinline__ void step3_pair(const Step3<S> &a, uint32_t x, uint32
         for (int i = 0; i < Q; ++i) g[i] = pk2(ga[i], gb[i]);
     }
     f2 drho, ux, uy, uz;
-    collide3_2(a.k2, g, drho, ux, uy, uz);
+    collide3_2(a.k2, a.k.force, g, drho, ux, uy, uz);
     float da, db;
     up2(drho, da, db);
     if ((fa && !isfinite(da)) || (fb && !isfinite(db))) atomicOr(a.err, 1u);

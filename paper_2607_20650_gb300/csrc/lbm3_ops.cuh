@@ -46,6 +46,7 @@ Step3<S> make3(const lbm3_lattice *L, int src, int toff, int mom) {
     }
     a.N = (uint32_t)L->pl.N;
     make_relax3(1.0 / p.tau, p.force, a.k.r);
+    a.k.force = (p.force[0] != 0.0 || p.force[1] != 0.0 || p.force[2] != 0.0) ? 1 : 0;
     {
         const int64_t N = L->pl.N, nx = p.nx, nxy = (int64_t)p.nx * p.ny;
         for (int i = 0; i < Q; ++i) {

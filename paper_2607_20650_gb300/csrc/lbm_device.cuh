@@ -313,14 +313,13 @@ template <> struct Relax<double> {
     double k[2], c[2];         // (1 - omega/2) F, (1 - omega/2) F / 3
     double o3, o36;            // omega/3, omega/36
 };
-// T = float or f2 (each value duplicated); kF = (1 - omega/2)/omega F.
+// T = float or f2 (each value duplicated).
 template <class T> struct NarrowRelax {
     T nomega;                  // -omega
-    T nw[3], nwl[3];           // -w (diagonal, axis, rest), rounded value and residual
+    T nw[3], nwl[3], kw[3];    // by weight (diagonal, axis, rest): -w, rounded value and residual; (1 - omega/2) w
     T hfx, hfy;                // F/2
-    T a3[2], a9[2];            // 3 tau F, 9 tau F
-    T cp[4], cm[4], c0;        // constants of the even parts (collide_narrow)
-    T c15, cm15, c45, c3, cm3; // 1.5, -1.5, 4.5, 3, -3
+    T fx, fy, sF, dF;          // F, fx+fy, fx-fy
+    T c45, c9, c3, cm3, cm15;  // 4.5, 9, 3, -3, -1.5
 };
 
 struct NoPairs {};   // stands for the pair constants of storage types without node pairs
@@ -369,36 +368,24 @@ inline void make_relax(double omega, double fx, double fy, Relax<double> &q) {
     q.o36 = om / 36.0;
 }
 inline void make_relax(double omega, double fx, double fy, NarrowRelax<float> &q) {
-    const double w[3] = {1.0 / 36.0, 1.0 / 9.0, 4.0 / 9.0};
-    // Without relaxation (tau infinite) a force needs omega kF = F all the
-    // same: a power of two far below every rounding stands for omega.
-    const bool force = fx != 0.0 || fy != 0.0;
-    const double om = omega == 0.0 && force ? 0x1p-60 : omega;
-    const double k = force ? (1.0 - 0.5 * omega) / om : 0.0, tau = force ? k + 0.5 : 0.0;
-    q.nomega = (float)-om;
+    const double w[3] = {1.0 / 36.0, 1.0 / 9.0, 4.0 / 9.0}, kf = 1.0 - 0.5 * omega;
+    q.nomega = (float)-omega;
     for (int s = 0; s < 3; ++s) {
         q.nw[s] = (float)-w[s];
         q.nwl[s] = (float)(-w[s] - (double)q.nw[s]);
+        q.kw[s] = (float)(s == 1 ? kf / 9.0 : (s == 0 ? kf / 36.0 : 4.0 * kf / 9.0));
     }
     q.hfx = (float)(0.5 * fx);
     q.hfy = (float)(0.5 * fy);
-    const double F[2] = {fx, fy}, c[4] = {fx + fy, fy, fx - fy, fx};
-    for (int a = 0; a < 2; ++a) {
-        q.a3[a] = (float)(3.0 * tau * F[a]);
-        q.a9[a] = (float)(9.0 * tau * F[a]);
-    }
-    const double k0 = (0.375 + 1.5 * k) * (fx * fx + fy * fy);
-    q.c0 = (float)-k0;
-    for (int m = 0; m < 4; ++m) {
-        const double e = (1.125 + 4.5 * k) * c[m] * c[m] - k0, o = 3.0 * tau * c[m];
-        q.cp[m] = (float)(e + o);
-        q.cm[m] = (float)(e - o);
-    }
-    q.c15 = 1.5f;
-    q.cm15 = -1.5f;
+    q.fx = (float)fx;
+    q.fy = (float)fy;
+    q.sF = (float)(fx + fy);
+    q.dF = (float)(fx - fy);
     q.c45 = 4.5f;
+    q.c9 = 9.0f;
     q.c3 = 3.0f;
     q.cm3 = -3.0f;
+    q.cm15 = -1.5f;
 }
 // A block of float constants with each duplicated into both lanes.
 template <template <class> class R>
@@ -480,72 +467,65 @@ __device__ __forceinline__ void collide_ops(const Relax<float> &k, int force, fl
     }
 }
 
-// Density and momentum of the populations (without the force's half).
-template <class T>
-__device__ __forceinline__ void moments2(const T *g, T &drho, T &mx, T &my) {
-    using A = Op<T>;
-    const T cw = A::add(A::add(g[0], g[6]), g[3]);   // c_x = -1 column
-    const T cm = A::add(A::add(g[1], g[7]), g[4]);   // c_x =  0
-    const T ce = A::add(A::add(g[2], g[8]), g[5]);   // c_x = +1
-    drho = A::add(A::add(cw, ce), cm);
-    mx = A::sub(ce, cw);
-    my = A::add(A::add(A::sub(g[6], g[0]), A::sub(g[8], g[2])), A::sub(g[7], g[1]));
-}
-
 // 16-bit storage, one node or a packed pair: the update above as
-//   h*_i = g_i - omega (g_i - w_i P_i),
-//   P_i  = drho - 3/2 u^2 + cu (3 + 9/2 cu) + k [cF (3 + 9 cu) - 3 u.F],  k = (1 - omega/2)/omega,
-// with u = m + F/2 written out in the populations' momentum m. Opposite
-// directions share the even part of P and differ in the sign of the odd part:
-//   P_+- = drho - T + A_c m_c + (e_c +- 3 tau F_c) +- 3 m_c,
-//   T = (3/2 m + 3 tau F).m,   A = 9/2 m + 9 tau F,   c = x, y, x + y, x - y,
-// e_c the terms in F^2. 73 operations (direction by direction 92) or, without
-// a force (NF), 62 (64). The kernels are bound by instruction issue: the node
-// pairs on 8192 x 4096 porous nodes, FP16, 246 -> 232 us an update. The force enters as a
-// constant added to an even part: added to the momentum or to h*, which lie
-// on a coarser grid, a constant is rounded the same way at every update, and
-// a forced flow drifts by 1e-6 in 100 updates (this order: 1e-7). w P is not
-// rounded by itself, and w is used as rounded value plus residual, for the
-// same reason. No run-time negations (t = g - w P), so that one node and a
-// packed pair run the same code and agree bit for bit.
+//   h*_i = g_i - omega (g_i - w_i P_i) + (1 - omega/2) w_i [cF_i (3 + 9 cu_i) - 3 u.F]
+// Every direction is written through the signed velocity c of its pair (u_x, u_y,
+// u_x + u_y, u_x - u_y) and the sign sg of cu_i = sg c:
+//   cu_i (3 + 9/2 cu_i) = c (9/2 c + 3 sg),  cF_i (3 + 9 cu_i) = cF+ (9 c + 3 sg)
+// with cF+ = sg cF_i, so no operand is negated at run time and one node and a
+// packed pair perform the same rounded operations. 92 operations, 64 without a
+// force (NF). The force enters after the relaxation: with (1 - omega/2)/omega F in P,
+// 73 operations, the node pairs take the same time (8192 x 4096 porous nodes, 16
+// updates: 3.57 against 3.59 ms), and the form overflows where tau F does.
 template <bool NF, class T>
 __device__ __forceinline__ void collide_narrow(const NarrowRelax<T> &q, T *g, T &drho, T &ux, T &uy) {
     using A = Op<T>;
-    T mx, my;
-    moments2(g, drho, mx, my);
-    const T c15 = A::lit(q.c15, 1.5), cm15 = A::lit(q.cm15, -1.5), c45 = A::lit(q.c45, 4.5), c3 = A::lit(q.c3, 3.0),
+    const T cw = A::add(A::add(g[0], g[3]), g[6]);   // c_x = -1 column
+    const T cm = A::add(A::add(g[1], g[4]), g[7]);   // c_x =  0
+    const T ce = A::add(A::add(g[2], g[5]), g[8]);   // c_x = +1
+    const T rs = A::add(A::add(g[0], g[1]), g[2]);   // c_y = -1 row
+    const T rn = A::add(A::add(g[6], g[7]), g[8]);   // c_y = +1
+    drho = A::add(A::add(cw, cm), ce);
+    ux = A::add(A::sub(ce, cw), q.hfx);
+    uy = A::add(A::sub(rn, rs), q.hfy);
+    const T cm15 = A::lit(q.cm15, -1.5), c45 = A::lit(q.c45, 4.5), c9 = A::lit(q.c9, 9.0), c3 = A::lit(q.c3, 3.0),
             cm3 = A::lit(q.cm3, -3.0);
+    const T base = A::fma(cm15, A::fma(ux, ux, A::mul(uy, uy)), drho);
+    T m3uF = cm3;
+    if constexpr (!NF) m3uF = A::mul(cm3, A::fma(ux, q.fx, A::mul(uy, q.fy)));
     // pairs (0, 8), (1, 7), (6, 2), (3, 5); c points to the second
-    const T m[4] = {A::add(mx, my), my, A::sub(mx, my), mx};
-    T base, Ac[4];
-    if constexpr (NF) {
-        base = A::fma(cm15, A::fma(mx, mx, A::mul(my, my)), drho);
-    } else {
-        const T ax = A::fma(c15, mx, q.a3[0]), ay = A::fma(c15, my, q.a3[1]);
-        base = A::sub(drho, A::fma(ax, mx, A::mul(ay, my)));
-        Ac[3] = A::fma(c45, mx, q.a9[0]);
-        Ac[1] = A::fma(c45, my, q.a9[1]);
-        Ac[0] = A::add(Ac[3], Ac[1]);
-        Ac[2] = A::sub(Ac[3], Ac[1]);
-    }
+    const T c[4] = {A::add(ux, uy), uy, A::sub(ux, uy), ux};
+    const T cF[4] = {q.sF, q.fy, q.dF, q.fx};
     const int lo[4] = {0, 1, 6, 3};
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
         const int s = p & 1;   // axis directions
-        const T E = A::fma(NF ? A::mul(c45, m[p]) : Ac[p], m[p], base);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int i = e ? opp(lo[p]) : lo[p];
-            const T P = A::fma(e ? c3 : cm3, m[p], NF ? E : A::add(E, e ? q.cp[p] : q.cm[p]));
+            const T sg3 = e ? c3 : cm3;
+            const T P = A::fma(c[p], A::fma(c45, c[p], sg3), base);
             const T t = A::fma(q.nwl[s], P, A::fma(q.nw[s], P, g[i]));   // g - w P
-            g[i] = A::fma(q.nomega, t, g[i]);
+            T o = A::fma(q.nomega, t, g[i]);
+            if constexpr (!NF) o = A::fma(q.kw[s], A::fma(cF[p], A::fma(c9, c[p], sg3), m3uF), o);
+            g[i] = o;
         }
     }
-    if constexpr (!NF) base = A::add(base, q.c0);
     const T t = A::fma(q.nwl[2], base, A::fma(q.nw[2], base, g[4]));
-    g[4] = A::fma(q.nomega, t, g[4]);
-    ux = NF ? mx : A::add(mx, q.hfx);
-    uy = NF ? my : A::add(my, q.hfy);
+    T o = A::fma(q.nomega, t, g[4]);
+    if constexpr (!NF) o = A::fma(q.kw[2], m3uF, o);
+    g[4] = o;
+}
+
+// Density and momentum of the populations (without the force's half).
+__device__ __forceinline__ void moments2(const double *g, double &drho, double &mx, double &my) {
+    using A = Ar<double>;
+    const double cw = A::add(A::add(g[0], g[6]), g[3]);   // c_x = -1 column
+    const double cm = A::add(A::add(g[1], g[7]), g[4]);   // c_x =  0
+    const double ce = A::add(A::add(g[2], g[8]), g[5]);   // c_x = +1
+    drho = A::add(A::add(cw, ce), cm);
+    mx = A::sub(ce, cw);
+    my = A::add(A::add(A::sub(g[6], g[0]), A::sub(g[8], g[2])), A::sub(g[7], g[1]));
 }
 
 // FP64 (its arithmetic bounds every FP64 kernel, and its rounding is no
