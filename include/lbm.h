@@ -181,9 +181,10 @@ lbm_status lbm_wait(lbm_lattice *L, double timeout_s);
 /* Moments of the last update that stored them (or of lbm_init), as host
  * doubles, N each (solid nodes: rho = 1, v = 0); a NULL array is skipped.
  * Synchronous. FP32 moments are widened by the device straight into
- * page-locked destinations (cudaHostAlloc, cudaHostRegister) and into
- * pageable ones of 8 MB and more, which are page-locked during the call;
- * smaller ones, and memory that cannot be locked, on the host. */
+ * page-locked destinations (cudaHostAlloc, cudaHostRegister); fields of 8 MB
+ * and more in other memory come through page-locked buffers of the calling
+ * thread (32 MB, allocated by its first large transfer, freed when it ends),
+ * smaller ones are widened on the host. */
 lbm_status lbm_read_moments(lbm_lattice *L, double *rho, double *ux, double *uy);
 
 /* Same moments as FP32 device arrays (N each), enqueued on the stream. */
@@ -202,8 +203,9 @@ lbm_status lbm_force(lbm_lattice *L, const uint8_t *d_body, double out[2]);
 /* Copy the state to / from host memory in canonical order h[i*N + n],
  * as = LBM_F64 (double) or LBM_F32 (float). Writes round to the storage
  * type (via FP32 for F16S/BF16S, nearest-even). Synchronous. The device
- * converts; pageable buffers of 1 MB and more are page-locked during the
- * call (memory that cannot be locked is copied and converted on the host). */
+ * converts: in page-locked memory in place, 1 MB and more of other memory
+ * through the thread's page-locked buffers (lbm_read_moments); less is copied
+ * and converted on the host. */
 lbm_status lbm_read_populations(lbm_lattice *L, void *host, int32_t as);
 lbm_status lbm_write_populations(lbm_lattice *L, const void *host, int32_t as);
 

@@ -379,19 +379,27 @@ static lbm_status state_readable(const lbm3_lattice *L) {
     return LBM_OK;
 }
 
+static lbm_status transfer_state3(lbm3_lattice *L, void *host, int32_t as, bool read, bool *done) {
+    struct Ctx {
+        lbm3_lattice *L;
+        bool f64, read;
+    } ctx{L, as == LBM_F64, read};
+    auto move = [](void *c, void *rows, int64_t n0, int64_t count, int64_t stride) {
+        const Ctx &x = *(const Ctx *)c;
+        return x.L->ops->transfer(x.L, rows, x.read, x.f64, n0, count, stride, x.L->stream);
+    };
+    return lbm_transfer_state(19, L->pl.N, as == LBM_F64 ? 8 : 4, host, read, L->stream, move, &ctx, done);
+}
+
 extern "C" lbm_status lbm3_read_populations(lbm3_lattice *L, void *host, int32_t as) {
     if (!L || !host) return lbm_fail(LBM_EINVAL, "NULL argument");
     if (state_readable(L) != LBM_OK) return LBM_EINVAL;
     if (as != LBM_F64 && as != LBM_F32) return lbm_fail(LBM_EINVAL, "as must be LBM_F64 or LBM_F32");
     const int64_t N = L->pl.N;
-    {
-        HostView v(host, 19 * (size_t)N * (as == LBM_F64 ? 8 : 4), true);
-        if (v.ok()) {
-            CK3(L->ops->transfer(L, v.dev(), nullptr, as == LBM_F64, L->stream));
-            CK3(cudaStreamSynchronize(L->stream));
-            return lbm3_check(L);
-        }
-    }
+    bool done;
+    const lbm_status s = transfer_state3(L, host, as, true, &done);
+    if (s != LBM_OK) return s;
+    if (done) return lbm3_check(L);
     std::vector<unsigned char> raw(19 * (size_t)N * L->pl.elem);
     CK3(cudaStreamSynchronize(L->stream));
     CK3(cudaMemcpy(raw.data(), L->ws + L->pl.pop[L->cur], raw.size(), cudaMemcpyDeviceToHost));
@@ -410,29 +418,24 @@ extern "C" lbm_status lbm3_write_populations(lbm3_lattice *L, const void *host, 
     if (state_readable(L) != LBM_OK) return LBM_EINVAL;
     if (as != LBM_F64 && as != LBM_F32) return lbm_fail(LBM_EINVAL, "as must be LBM_F64 or LBM_F32");
     const int64_t N = L->pl.N;
-    {
-        HostView v((void *)host, 19 * (size_t)N * (as == LBM_F64 ? 8 : 4), false);
-        if (v.ok()) {
-            CK3(L->ops->transfer(L, nullptr, v.dev(), as == LBM_F64, L->stream));
-            if (L->pl.halo_parity) CK3(L->ops->publish(L, L->cur, L->stream));
-            CK3(cudaStreamSynchronize(L->stream));
-            return LBM_OK;
-        }
-    }
-    std::vector<unsigned char> raw(19 * (size_t)N * L->pl.elem);
-    for (int i = 0; i < 19; ++i)
-        for (int64_t n = 0; n < N; ++n) {
-            const double v = as == LBM_F64 ? ((const double *)host)[(int64_t)i * N + n]
-                                           : (double)((const float *)host)[(int64_t)i * N + n];
-            set_raw(raw.data(), L->p.storage, lbm3_layout_index(L->p.layout, N, n, L->p.algo == LBM_NSOL ? 18 - i : i),
-                    v);
-        }
-    CK3(cudaStreamSynchronize(L->stream));
-    CK3(cudaMemcpy(L->ws + L->pl.pop[L->cur], raw.data(), raw.size(), cudaMemcpyHostToDevice));
-    if (L->pl.halo_parity) {   // NPOL: the next update reads parity cur of the buffer grid
-        CK3(L->ops->publish(L, L->cur, L->stream));
+    bool done;
+    const lbm_status s = transfer_state3(L, (void *)host, as, false, &done);
+    if (s != LBM_OK) return s;
+    if (!done) {
+        std::vector<unsigned char> raw(19 * (size_t)N * L->pl.elem);
+        for (int i = 0; i < 19; ++i)
+            for (int64_t n = 0; n < N; ++n) {
+                const double v = as == LBM_F64 ? ((const double *)host)[(int64_t)i * N + n]
+                                               : (double)((const float *)host)[(int64_t)i * N + n];
+                set_raw(raw.data(), L->p.storage,
+                        lbm3_layout_index(L->p.layout, N, n, L->p.algo == LBM_NSOL ? 18 - i : i), v);
+            }
         CK3(cudaStreamSynchronize(L->stream));
+        CK3(cudaMemcpy(L->ws + L->pl.pop[L->cur], raw.data(), raw.size(), cudaMemcpyHostToDevice));
     }
+    // NPOL, NSOL: the next update reads parity cur of the buffer grid
+    if (L->pl.halo_parity) CK3(L->ops->publish(L, L->cur, L->stream));
+    CK3(cudaStreamSynchronize(L->stream));
     return LBM_OK;
 }
 

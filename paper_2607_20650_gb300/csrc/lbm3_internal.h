@@ -58,9 +58,10 @@ struct Ops3 {
                         cudaStream_t st);
     // rho, u of the stored state into the moments array.
     cudaError_t (*state_moments)(const lbm3_lattice *L, cudaStream_t st);
-    // The current state to `out` or from `in` (one of them null), canonical
-    // order in mapped host memory, doubles or floats.
-    cudaError_t (*transfer)(const lbm3_lattice *L, void *out, const void *in, bool f64, cudaStream_t st);
+    // Nodes n0 .. n0 + count - 1 of the current state to (read) or from
+    // rows[i stride + n - n0] in mapped host memory, doubles or floats.
+    cudaError_t (*transfer)(const lbm3_lattice *L, void *rows, bool read, bool f64, int64_t n0, int64_t count,
+                            int64_t stride, cudaStream_t st);
     // Fill buffer-grid parity `parity` from the stored state (NPOL, NSOL).
     cudaError_t (*publish)(const lbm3_lattice *L, int parity, cudaStream_t st);
     // FP64 block partial sums of the mass (one per block) and force (three).

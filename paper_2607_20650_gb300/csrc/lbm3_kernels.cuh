@@ -926,24 +926,27 @@ __global__ void k3_init(const Step3<S> a, const double *rho, const double *ux, c
     }
 }
 
-// The stored state to / from canonical order in mapped host memory (as the 2-D
-// k_export / k_import; values of solid nodes are stored as given).
+// Nodes n0 .. n0 + count - 1 of the stored state to / from canonical order in
+// mapped host memory (as the 2-D k_export / k_import; values of solid nodes are
+// stored as given).
 template <class S, int L, class H>
-__global__ void __launch_bounds__(256) k3_export(const Step3<S> a, H *out) {
-    const uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= a.N) return;
+__global__ void __launch_bounds__(256) k3_export(const Step3<S> a, H *rows, uint64_t n0, uint32_t count,
+                                                 uint64_t stride) {
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= count) return;
 #pragma unroll
     for (int i = 0; i < Q; ++i)
-        out[(uint64_t)i * a.N + n] = (H)Codec<S>::dec(a.src[addr<L>(a.N, (int64_t)n, slot3(a, i))]);
+        rows[i * stride + k] = (H)Codec<S>::dec(a.src[addr<L>(a.N, (int64_t)(n0 + k), slot3(a, i))]);
 }
 template <class S, int L, class H>
-__global__ void __launch_bounds__(256) k3_import(const Step3<S> a, const H *in) {
+__global__ void __launch_bounds__(256) k3_import(const Step3<S> a, const H *rows, uint64_t n0, uint32_t count,
+                                                 uint64_t stride) {
     using C = typename Codec<S>::C;
-    const uint64_t n = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= a.N) return;
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= count) return;
 #pragma unroll
     for (int i = 0; i < Q; ++i)
-        a.dst[addr<L>(a.N, (int64_t)n, slot3(a, i))] = Codec<S>::enc((C)in[(uint64_t)i * a.N + n], false, 0u);
+        a.dst[addr<L>(a.N, (int64_t)(n0 + k), slot3(a, i))] = Codec<S>::enc((C)rows[i * stride + k], false, 0u);
 }
 
 template <class S, int L>

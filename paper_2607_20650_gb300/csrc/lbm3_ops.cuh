@@ -242,22 +242,25 @@ cudaError_t init3(const lbm3_lattice *L, const double *const dv[4], uint32_t n0,
 }
 
 template <class S, int L>
-cudaError_t transfer_k(const lbm3_lattice *L_, void *out, const void *in, bool f64, cudaStream_t st) {
+cudaError_t transfer_k(const lbm3_lattice *L_, void *rows, bool read, bool f64, int64_t n0, int64_t count,
+                       int64_t stride, cudaStream_t st) {
     // current lattice as the source of an export and the destination of an import
-    const Step3<S> a = make3<S>(L_, in ? L_->cur ^ 1 : L_->cur, 0, 0);
-    const unsigned g = (unsigned)((L_->pl.N + 255) / 256);
-    if (out && f64) k3_export<S, L, double><<<g, 256, 0, st>>>(a, (double *)out);
-    else if (out) k3_export<S, L, float><<<g, 256, 0, st>>>(a, (float *)out);
-    else if (f64) k3_import<S, L, double><<<g, 256, 0, st>>>(a, (const double *)in);
-    else k3_import<S, L, float><<<g, 256, 0, st>>>(a, (const float *)in);
+    const Step3<S> a = make3<S>(L_, read ? L_->cur : L_->cur ^ 1, 0, 0);
+    const unsigned g = (unsigned)((count + 255) / 256);
+    const uint32_t c = (uint32_t)count;
+    if (read && f64) k3_export<S, L, double><<<g, 256, 0, st>>>(a, (double *)rows, n0, c, stride);
+    else if (read) k3_export<S, L, float><<<g, 256, 0, st>>>(a, (float *)rows, n0, c, stride);
+    else if (f64) k3_import<S, L, double><<<g, 256, 0, st>>>(a, (const double *)rows, n0, c, stride);
+    else k3_import<S, L, float><<<g, 256, 0, st>>>(a, (const float *)rows, n0, c, stride);
     return cudaGetLastError();
 }
 
 template <class S>
-cudaError_t transfer3(const lbm3_lattice *L, void *out, const void *in, bool f64, cudaStream_t st) {
-    if (L->p.layout == LBM_LAYOUT_STREAM) return transfer_k<S, STREAM>(L, out, in, f64, st);
-    if (L->p.layout == LBM_LAYOUT_BUNDLE) return transfer_k<S, BUNDLE>(L, out, in, f64, st);
-    return transfer_k<S, COLLISION>(L, out, in, f64, st);
+cudaError_t transfer3(const lbm3_lattice *L, void *rows, bool read, bool f64, int64_t n0, int64_t count,
+                      int64_t stride, cudaStream_t st) {
+    auto f = L->p.layout == LBM_LAYOUT_STREAM ? transfer_k<S, STREAM>
+             : L->p.layout == LBM_LAYOUT_BUNDLE ? transfer_k<S, BUNDLE> : transfer_k<S, COLLISION>;
+    return f(L, rows, read, f64, n0, count, stride, st);
 }
 
 template <class S>

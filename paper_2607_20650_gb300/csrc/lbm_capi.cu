@@ -15,7 +15,6 @@
 #include <cstring>
 #include <new>
 #include <string>
-#include <system_error>
 #include <memory>
 #include <thread>
 #include <vector>
@@ -24,6 +23,7 @@
 #include "lbm_capi_internal.h"
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
+#include "lbm_staging.h"
 
 using namespace lbm;
 
@@ -531,33 +531,6 @@ extern "C" lbm_status lbm_wait(lbm_lattice *L, double timeout_s) {
     return lbm_sync(L);
 }
 
-// ------------------------------------------------------------ host loops
-// Run fn(begin, end) over [0, count) on up to 16 host threads (large arrays
-// only; the conversions below are independent per element).
-template <class Fn>
-static void parallel_for(int64_t count, Fn fn, int64_t grain = 1 << 20) {
-    int nt = (int)std::min<int64_t>(16, std::max<int64_t>(1, count / grain));
-    const unsigned hw = std::thread::hardware_concurrency();
-    if (hw > 0) nt = std::min<int>(nt, (int)hw);
-    if (nt <= 1) {
-        fn((int64_t)0, count);
-        return;
-    }
-    std::thread th[16];
-    const int64_t step = (count + nt - 1) / nt;
-    for (int t = 0; t < nt; ++t) {
-        const int64_t b = t * step, e = std::min(count, b + step);
-        if (b >= e) break;
-        try {
-            th[t] = std::thread(fn, b, e);
-        } catch (const std::system_error &) {   // no thread to be had: this one does it
-            fn(b, e);
-        }
-    }
-    for (auto &x : th)
-        if (x.joinable()) x.join();
-}
-
 // ------------------------------------------------------------ read-out
 // Device address of a page-locked, mapped host buffer (cudaHostAlloc,
 // cudaHostRegister, torch pin_memory), or NULL for pageable memory.
@@ -569,40 +542,113 @@ static void *mapped_host(const void *p) {
     }
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
-
-// Locking 1.4 MB costs about 60 us and 151 MB 0.7 ms once its pages exist;
-// below this size host loops are as fast.
-static constexpr size_t kRegisterBytes = (size_t)1 << 20;
-
-void HostView::open(void *p, size_t bytes, bool write) {
-    if (!p || bytes == 0) return;
-    char *last = (char *)p + (bytes - 1);
-    if (char *d = (char *)mapped_host(p)) {
-        if ((char *)mapped_host(last) == d + (bytes - 1)) dev_ = d;
-        return;
-    }
-    if (bytes < kRegisterBytes) return;
-    if (write) {
-        // Locking a page that does not exist yet makes the kernel allocate it
-        // on one thread; touching the pages first on several is 3 times faster.
-        const int64_t page = 4096;
-        parallel_for((int64_t)(bytes / page), [p, page](int64_t b, int64_t e) {
-            for (int64_t k = b; k < e; ++k) ((volatile char *)p)[k * page] = 0;
-        }, 2048);
-    }
-    if (cudaHostRegister(p, bytes, cudaHostRegisterMapped) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return;
-    }
-    locked_ = p;
-    if (cudaHostGetDevicePointer(&dev_, p, 0) != cudaSuccess) {
-        (void)cudaGetLastError();
-        dev_ = nullptr;
-    }
+// The same for `bytes` bytes.
+static void *mapped_host(const void *p, size_t bytes) {
+    char *d = (char *)mapped_host(p);
+    return d && (char *)mapped_host((const char *)p + (bytes - 1)) == d + (bytes - 1) ? d : nullptr;
 }
 
-HostView::~HostView() {
-    if (locked_ && cudaHostUnregister(locked_) != cudaSuccess) (void)cudaGetLastError();
+// Page-locked slots of the calling thread (32 MB in all), allocated by its first
+// large transfer (1 ms) and freed when it ends; nullptr if there are none to be had.
+// The caller's own pages are never locked: a lock would be seen, and could be
+// used or released too early, by other calls and by copies elsewhere in the
+// program that touch the same memory.
+// Chunks of 2 MB, of 1 MB where that would be fewer than eight: each is one kernel,
+// and kernels of 1 MB one after another fall short of the link. FP32 state to /
+// from doubles, 6 / 151 / 1,300 MB on the host, ms: chunks of 0.5 MB 0.48 / 4.0 / 23.5 to
+// fresh pages and 0.42 / 4.3 / 33.4 back, 1 MB 0.27 / 3.8 / 21.5 and 0.24 / 2.9 / 20.6, 2 MB
+// 0.51 / 3.65 / 20.7 and 0.36 / 2.0 / 14.9, 4 MB no faster; 7 instead of 15 workers 26 and
+// 16 ms for the largest. (Copies of the raw state and loops on the host: 1.6 / 23.8 / 62
+// and 1.4 / 22.9 / 62 ms.)
+constexpr size_t kSlotBytes = (size_t)2 << 20;
+static size_t chunk_bytes(size_t total) { return total < 8 * kSlotBytes ? kSlotBytes / 2 : kSlotBytes; }
+
+static char *stage_slots() {
+    struct Slots {
+        char *p = nullptr;
+        ~Slots() {
+            if (p && cudaFreeHost(p) != cudaSuccess) (void)cudaGetLastError();
+        }
+    };
+    static thread_local Slots slots;
+    if (slots.p && !mapped_host(slots.p)) slots.p = nullptr;   // released by a device reset
+    if (!slots.p && cudaHostAlloc((void **)&slots.p, kStageSlots * kSlotBytes,
+                                  cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        (void)cudaGetLastError();
+        slots.p = nullptr;
+    }
+    return slots.p;
+}
+
+// staged_transfer() over a stream: launch(chunk, slot memory) enqueues the
+// device's part, rows(chunk, slot memory, f) calls f(array, slot, bytes) for each
+// contiguous piece of the chunk.
+template <class Launch, class Rows> struct StageIo {
+    char *slots;
+    cudaStream_t st;
+    Launch enqueue;
+    Rows rows;
+    bool to_host;
+    cudaEvent_t ev[kStageSlots];
+    cudaError_t err;
+    char *at(int slot) const { return slots + (size_t)slot * kSlotBytes; }
+    bool check(cudaError_t e) {
+        if (e != cudaSuccess && err == cudaSuccess) err = e;
+        return e == cudaSuccess;
+    }
+    bool launch(int64_t chunk, int slot) { return check(enqueue(chunk, at(slot))) && check(cudaEventRecord(ev[slot], st)); }
+    bool wait(int slot) { return check(cudaEventSynchronize(ev[slot])); }
+    void copy(int64_t chunk, int slot) {
+        rows(chunk, at(slot), [this](char *h, char *s, size_t bytes) {
+            if (to_host) memcpy(h, s, bytes);
+            else memcpy(s, h, bytes);
+        });
+    }
+};
+
+// Starting a thread costs 50 us, so their number grows with the transfer.
+template <class Launch, class Rows>
+static cudaError_t run_staged(char *slots, int64_t chunks, bool to_host, cudaStream_t st, Launch launch, Rows rows) {
+    StageIo<Launch, Rows> io{slots, st, launch, rows, to_host, {}, cudaSuccess};
+    const int hw = (int)std::thread::hardware_concurrency();
+    const int most = std::min(kStageSlots, hw) - 1;
+    const int workers = chunks > 2 ? (int)std::min<int64_t>(most, std::min(chunks / 2, 6 + chunks / 32)) : 0;
+    int made = 0;
+    const int used = (int)std::min<int64_t>(kStageSlots, chunks);
+    while (made < used && io.check(cudaEventCreateWithFlags(&io.ev[made], cudaEventDisableTiming))) ++made;
+    if (made == used && !staged_transfer(io, chunks, std::max(0, workers), to_host))
+        (void)cudaStreamSynchronize(st);   // also for a launch whose event failed
+    for (int k = 0; k < made; ++k) cudaEventDestroy(io.ev[k]);
+    if (io.err != cudaSuccess) (void)cudaGetLastError();
+    return io.err;
+}
+
+// From here state goes through the slots.
+static constexpr size_t kStageBytes = (size_t)1 << 20;
+
+lbm_status lbm_transfer_state(int q, int64_t N, size_t es, void *host, bool read, cudaStream_t st, MoveState move,
+                              void *ctx, bool *done) {
+    *done = true;
+    if (void *d = mapped_host(host, (size_t)q * N * es)) {
+        const cudaError_t e = move(ctx, d, 0, N, N);
+        CK(cudaStreamSynchronize(st));
+        CK(e);
+        return LBM_OK;
+    }
+    char *slots = (size_t)q * N * es >= kStageBytes ? stage_slots() : nullptr;
+    if (!slots) {
+        *done = false;
+        return LBM_OK;
+    }
+    const int64_t m = (int64_t)(chunk_bytes((size_t)q * N * es) / (q * es)) / 32 * 32;   // nodes per chunk
+    auto launch = [=](int64_t c, char *slot) { return move(ctx, slot, c * m, std::min(m, N - c * m), m); };
+    auto rows = [=](int64_t c, char *slot, auto f) {
+        const size_t bytes = (size_t)std::min(m, N - c * m) * es;
+        for (int i = 0; i < q; ++i)
+            f((char *)host + ((size_t)i * N + (size_t)(c * m)) * es, slot + (size_t)i * m * es, bytes);
+    };
+    CK(run_staged(slots, (N + m - 1) / m, read, st, launch, rows));
+    return LBM_OK;
 }
 
 // FP32 -> FP64 widening straight into mapped host memory (over the
@@ -615,15 +661,16 @@ __global__ void k_widen(const float *__restrict__ s, double *__restrict__ d, int
 
 // `fields` FP32 fields of N values each (device, contiguous) to host doubles,
 // dst[k] == NULL skipped; complete when it returns.
-//  - Page-locked destinations, and pageable ones of at least kWideLock bytes
-//    (locked for the call), are widened into by the device: 151 MB of fresh
-//    pages 4 ms, where a copy and a host loop took 13.
+//  - Page-locked destinations are widened into by the device.
+//  - Pageable ones of at least kWideStage bytes are widened by the device into
+//    the thread's page-locked slots and copied from there by several threads, which
+//    fault in fresh pages side by side.
 //  - Smaller pageable ones are widened on the host, through a scratch buffer
 //    that the thread keeps (kScratch values, freed when the thread ends): most
 //    of their time goes into the destination's fresh pages, which the host
 //    faults in 9 times faster than a copy or a kernel does, and a fresh
 //    scratch buffer would add as many again.
-static constexpr size_t kWideLock = (size_t)8 << 20;
+static constexpr size_t kWideStage = (size_t)8 << 20;
 static constexpr int64_t kScratch = 1 << 18;
 // Up to here a field takes the host's loop whatever its memory: asking what the
 // memory is costs 0.4 us, a launch more than the loop.
@@ -650,16 +697,36 @@ lbm_status lbm_fields_to_host(const double *src, int64_t N, int fields, double *
 }
 
 lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *const *dst, cudaStream_t st) {
-    HostView views[4];
+    const size_t bytes = (size_t)N * sizeof(double);
     bool small[4] = {false, false, false, false};
+    int staged[4], nstaged = 0;
+    char *slots = nullptr;
+    auto widen = [src, N, st](int field, int64_t v, int64_t n, double *to) {
+        const int blocks = (int)std::min<int64_t>(kWidenBlocks, (n + 255) / 256);
+        k_widen<<<blocks, 256, 0, st>>>(src + (size_t)field * N + v, to, n);
+        return cudaGetLastError();
+    };
     for (int k = 0; k < fields; ++k) {
         if (!dst[k]) continue;
-        const size_t bytes = (size_t)N * sizeof(double);
-        if (bytes >= kWideLock || (bytes > kSmallField && mapped_host(dst[k]))) views[k].open(dst[k], bytes, true);
-        small[k] = !views[k].ok();
-        if (small[k]) continue;
-        k_widen<<<kWidenBlocks, 256, 0, st>>>(src + (size_t)k * N, (double *)views[k].dev(), N);
-        CK(cudaGetLastError());
+        if (double *d = bytes > kSmallField ? (double *)mapped_host(dst[k], bytes) : nullptr) {
+            CK(widen(k, 0, N, d));
+        } else if (bytes >= kWideStage && (slots || (slots = stage_slots()))) {
+            staged[nstaged++] = k;
+        } else {
+            small[k] = true;
+        }
+    }
+    if (nstaged) {
+        const int64_t m = (int64_t)(chunk_bytes(nstaged * bytes) / sizeof(double)), per = (N + m - 1) / m;   // values, chunks a field
+        auto launch = [&](int64_t c, char *slot) {
+            const int64_t v = c % per * m;
+            return widen(staged[c / per], v, std::min(m, N - v), (double *)slot);
+        };
+        auto rows = [&](int64_t c, char *slot, auto f) {
+            const int64_t v = c % per * m;
+            f((char *)(dst[staged[c / per]] + v), slot, (size_t)std::min(m, N - v) * sizeof(double));
+        };
+        CK(run_staged(slots, nstaged * per, true, st, launch, rows));
     }
     // consecutive small fields are one range of values: chunks of it, copied and widened
     for (int k = 0; k < fields; ++k) {
@@ -683,7 +750,7 @@ lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *co
         }
         k = e - 1;
     }
-    CK(cudaStreamSynchronize(st));   // before the views let go of their pages
+    CK(cudaStreamSynchronize(st));
     return LBM_OK;
 }
 
@@ -776,21 +843,18 @@ static void raw_set(unsigned char *raw, int storage, int64_t k, double v) {
     }
 }
 
-lbm_status lbm_pops_to_host(const unsigned char *raw, int storage, int layout, int rev, int64_t N, void *host,
-                            int32_t as) {
-    for (int i = 0; i < 9; ++i) {
-        const int slot = rev ? 8 - i : i;
-        parallel_for(N, [=](int64_t b, int64_t e) {
-            for (int64_t n = b; n < e; ++n) {
-                const double v = raw_get(raw, storage, layout_addr(layout, N, n, slot));
-                if (as == LBM_F64)
-                    ((double *)host)[(int64_t)i * N + n] = v;
-                else
-                    ((float *)host)[(int64_t)i * N + n] = (float)v;
-            }
-        });
-    }
-    return LBM_OK;
+static lbm_status transfer_state(lbm_lattice *L, void *host, int32_t as, bool read, bool *done) {
+    struct Ctx {
+        lbm_lattice *L;
+        bool f64, read;
+    } ctx{L, as == LBM_F64, read};
+    auto move = [](void *c, void *rows, int64_t n0, int64_t count, int64_t stride) {
+        const Ctx &x = *(const Ctx *)c;
+        const lbm_lattice *l = x.L;
+        return x.read ? l->ops->export_state(l->h, l->cur, rows, x.f64, n0, count, stride, l->stream)
+                      : l->ops->import_state(l->h, l->cur, rows, x.f64, n0, count, stride, l->stream);
+    };
+    return lbm_transfer_state(9, L->pl.N, as == LBM_F64 ? 8 : 4, host, read, L->stream, move, &ctx, done);
 }
 
 extern "C" lbm_status lbm_read_populations(lbm_lattice *L, void *host, int32_t as) {
@@ -798,19 +862,20 @@ extern "C" lbm_status lbm_read_populations(lbm_lattice *L, void *host, int32_t a
     if (aa_state_readable(L) != LBM_OK) return LBM_EINVAL;
     if (as != LBM_F64 && as != LBM_F32) return lbm_fail(LBM_EINVAL, "as must be LBM_F64 or LBM_F32");
     const int64_t N = L->pl.N;
-    {
-        HostView v(host, 9 * (size_t)N * (as == LBM_F64 ? 8 : 4), true);
-        if (v.ok()) {
-            CK(L->ops->export_state(L->h, L->cur, v.dev(), as == LBM_F64, L->stream));
-            CK(cudaStreamSynchronize(L->stream));
-            return check_err(L);
-        }
-    }
+    bool done;
+    const lbm_status s = transfer_state(L, host, as, true, &done);
+    if (s != LBM_OK) return s;
+    if (done) return check_err(L);
     std::vector<unsigned char> raw(9 * (size_t)N * L->ops->elem);
     CK(cudaStreamSynchronize(L->stream));
     CK(cudaMemcpy(raw.data(), L->h.pop[L->cur], raw.size(), cudaMemcpyDeviceToHost));
-    lbm_pops_to_host(raw.data(), L->p.storage, L->p.layout, L->p.algo == LBM_NSOL || L->p.algo == LBM_AA, N,
-                     host, as);
+    const int rev = L->p.algo == LBM_NSOL || L->p.algo == LBM_AA;
+    for (int i = 0; i < 9; ++i)
+        for (int64_t n = 0; n < N; ++n) {
+            const double v = raw_get(raw.data(), L->p.storage, layout_addr(L->p.layout, N, n, rev ? 8 - i : i));
+            if (as == LBM_F64) ((double *)host)[(int64_t)i * N + n] = v;
+            else ((float *)host)[(int64_t)i * N + n] = (float)v;
+        }
     return check_err(L);
 }
 
@@ -819,32 +884,22 @@ extern "C" lbm_status lbm_write_populations(lbm_lattice *L, const void *host, in
     if (aa_state_readable(L) != LBM_OK) return LBM_EINVAL;
     if (as != LBM_F64 && as != LBM_F32) return lbm_fail(LBM_EINVAL, "as must be LBM_F64 or LBM_F32");
     const int64_t N = L->pl.N;
-    {
-        HostView v((void *)host, 9 * (size_t)N * (as == LBM_F64 ? 8 : 4), false);
-        if (v.ok()) {
-            CK(L->ops->import_state(L->h, L->cur, v.dev(), as == LBM_F64, L->stream));
-            if (L->pl.halo_grid) CK(L->ops->publish(L->h, L->cur, (int)(L->steps & 1), L->stream));
-            CK(cudaStreamSynchronize(L->stream));
-            return LBM_OK;
-        }
-    }
-    std::vector<unsigned char> raw(9 * (size_t)N * L->ops->elem);
-    const int rev = L->p.algo == LBM_NSOL || L->p.algo == LBM_AA;
-    unsigned char *rawp = raw.data();
-    const int storage = L->p.storage, layout = L->p.layout;
-    for (int i = 0; i < 9; ++i) {
-        const int slot = rev ? 8 - i : i;
-        parallel_for(N, [=](int64_t b, int64_t e) {
-            for (int64_t n = b; n < e; ++n) {
+    bool done;
+    const lbm_status s = transfer_state(L, (void *)host, as, false, &done);
+    if (s != LBM_OK) return s;
+    if (!done) {
+        std::vector<unsigned char> raw(9 * (size_t)N * L->ops->elem);
+        const int rev = L->p.algo == LBM_NSOL || L->p.algo == LBM_AA;
+        for (int i = 0; i < 9; ++i)
+            for (int64_t n = 0; n < N; ++n) {
                 const double v = as == LBM_F64 ? ((const double *)host)[(int64_t)i * N + n]
                                                : (double)((const float *)host)[(int64_t)i * N + n];
-                raw_set(rawp, storage, layout_addr(layout, N, n, slot), v);
+                raw_set(raw.data(), L->p.storage, layout_addr(L->p.layout, N, n, rev ? 8 - i : i), v);
             }
-        });
+        CK(cudaStreamSynchronize(L->stream));
+        CK(cudaMemcpy(L->h.pop[L->cur], raw.data(), raw.size(), cudaMemcpyHostToDevice));
+        CK(L->ops->zero_solid(L->h, L->cur, L->stream));
     }
-    CK(cudaStreamSynchronize(L->stream));
-    CK(cudaMemcpy(L->h.pop[L->cur], raw.data(), raw.size(), cudaMemcpyHostToDevice));
-    CK(L->ops->zero_solid(L->h, L->cur, L->stream));
     if (L->pl.halo_grid) CK(L->ops->publish(L->h, L->cur, (int)(L->steps & 1), L->stream));
     CK(cudaStreamSynchronize(L->stream));
     return LBM_OK;

@@ -47,25 +47,15 @@ template <class P> inline bool lbm_draws(const P *p) {
     return p->rounding == LBM_ROUND_SR && (p->storage == LBM_F16S || p->storage == LBM_BF16S);
 }
 
-// Device address of a host buffer for the duration of one synchronous call:
-// page-locked memory as it is, pageable memory of at least kRegisterBytes
-// page-locked for the call (released by the destructor, after the caller has
-// waited for its kernels). ok() is false where neither works (small buffers,
-// memory that cannot be locked): the caller then copies through the host.
-class HostView {
-  public:
-    HostView() = default;
-    HostView(void *p, size_t bytes, bool write) { open(p, bytes, write); }
-    ~HostView();
-    void open(void *p, size_t bytes, bool write);   // once
-    HostView(const HostView &) = delete;
-    HostView &operator=(const HostView &) = delete;
-    bool ok() const { return dev_ != nullptr; }
-    void *dev() const { return dev_; }
-
-  private:
-    void *dev_ = nullptr, *locked_ = nullptr;
-};
+// The state of N nodes, q populations each in canonical order host[i N + n] of
+// es-byte values, to (`read`) or from host memory, complete when it returns:
+// `move` enqueues the conversion of nodes n0 .. n0 + count - 1 into / out of
+// rows[i stride + n - n0], device-accessible host memory. *done is false, and
+// nothing has happened, where the caller has to copy and convert on the host: up
+// to 1 MB of pageable memory, or no page-locked memory to be had (lbm_capi.cu).
+using MoveState = cudaError_t (*)(void *ctx, void *rows, int64_t n0, int64_t count, int64_t stride);
+lbm_status lbm_transfer_state(int q, int64_t N, size_t es, void *host, bool read, cudaStream_t st, MoveState move,
+                              void *ctx, bool *done);
 
 // Up to four moments fields on the device, FP64 or FP32, to host doubles (lbm_capi.cu).
 lbm_status lbm_fields_to_host(const double *src, int64_t N, int fields, double *const *dst, cudaStream_t st);
@@ -83,5 +73,3 @@ lbm_status lbm_plan(const lbm_params *p, Plan *pl);
 const lbm::Ops *ops_for_storage(int storage);
 void lbm_fill_args(const lbm_params *p, const Plan &pl, char *ws, const lbm::Ops *ops, lbm::HostArgs *h);
 int64_t layout_addr(int layout, int64_t N, int64_t n, int i);
-lbm_status lbm_pops_to_host(const unsigned char *raw, int storage, int layout, int rev, int64_t N,
-                            void *host, int32_t as);

@@ -93,9 +93,12 @@ struct Ops {
     cudaError_t (*publish)(const HostArgs &, int src, int parity, cudaStream_t);
     // Store h = 0 at every solid node of lattice `src`.
     cudaError_t (*zero_solid)(const HostArgs &, int src, cudaStream_t);
-    // Lattice src / dst to / from canonical order in mapped host memory (doubles or floats).
-    cudaError_t (*export_state)(const HostArgs &, int src, void *out, bool f64, cudaStream_t);
-    cudaError_t (*import_state)(const HostArgs &, int dst, const void *in, bool f64, cudaStream_t);
+    // Nodes n0 .. n0 + count - 1 of lattice src / dst to / from rows[i stride + n - n0] in mapped
+    // host memory (doubles or floats).
+    cudaError_t (*export_state)(const HostArgs &, int src, void *rows, bool f64, int64_t n0, int64_t count,
+                                int64_t stride, cudaStream_t);
+    cudaError_t (*import_state)(const HostArgs &, int dst, const void *rows, bool f64, int64_t n0, int64_t count,
+                                int64_t stride, cudaStream_t);
     // rho = 1 + sum h, v = sum h c (- F/2 if post_collision) into mom.
     cudaError_t (*state_moments)(const HostArgs &, int src, int post_collision, cudaStream_t);
     // FP64 block partial sums: mass (1 value) or force (2 values) per block.

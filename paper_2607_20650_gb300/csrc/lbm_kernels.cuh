@@ -1647,28 +1647,30 @@ __global__ void k_publish(const Step<S> a, S *hw, int rev) {
     halo_publish(a, hw, bx, by, x, y, x0, y0, x1, y1, e);
 }
 
-// The stored state to / from canonical order h[i N + n] in (page-locked, mapped)
-// host memory, H = double or float; rev: populations are stored in opposite
-// slots. The host side of the copy is the coalesced one, and it alone bounds
-// these kernels (the CPU-GPU link). FP32 state to doubles and back, 2M nodes
-// (151 MB on the host): 1.1 ms each, where copies and conversion loops on the
-// host took 23 ms. Solid nodes are stored as zeros.
+// Nodes n0 .. n0 + count - 1 of the stored state to / from rows of canonical
+// order, rows[i stride + n - n0], in page-locked, mapped host memory; H = double or
+// float; rev: populations are stored in opposite slots. The host side of the copy
+// is the coalesced one, and it alone bounds these kernels (the CPU-GPU link).
+// Solid nodes are stored as zeros.
 template <class S, int L, class H>
-__global__ void __launch_bounds__(256) k_export(const S *lat, uint32_t N, int rev, H *out) {
-    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+__global__ void __launch_bounds__(256) k_export(const S *lat, uint32_t N, int rev, H *rows, uint32_t n0,
+                                                uint32_t count, size_t stride) {
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= count) return;
 #pragma unroll
-    for (int i = 0; i < 9; ++i) out[(size_t)i * N + n] = (H)ldp<S, L>(lat, N, n, rev ? opp(i) : i);
+    for (int i = 0; i < 9; ++i) rows[i * stride + k] = (H)ldp<S, L>(lat, N, n0 + k, rev ? opp(i) : i);
 }
 template <class S, int L, class H>
-__global__ void __launch_bounds__(256) k_import(S *lat, const uint8_t *links, uint32_t N, int rev, const H *in) {
+__global__ void __launch_bounds__(256) k_import(S *lat, const uint8_t *links, uint32_t N, int rev, const H *rows,
+                                                uint32_t n0, uint32_t count, size_t stride) {
     using C = typename Codec<S>::C;
-    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+    const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= count) return;
+    const uint32_t n = n0 + k;
     const bool solid = links[n] == SOLID_LINKS;
 #pragma unroll
     for (int i = 0; i < 9; ++i)
-        lat[addr<L>(N, n, rev ? opp(i) : i)] = Codec<S>::enc(solid ? C(0) : (C)in[(size_t)i * N + n], false, 0u);
+        lat[addr<L>(N, n, rev ? opp(i) : i)] = Codec<S>::enc(solid ? C(0) : (C)rows[i * stride + k], false, 0u);
 }
 
 // Moments from a stored state: rho = 1 + sum h, v = sum h c (- F/2 for a
@@ -1946,23 +1948,27 @@ cudaError_t op_zero_solid(const HostArgs &h, int src, cudaStream_t st) {
 
 // f64: the host values are doubles, else floats.
 template <class S>
-cudaError_t op_export(const HostArgs &h, int src, void *out, bool f64, cudaStream_t st) {
-    const unsigned g = (unsigned)((h.N + 255) / 256);
+cudaError_t op_export(const HostArgs &h, int src, void *rows, bool f64, int64_t n0, int64_t count, int64_t stride,
+                      cudaStream_t st) {
+    const unsigned g = (unsigned)((count + 255) / 256);
+    const uint32_t N = (uint32_t)h.N, b = (uint32_t)n0, c = (uint32_t)count;
     const int rev = h.algo == NSOL || h.algo == AA;
     const S *lat = (const S *)h.pop[src];
-    LBM_LAYOUT_SWITCH(h, (f64 ? k_export<S, L_, double><<<g, 256, 0, st>>>(lat, (uint32_t)h.N, rev, (double *)out)
-                              : k_export<S, L_, float><<<g, 256, 0, st>>>(lat, (uint32_t)h.N, rev, (float *)out)));
+    LBM_LAYOUT_SWITCH(h, (f64 ? k_export<S, L_, double><<<g, 256, 0, st>>>(lat, N, rev, (double *)rows, b, c, stride)
+                              : k_export<S, L_, float><<<g, 256, 0, st>>>(lat, N, rev, (float *)rows, b, c, stride)));
     return cudaGetLastError();
 }
 
 template <class S>
-cudaError_t op_import(const HostArgs &h, int dst, const void *in, bool f64, cudaStream_t st) {
-    const unsigned g = (unsigned)((h.N + 255) / 256);
+cudaError_t op_import(const HostArgs &h, int dst, const void *rows, bool f64, int64_t n0, int64_t count,
+                      int64_t stride, cudaStream_t st) {
+    const unsigned g = (unsigned)((count + 255) / 256);
+    const uint32_t N = (uint32_t)h.N, b = (uint32_t)n0, c = (uint32_t)count;
     const int rev = h.algo == NSOL || h.algo == AA;
     S *lat = (S *)h.pop[dst];
     LBM_LAYOUT_SWITCH(
-        h, (f64 ? k_import<S, L_, double><<<g, 256, 0, st>>>(lat, h.links, (uint32_t)h.N, rev, (const double *)in)
-                : k_import<S, L_, float><<<g, 256, 0, st>>>(lat, h.links, (uint32_t)h.N, rev, (const float *)in)));
+        h, (f64 ? k_import<S, L_, double><<<g, 256, 0, st>>>(lat, h.links, N, rev, (const double *)rows, b, c, stride)
+                : k_import<S, L_, float><<<g, 256, 0, st>>>(lat, h.links, N, rev, (const float *)rows, b, c, stride)));
     return cudaGetLastError();
 }
 
