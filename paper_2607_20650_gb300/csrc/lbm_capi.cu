@@ -685,61 +685,63 @@ static float *host_scratch() {
 // The same for FP64 fields. Few values go through the thread's scratch buffer
 // in one copy, as above; a copy per field straight to the caller's fresh pages
 // took 53 instead of 35 us for the four fields of a box of 4,000 nodes.
+// (Whatever fails, these two return only when nothing writes to dst any more.)
 lbm_status lbm_fields_to_host(const double *src, int64_t N, int fields, double *const *dst, cudaStream_t st) {
-    double *f = (size_t)fields * N * sizeof(double) <= kScratch * sizeof(float) ? (double *)host_scratch() : nullptr;
-    if (f) CK(cudaMemcpyAsync(f, src, (size_t)fields * N * sizeof(double), cudaMemcpyDeviceToHost, st));
-    for (int k = 0; k < fields && !f; ++k)
-        if (dst[k]) CK(cudaMemcpyAsync(dst[k], src + (size_t)k * N, (size_t)N * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+    const size_t bytes = (size_t)N * sizeof(double);
+    double *f = fields * bytes <= kScratch * sizeof(float) ? (double *)host_scratch() : nullptr;
+    cudaError_t e = f ? cudaMemcpyAsync(f, src, fields * bytes, cudaMemcpyDeviceToHost, st) : cudaSuccess;
+    for (int k = 0; k < fields && !f && e == cudaSuccess; ++k)
+        if (dst[k]) e = cudaMemcpyAsync(dst[k], src + (size_t)k * N, bytes, cudaMemcpyDeviceToHost, st);
+    const cudaError_t done = cudaStreamSynchronize(st);
+    CK(e);
+    CK(done);
     for (int k = 0; k < fields && f; ++k)
-        if (dst[k]) memcpy(dst[k], f + (size_t)k * N, (size_t)N * sizeof(double));
+        if (dst[k]) memcpy(dst[k], f + (size_t)k * N, bytes);
     return LBM_OK;
 }
 
 lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *const *dst, cudaStream_t st) {
     const size_t bytes = (size_t)N * sizeof(double);
+    // every field's route, and the memory it needs, before the first launch
+    double *direct[4] = {nullptr, nullptr, nullptr, nullptr};
     bool small[4] = {false, false, false, false};
     int staged[4], nstaged = 0;
     char *slots = nullptr;
+    float *f = nullptr;
+    for (int k = 0; k < fields; ++k) {
+        if (!dst[k]) continue;
+        if (bytes > kSmallField && (direct[k] = (double *)mapped_host(dst[k], bytes))) continue;
+        if (bytes >= kWideStage && (slots || (slots = stage_slots()))) {
+            staged[nstaged++] = k;
+        } else {
+            small[k] = true;
+            if (!f && !(f = host_scratch())) return lbm_fail(LBM_ENOMEM, "host allocation failed");
+        }
+    }
     auto widen = [src, N, st](int field, int64_t v, int64_t n, double *to) {
         const int blocks = (int)std::min<int64_t>(kWidenBlocks, (n + 255) / 256);
         k_widen<<<blocks, 256, 0, st>>>(src + (size_t)field * N + v, to, n);
         return cudaGetLastError();
     };
-    for (int k = 0; k < fields; ++k) {
-        if (!dst[k]) continue;
-        if (double *d = bytes > kSmallField ? (double *)mapped_host(dst[k], bytes) : nullptr) {
-            CK(widen(k, 0, N, d));
-        } else if (bytes >= kWideStage && (slots || (slots = stage_slots()))) {
-            staged[nstaged++] = k;
-        } else {
-            small[k] = true;
-        }
-    }
-    if (nstaged) {
+    auto through_slots = [&]() {
         const int64_t m = (int64_t)(chunk_bytes(nstaged * bytes) / sizeof(double)), per = (N + m - 1) / m;   // values, chunks a field
         auto launch = [&](int64_t c, char *slot) {
             const int64_t v = c % per * m;
             return widen(staged[c / per], v, std::min(m, N - v), (double *)slot);
         };
-        auto rows = [&](int64_t c, char *slot, auto f) {
+        auto rows = [&](int64_t c, char *slot, auto copy) {
             const int64_t v = c % per * m;
-            f((char *)(dst[staged[c / per]] + v), slot, (size_t)std::min(m, N - v) * sizeof(double));
+            copy((char *)(dst[staged[c / per]] + v), slot, (size_t)std::min(m, N - v) * sizeof(double));
         };
-        CK(run_staged(slots, nstaged * per, true, st, launch, rows));
-    }
-    // consecutive small fields are one range of values: chunks of it, copied and widened
-    for (int k = 0; k < fields; ++k) {
-        if (!small[k]) continue;
-        int e = k;
-        while (e < fields && small[e]) ++e;
-        float *f = host_scratch();
-        if (!f) return lbm_fail(LBM_ENOMEM, "host allocation failed");
-        const int64_t end = (int64_t)e * N;
-        for (int64_t v = (int64_t)k * N; v < end;) {
+        return run_staged(slots, nstaged * per, true, st, launch, rows);
+    };
+    // values v .. end - 1 of consecutive small fields: chunks, copied and widened
+    auto through_scratch = [&](int64_t v, int64_t end) {
+        while (v < end) {
             const int64_t c = std::min(kScratch, end - v);
-            CK(cudaMemcpyAsync(f, src + v, (size_t)c * sizeof(float), cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
+            cudaError_t e = cudaMemcpyAsync(f, src + v, (size_t)c * sizeof(float), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return e;
             for (int64_t done = 0; done < c;) {
                 const int64_t at = v + done, field = at / N, n = at - field * N, m = std::min(c - done, N - n);
                 double *d = dst[field] + n;
@@ -748,9 +750,21 @@ lbm_status lbm_widen_to_host(const float *src, int64_t N, int fields, double *co
             }
             v += c;
         }
-        k = e - 1;
+        return cudaSuccess;
+    };
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < fields && e == cudaSuccess; ++k)
+        if (direct[k]) e = widen(k, 0, N, direct[k]);
+    if (nstaged && e == cudaSuccess) e = through_slots();
+    for (int k = 0; k < fields && e == cudaSuccess; ++k) {
+        if (!small[k]) continue;
+        const int64_t first = k;
+        while (k < fields && small[k]) ++k;
+        e = through_scratch(first * N, (int64_t)k * N);
     }
-    CK(cudaStreamSynchronize(st));
+    const cudaError_t done = cudaStreamSynchronize(st);
+    CK(e);
+    CK(done);
     return LBM_OK;
 }
 

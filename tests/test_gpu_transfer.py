@@ -138,3 +138,37 @@ def test_moments_into_locked_memory_around_64_kb(N, storage):
     assert lbm.load().lbm_read_moments(lat.h, *(g.ctypes.data for g in got)) == 0
     for a, b in zip(got, want):
         assert np.array_equal(a, b)
+
+
+def test_a_failed_read_writes_nothing():
+    """Without host memory for the pageable field, the page-locked one is not written either,
+    then or later. A process of its own, whose address space may not grow during the call."""
+    import os
+    import subprocess
+    import sys
+    code = """
+import resource, numpy as np, torch
+from paper_2607_20650_gb300 import lbm
+lib = lbm.load()
+N = 1 << 19
+ux = np.full(N, 1e-2)
+lat = lbm.Lattice(N, 1, 0.8, storage="f32").init(1 + ux, ux, ux)
+rho = torch.full((N,), -1.0, dtype=torch.float64, pin_memory=True).numpy()
+uxo = np.full(N, -1.0)
+a, b = rho.ctypes.data, uxo.ctypes.data
+torch.cuda.synchronize()
+size = [int(l.split()[1]) << 10 for l in open("/proc/self/status") if l.startswith("VmSize")][0]
+old = resource.getrlimit(resource.RLIMIT_AS)
+resource.setrlimit(resource.RLIMIT_AS, (size, old[1]))
+s = lib.lbm_read_moments(lat.h, a, b, None)
+resource.setrlimit(resource.RLIMIT_AS, old)
+torch.cuda.synchronize()
+assert s == 2, s                                # LBM_ENOMEM
+assert (rho == -1.0).all() and (uxo == -1.0).all()
+assert lib.lbm_read_moments(lat.h, a, b, None) == 0
+assert abs(rho - 1.01).max() < 1e-5 and abs(uxo - 1e-2).max() < 1e-5
+"""
+    env = dict(os.environ, GLIBC_TUNABLES="glibc.malloc.mmap_threshold=65536")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
