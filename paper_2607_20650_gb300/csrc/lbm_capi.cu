@@ -542,10 +542,32 @@ static void *mapped_host(const void *p) {
     }
     return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
 }
-// The same for `bytes` bytes.
+// The same for `bytes` bytes from p on, if one allocation or registration holds
+// them all. (Page-locked first and last bytes do not show that: a program may
+// have locked two pieces of an array. The runtime has no query for the range;
+// the CUDA driver's is reached through it.)
 static void *mapped_host(const void *p, size_t bytes) {
-    char *d = (char *)mapped_host(p);
-    return d && (char *)mapped_host((const char *)p + (bytes - 1)) == d + (bytes - 1) ? d : nullptr;
+    using Query = CUresult (*)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+    static Query query = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            (void)cudaGetLastError();
+            fn = nullptr;
+        }
+        return (Query)fn;
+    }();
+    void *d = mapped_host(p);
+    if (!d || !query) return nullptr;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[2] = {&start, &size};
+    if (query(2, what, to, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) return nullptr;
+    const uint64_t at = (uint64_t)(uintptr_t)p - start;
+    return (uint64_t)(uintptr_t)p >= start && at <= size && bytes <= size - at ? d : nullptr;
 }
 
 // Page-locked slots of the calling thread (32 MB in all), allocated by its first

@@ -115,3 +115,53 @@ def test_memory_mapped_files(tmp_path, nx, ny):
     assert lbm.load().lbm_read_moments(lat.h, *(m.ctypes.data for m in mom)) == 0
     for a, b in zip(mom, want):
         assert np.array_equal(a, b.reshape(-1))
+
+
+def _lock(address, nbytes):
+    assert int(torch.cuda.cudart().cudaHostRegister(address, nbytes, 0)) == 0
+
+
+def _unlock(address):
+    assert int(torch.cuda.cudart().cudaHostUnregister(address)) == 0
+
+
+@pytest.mark.parametrize("pieces", [((0, 1), (-1, 1)), ((0, 8), (-8, 8)), ((0, 4),), ((-4, 4),), ((3, 5),), ((0, 16),)],
+                         ids=["ends", "half and half", "head", "tail", "middle", "whole"])
+def test_arrays_locked_in_pieces(pieces):
+    """The caller has page-locked pieces (in sixteenths) of the arrays that state and moments go to."""
+    h = _state(5)
+    src = h.copy()
+    out = np.full((9, N), -1.0)
+    mom = np.full((3, 1 << 21), -1.0)
+    lat = lbm.Lattice(NX, NY, 0.8, storage="f32")
+    r = np.random.default_rng(6)
+    ux = 1e-2 * r.standard_normal(mom.shape[1])
+    strip = lbm.Lattice(mom.shape[1], 1, 0.8, storage="f32").init(1 + ux, ux, ux)
+    want = [np.array(f).reshape(-1) for f in strip.moments()]
+    locked = []
+    for a in (src, out, mom[1]):
+        unit = a.nbytes // 16 // 65536 * 65536   # whole pages, not a page in two pieces
+        base = (a.ctypes.data + 65535) // 65536 * 65536
+        for first, count in pieces:
+            if count == 16:
+                start, nbytes = a.ctypes.data, a.nbytes
+            elif first == 0:
+                start, nbytes = a.ctypes.data, base - a.ctypes.data + count * unit
+            elif first < 0:
+                start = base + (16 + first) * unit
+                nbytes = a.ctypes.data + a.nbytes - start
+            else:
+                start, nbytes = base + first * unit, count * unit
+            _lock(start, nbytes)
+            locked.append(start)
+    try:
+        lib = lbm.load()
+        assert lib.lbm_write_populations(lat.h, src.ctypes.data, 0) == 0
+        assert lib.lbm_read_populations(lat.h, out.ctypes.data, 0) == 0
+        assert lib.lbm_read_moments(strip.h, *(m.ctypes.data for m in mom)) == 0
+    finally:
+        for a in locked:
+            _unlock(a)
+    assert np.array_equal(out, h)
+    for a, b in zip(mom, want):
+        assert np.array_equal(a, b)
