@@ -609,7 +609,7 @@ struct Halo3 {
     int yl, yh, zl, zh;    // shift of y (z) by a pull with c > 0 / c < 0, periodic
     int nx, ny;
 
-    __device__ __forceinline__ Halo3(const Geo3 &g, const int *nt, const int *b, const int *p, const int *tlo,
+    __host__ __device__ __forceinline__ Halo3(const Geo3 &g, const int *nt, const int *b, const int *p, const int *tlo,
                                      const int *thi) {
         nx = g.nx;
         ny = g.ny;
@@ -637,28 +637,29 @@ struct Halo3 {
         zh = p[2] == g.nz - 1 ? 1 - g.nz : 1;
     }
     // Does the pull of direction i leave the tile along axis a?
-    __device__ __forceinline__ bool crosses(int i, int a) const {
+    __host__ __device__ __forceinline__ bool crosses(int i, int a) const {
         const int c = a == 0 ? cx(i) : (a == 1 ? cy(i) : cz(i));
         return c > 0 ? lo[a] : (c < 0 ? hi[a] : false);
     }
-    // Element that the pull of direction i, which leaves the tile, reads.
-    __device__ __forceinline__ I at(int i) const {
+    // Element that the pull of direction i, which leaves the tile, reads. (dz reaches
+    // nz - 1 where a pull wraps: its products need the grid's width.)
+    __host__ __device__ __forceinline__ I at(int i) const {
         const int dy = cy(i) > 0 ? yl : (cy(i) < 0 ? yh : 0), dz = cz(i) > 0 ? zl : (cz(i) < 0 ? zh : 0);
         I r = 0;
         if (cz(i)) r = Z + (cz(i) > 0 ? zb : zf) + (I)((cz(i) < 0 ? 5 : 0) + face_rank(i, 2)) * pz - (I)(cx(i) + cy(i) * nx);
         if (cy(i)) {
-            const I v = Y + (cy(i) > 0 ? yb : yf) + (I)((cy(i) < 0 ? 5 : 0) + face_rank(i, 1)) * py + (I)(dz * nx - cx(i));
+            const I v = Y + (cy(i) > 0 ? yb : yf) + (I)((cy(i) < 0 ? 5 : 0) + face_rank(i, 1)) * py + (I)dz * (I)nx - (I)cx(i);
             r = !cz(i) || crosses(i, 1) ? v : r;
         }
         if (cx(i)) {
-            const I v = X + (cx(i) > 0 ? xb : xf) + (I)((cx(i) < 0 ? 5 : 0) + face_rank(i, 0)) * px + (I)(dy + dz * ny);
+            const I v = X + (cx(i) > 0 ? xb : xf) + (I)((cx(i) < 0 ? 5 : 0) + face_rank(i, 0)) * px + (I)dy + (I)dz * (I)ny;
             r = !(cy(i) || cz(i)) || crosses(i, 0) ? v : r;
         }
         return r;
     }
     // Publish the outgoing populations e (canonical order) of the node.
     template <class S>
-    __device__ __forceinline__ void publish(S *hw, const S *e) const {
+    __host__ __device__ __forceinline__ void publish(S *hw, const S *e) const {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const I base = a == 0 ? X : (a == 1 ? Y : Z), plane = a == 0 ? px : (a == 1 ? py : pz);
