@@ -242,6 +242,7 @@ extern "C" lbm_status lbm3_create(const lbm3_params *p, const uint8_t *mask_host
     L->stream = (cudaStream_t)cuda_stream;
     L->ops = ops3_for(p->storage);
     L->block_1d = L->ops->block_1d(p->layout);
+    L->sms = lbm::device_size().sms;
     L->ops->prepare(p->algo);
     L->off32 = (lbm3_offsets_fit(p, pl.N) && !(p->flags & LBM_FLAG_WIDE_OFFSETS)) ? 1 : 0;
     L->err = (unsigned int *)(L->ws + pl.misc);

@@ -90,6 +90,7 @@ struct lbm3_batch {
     cudaStream_t stream, cap;
     unsigned int *err;
     long long *tctr;
+    int sms;       // SMs of the device
     bool draws;    // some box uses stochastic rounding (the update counter's only reader)
     int cur;
     int64_t steps;
@@ -135,6 +136,7 @@ extern "C" lbm_status lbm3_batch_create(int32_t ncases, const lbm3_params *param
     B->ncases = ncases;
     B->p0 = params[0];
     B->ops = ops3_for(params[0].storage);
+    B->sms = lbm::device_size().sms;
     for (int c = 0; c < ncases; ++c) B->draws = B->draws || lbm_draws(&params[c]);
     B->ws = (char *)d_workspace;
     B->stream = (cudaStream_t)cuda_stream;
@@ -201,6 +203,7 @@ static cudaError_t batch3_block(lbm3_batch *B, cudaStream_t st, int64_t count, i
     b.ty = B->bl.plans[0].ty;
     b.tz = B->bl.plans[0].tz;
     b.block_1d = kBatch3Nodes;
+    b.sms = B->sms;
     int cur = B->cur;
     for (int64_t k = 0; k < count; ++k) {
         b.src = cur;

@@ -32,6 +32,7 @@ struct lbm3_lattice {
     int64_t steps;
     int64_t fluid;
     int block_1d;
+    int sms;              // SMs of the device
     int off32;            // 32-bit offset tables usable (19 N and the pull shifts fit 31 bits)
     unsigned int *err;    // divergence flag (the box's own, or its batch's)
     long long *tctr;      // update counter: stochastic-rounding keys (the box's own, or its batch's)
@@ -44,7 +45,7 @@ struct Batch3Launch {
     const void *cases;
     const void *items;    // (case, local item) pairs of uint32
     uint32_t nitems;
-    int tx, ty, tz, block_1d;
+    int tx, ty, tz, block_1d, sms;
     int src, toff, mom;
 };
 

@@ -97,7 +97,7 @@ bool pairs3_ok(const lbm3_lattice *L) {
 
 template <class S>
 bool chained3(const lbm3_lattice *L, dim3 grid, dim3 block) {
-    return chained_updates(sizeof(S), L->pl.N) && spread_evenly(grid, block);
+    return chained_updates(sizeof(S), L->pl.N) && spread_evenly(grid, block, L->sms);
 }
 
 template <class S, bool LINEAR>
@@ -335,7 +335,7 @@ void batch_k(const Batch3Launch &b, cudaStream_t st) {
     const size_t sm = ALGO == LBM_NSOL ? nsol3_smem_bytes<S>(b.tx, b.ty, b.tz) : 0;
     // (100 updates and the read-out of 48 boxes of edge 12-48: 11.3 ms chained, 11.7
     // not; 16 of edge 12-20, 200 blocks, 6.9 and 4.9 us an update)
-    const bool chain = sizeof(S) < 8 && spread_evenly(dim3(b.nitems), block);
+    const bool chain = sizeof(S) < 8 && spread_evenly(dim3(b.nitems), block, b.sms);
     launch_update(chain, k3_batch<S, L, ALGO, OFF32>, dim3(b.nitems), block, sm, st, (const Case3<S> *)b.cases,
                   (const uint2 *)b.items, b.src, b.toff, b.mom);
 }

@@ -195,9 +195,7 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
         if (params[c].layout * 4 + params[c].algo != B->kind) B->kind = -1;
     double lattices = 0.0;   // bytes of the source lattices
     for (int c = 0; c < ncases; ++c) lattices += 9.0 * (double)B->bl.plans[c].N * (double)B->ops->elem;
-    int dev = 0, l2 = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
-        (void)cudaGetLastError();
+    const int64_t l2 = device_size().l2;
     B->pf = l2 > 0 && lattices > (double)l2 && !(params[0].flags & LBM_FLAG_NO_PREFETCH) ? 1 : 0;
     const int g = B->ops->batch_grid(B->kind);
     B->grid = (int)std::max<int64_t>(1, std::min<int64_t>(g > 0 ? g : 152, B->bl.ntiles));

@@ -181,7 +181,8 @@ extern "C" lbm_status lbm_workspace_bytes(const lbm_params *p, size_t *bytes) {
 #ifndef LBM_PF_PAIRS
 #define LBM_PF_PAIRS 1
 #endif
-static uint32_t prefetch_distance(const lbm_params *p, int64_t N, size_t elem, int tile_x) {
+static uint32_t prefetch_distance(const lbm_params *p, int64_t N, size_t elem, int tile_x, const DeviceSize &dev,
+                                  bool beyond_l2) {
     if (p->flags & LBM_FLAG_NO_PREFETCH) return 0;
     // 16-bit storage: only the node-pair kernel (LPTL/NPTL, bundle layout,
     // nx even) prefetches; its distance counts pairs of nodes. Measured on
@@ -193,20 +194,12 @@ static uint32_t prefetch_distance(const lbm_params *p, int64_t N, size_t elem, i
     if (elem != 4 && !pairs) return 0;
     if (p->algo == LBM_NSOL || p->layout == LBM_LAYOUT_COLLISION) return 0;
     if (p->algo == LBM_NPOL && p->layout != LBM_LAYOUT_BUNDLE) return 0;
-    int dev = 0, sms = 0, threads = 0, l2 = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return 0;
-    }
-    if ((double)N * 9.0 * (double)elem <= (double)l2) return 0;
+    if (!beyond_l2) return 0;
 #ifndef LBM_PF_NUM
 #define LBM_PF_NUM 5
 #endif
     // pairs: LPTL distances count pairs (the kernel doubles them), NPTL rows
-    const int64_t nodes = (int64_t)sms * threads * LBM_PF_NUM / 4 * (pairs && p->algo == LBM_NPTL ? 2 : 1);
+    const int64_t nodes = (int64_t)dev.sms * dev.sm_threads * LBM_PF_NUM / 4 * (pairs && p->algo == LBM_NPTL ? 2 : 1);
     if (p->algo == LBM_LPTL) return nodes < N ? (uint32_t)nodes : 0;
     const int64_t rows = std::max<int64_t>(1, (nodes + p->nx / 2) / p->nx);
     return rows < p->ny ? (uint32_t)rows : 0;
@@ -294,17 +287,15 @@ void lbm_fill_args(const lbm_params *p, const Plan &pl, char *ws, const Ops *ops
     h->ntx = pl.ntx;
     h->nty = pl.nty;
     ops->prepare();
-    int dev = 0;
-    h->sms = 152;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        (void)cudaGetLastError();
+    const DeviceSize dev = device_size();
+    h->sms = dev.sms;
+    h->beyond_l2 = dev.l2 > 0 && 9 * pl.N * (int64_t)ops->elem > dev.l2;
     h->block_1d = p->algo == LBM_LPTL ? ops->lptl_block(p->layout) : 0;
     // a lattice of few blocks is cut into smaller ones that spread over all SMs
     while (h->block_1d > 64 && (pl.N + h->block_1d - 1) / h->block_1d < 4 * (int64_t)h->sms) h->block_1d /= 2;
     h->flags = p->flags;
     h->nx_magic = p->nx == 1 ? 0ull : (~0ull / (uint64_t)p->nx) + 1ull;
-    h->pf = prefetch_distance(p, pl.N, ops->elem, pl.tx);
+    h->pf = prefetch_distance(p, pl.N, ops->elem, pl.tx, dev, h->beyond_l2);
     h->links = (const uint8_t *)(ws + pl.links);
     h->pop[0] = ws + pl.pop[0];
     h->pop[1] = pl.two ? ws + pl.pop[1] : nullptr;

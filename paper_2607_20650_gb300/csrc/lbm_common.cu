@@ -91,6 +91,18 @@ cudaError_t launch_links(int nx, int ny, int bw, int be, int bs, int bn, const u
     return cudaGetLastError();
 }
 
+DeviceSize device_size() {
+    int dev = 0, sms = 0, threads = 0, l2 = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return {152, 0, 0};
+    }
+    return {sms, threads, l2};
+}
+
 cudaError_t launch_count_fluid(const uint8_t *links, int64_t N, unsigned long long *out,
                                cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), st);

@@ -24,14 +24,15 @@ struct alignas(64) TmaDesc {
 // 3.1 / 1.9, 3.8 / 2.6, 6.5 / 5.2.
 inline bool chained_updates(size_t elem, int64_t nodes) { return elem < 8 || nodes >= (int64_t)1 << 19; }
 // Nor are kernels with blocks of a tile's size, or of one node a thread in three
-// dimensions, while their blocks neither fill the SMs (152 of 1,536 threads) nor
-// leave most of them empty, for the same reason. D3Q19 FP32, us an update,
-// unchained / chained: NPOL 8 x 8 x 8, 30 x 28 x 33 nodes (80 blocks) 4.7 / 8.1, 48 x
-// 40 x 44 (180) 5.4 / 8.4, 64 x 64 x 64 (512) 11.1 / 10.7; LPTL (256 nodes a block)
-// 4.0 / 4.9, 5.9 / 6.5 and 8.9 / 8.4; 12 x 12 x 12 (7 blocks) 3.7 / 3.2.
-inline bool spread_evenly(dim3 grid, dim3 block) {
+// dimensions, while their blocks neither fill the device's SMs (1,536 threads each,
+// what these kernels keep resident at 40 registers) nor leave three quarters of
+// them empty, for the same reason. D3Q19 FP32 on 152 SMs, us an update, unchained /
+// chained: NPOL 8 x 8 x 8, 30 x 28 x 33 nodes (80 blocks) 4.7 / 8.1, 48 x 40 x 44 (180)
+// 5.4 / 8.4, 64 x 64 x 64 (512) 11.1 / 10.7; LPTL (256 nodes a block) 4.0 / 4.9,
+// 5.9 / 6.5 and 8.9 / 8.4; 12 x 12 x 12 (7 blocks) 3.7 / 3.2.
+inline bool spread_evenly(dim3 grid, dim3 block, int sms) {
     const int64_t blocks = (int64_t)grid.x * grid.y * grid.z;
-    return blocks * block.x * block.y * block.z >= 152 * 1536 || blocks <= 152 / 4;
+    return blocks * block.x * block.y * block.z >= (int64_t)sms * 1536 || blocks <= sms / 4;
 }
 
 template <class... P, class... A>
@@ -50,6 +51,14 @@ inline cudaError_t launch_update(bool chained, void (*kernel)(P...), dim3 grid, 
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(a)...);
 }
 
+// What the launch rules ask of the current device (lbm_common.cu).
+struct DeviceSize {
+    int sms;          // 152 where there is no device to ask
+    int sm_threads;   // the same: 0
+    int64_t l2;       // bytes; the same: 0
+};
+DeviceSize device_size();
+
 // Everything a kernel launch needs, in host types.
 struct HostArgs {
     int nx, ny;
@@ -61,6 +70,7 @@ struct HostArgs {
     int tile_x, tile_y, ntx, nty;
     int block_1d;              // LPTL block size
     int sms;                   // SMs of the device
+    bool beyond_l2;            // a lattice's populations exceed the L2 cache
     uint32_t flags;            // lbm_params.flags
     uint64_t nx_magic;         // ceil(2^64 / nx) for n -> (x, y); 0 when nx == 1
     uint32_t pf;               // L2 prefetch distance: nodes (LPTL) or rows (NPTL); 0 = off

@@ -1832,7 +1832,7 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h)) {
                 const dim3 b(128), g((unsigned)((h.N / 2 + 127) / 128));
-                return launch_update(chain && spread_evenly(g, b), k_two_lattice_pair<S, L, true>, g, b, 0, st, a);
+                return launch_update(chain && spread_evenly(g, b, h.sms), k_two_lattice_pair<S, L, true>, g, b, 0, st, a);
             }
         }
         const int b = h.block_1d;
@@ -1843,10 +1843,10 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         }
         return launch_update(chain, k_two_lattice<S, L, true>, blocks, dim3(b), 0, st, a);
     }
-    const bool chain_tiles = chain && spread_evenly(grid, tile);
+    const bool chain_tiles = chain && spread_evenly(grid, tile, h.sms);
     if (h.algo == NPOL) {
         if constexpr (sizeof(S) == 4 && L != COLLISION) {
-            const bool large = L == BUNDLE ? h.pf != 0 : 9 * h.N * (int64_t)sizeof(S) > (int64_t)126 << 20;
+            const bool large = L == BUNDLE ? h.pf != 0 : h.beyond_l2;
             if (large) return launch_update(chain_tiles, k_npol<S, L, true>, grid, tile, 0, st, a);
         }
         return launch_update(chain_tiles, k_npol<S, L, false>, grid, tile, 0, st, a);
@@ -1869,7 +1869,7 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         }
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h) && !(h.tile_x & 1))
-                return launch_update(chain && spread_evenly(grid, dim3(h.tile_x / 2, h.tile_y)),
+                return launch_update(chain && spread_evenly(grid, dim3(h.tile_x / 2, h.tile_y), h.sms),
                                      k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st, a);
         }
         // Two nodes per thread on request (4- and 8-byte storage): one node
