@@ -118,7 +118,8 @@ typedef enum {
                                        pulled by the blocks launched next (default: on for
                                        32-bit storage in the stream and bundle layouts,
                                        NPOL in the bundle layout, when a lattice exceeds the
-                                       L2 cache) */
+                                       L2 cache; in a batch, LPTL/NPTL, when its lattices
+                                       together do, each case for itself) */
 #define LBM_FLAG_NO_PAIRS 0x20u  /* LPTL/NPTL, F16S/BF16S storage: one node per thread
                                     with scalar FP32 arithmetic (default when nx is even,
                                     the layout is bundle and tile_x is even: two

@@ -101,7 +101,6 @@ struct lbm_batch {
     int grid;
     bool draws;    // some case uses stochastic rounding (the update counter's only reader)
     int kind;      // layout * 4 + algo shared by every case, -1 if mixed
-    int pf;        // L2 prefetch within the work items: the lattices exceed the L2 cache
     int cur;
     int64_t steps;
     cudaGraphExec_t graph[2];
@@ -159,6 +158,12 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
         return lbm_cuda_fail(e, "cudaStreamCreateWithFlags");
     }
     const size_t rec = B->ops->batch_case_bytes;
+    // L2 prefetch within the work items where the source lattices together exceed
+    // the L2 cache, in the cases that do not decline it
+    const int64_t l2 = device_size().l2;
+    double lattices = 0.0;
+    for (int c = 0; c < ncases; ++c) lattices += 9.0 * (double)B->bl.plans[c].N * (double)B->ops->elem;
+    const bool beyond_l2 = l2 > 0 && lattices > (double)l2;
     std::vector<unsigned char> recs(4 * rec * ncases);
     std::vector<uint32_t> tiles;
     tiles.reserve(2 * (size_t)B->bl.ntiles);
@@ -172,7 +177,9 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
         B->cases.push_back(L);
         L->h.err = B->err;        // one divergence flag and update counter for the batch
         L->h.tctr = B->tctr;
-        for (int m = 0; m < 4; ++m) B->ops->batch_case(L->h, m & 1, m >> 1, recs.data() + ((size_t)m * ncases + c) * rec);
+        const int pf = beyond_l2 && !(params[c].flags & LBM_FLAG_NO_PREFETCH) ? 1 : 0;
+        for (int m = 0; m < 4; ++m)
+            B->ops->batch_case(L->h, m & 1, m >> 1, pf, recs.data() + ((size_t)m * ncases + c) * rec);
         const int64_t nt = case_tiles(params[c], B->bl.plans[c]);
         for (int64_t t = 0; t < nt; ++t) {
             tiles.push_back((uint32_t)c);
@@ -193,10 +200,6 @@ extern "C" lbm_status lbm_batch_create(int32_t ncases, const lbm_params *params,
     B->kind = params[0].layout * 4 + params[0].algo;
     for (int c = 1; c < ncases; ++c)
         if (params[c].layout * 4 + params[c].algo != B->kind) B->kind = -1;
-    double lattices = 0.0;   // bytes of the source lattices
-    for (int c = 0; c < ncases; ++c) lattices += 9.0 * (double)B->bl.plans[c].N * (double)B->ops->elem;
-    const int64_t l2 = device_size().l2;
-    B->pf = l2 > 0 && lattices > (double)l2 && !(params[0].flags & LBM_FLAG_NO_PREFETCH) ? 1 : 0;
     const int g = B->ops->batch_grid(B->kind);
     B->grid = (int)std::max<int64_t>(1, std::min<int64_t>(g > 0 ? g : 152, B->bl.ntiles));
     *out = B;
@@ -218,7 +221,7 @@ static cudaError_t batch_block(lbm_batch *B, cudaStream_t st, int64_t count, int
     int cur = B->cur;
     for (int64_t k = 0; k < count; ++k) {
         cudaError_t e = B->ops->batch_step(B->kind, B->d_cases, B->ncases, B->d_tiles, B->bl.ntiles, B->grid, cur,
-                                           (int)k, (want_moments && k == count - 1) ? 1 : 0, B->pf, st);
+                                           (int)k, (want_moments && k == count - 1) ? 1 : 0, st);
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }

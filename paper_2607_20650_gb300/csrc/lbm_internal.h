@@ -122,11 +122,12 @@ struct Ops {
     // Batches: one persistent launch over the packed tile list.
     // kind = layout * 4 + algo shared by every case, or -1 for a mixed batch.
     // recs: 4 ncases records (two lattice parities without, then with moments);
-    // cur: the parity; pf: L2 prefetch of the next tile's records.
+    // cur: the parity.
     cudaError_t (*batch_step)(int kind, const void *recs, int ncases, const void *tiles, uint32_t ntiles, int grid,
-                              int cur, int toff, int want_moments, int pf, cudaStream_t);
+                              int cur, int toff, int want_moments, cudaStream_t);
     int (*batch_grid)(int kind);                           // resident blocks on the device
-    void (*batch_case)(const HostArgs &, int parity, int moments, void *out);   // one device record
+    // One device record; pf: L2 prefetch of the next tile's records.
+    void (*batch_case)(const HostArgs &, int parity, int moments, int pf, void *out);
     size_t batch_case_bytes;
     size_t elem;               // bytes per stored population
     size_t compute;            // bytes per compute value

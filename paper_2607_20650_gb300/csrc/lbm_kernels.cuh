@@ -1420,6 +1420,7 @@ struct BatchCase {
     Step<S> st;                    // constants, links, pointers, tile shape of the case
     unsigned long long ntx_magic;  // ceil(2^64 / ntx), 0 when ntx == 1
     int layout, algo;
+    int pf;                        // L2 prefetch of the next tile's records
 };
 
 struct BatchTile {
@@ -1429,11 +1430,11 @@ struct BatchTile {
 
 // stage(): called once during the item, by every thread.
 template <class S, int L, class Stage>
-__device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uint32_t t, int tid, int pf,
+__device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uint32_t t, int tid,
                                            unsigned char *smem, Stage stage) {
     const Step<S> &a = bc.st;
     const int lane = tid & 31;
-    const bool ahead = sizeof(S) == 4 && L != COLLISION && pf != 0;
+    const bool ahead = sizeof(S) == 4 && L != COLLISION && bc.pf != 0;
     if (algo == LPTL) {
         // each tile's link bytes are loaded one tile ahead (256 channels 74.3 ->
         // 77.7 GLUPS, 71.8 before the pulls above)
@@ -1488,7 +1489,7 @@ __device__ __forceinline__ void batch_item(const BatchCase<S> &bc, int algo, uin
 // together at update 0, so they share the parity).
 template <class S, int LK, int AK>
 __global__ void __launch_bounds__(kBatchThreads, LK < 0 ? 2 : (AK <= NPTL ? (sizeof(S) == 8 ? 4 : 6) : 3))
-    k_batch(const BatchCase<S> *recs, const BatchTile *tiles, uint32_t ntiles, int toff, int pf) {
+    k_batch(const BatchCase<S> *recs, const BatchTile *tiles, uint32_t ntiles, int toff) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ __align__(16) BatchCase<S> buf[2];
     constexpr int kWords = (int)(sizeof(BatchCase<S>) / 4);
@@ -1527,9 +1528,9 @@ __global__ void __launch_bounds__(kBatchThreads, LK < 0 ? 2 : (AK <= NPTL ? (siz
         const int algo = AK >= 0 ? AK : bc.algo;
         const int layout = LK >= 0 ? LK : bc.layout;
         switch (layout) {
-            case STREAM: batch_item<S, STREAM>(bc, algo, bt.t, tid, pf, smem, stage); break;
-            case BUNDLE: batch_item<S, BUNDLE>(bc, algo, bt.t, tid, pf, smem, stage); break;
-            default: batch_item<S, COLLISION>(bc, algo, bt.t, tid, pf, smem, stage); break;
+            case STREAM: batch_item<S, STREAM>(bc, algo, bt.t, tid, smem, stage); break;
+            case BUNDLE: batch_item<S, BUNDLE>(bc, algo, bt.t, tid, smem, stage); break;
+            default: batch_item<S, COLLISION>(bc, algo, bt.t, tid, smem, stage); break;
         }
         if (wn >= ntiles) return;
         if (change) arrive();
@@ -1553,13 +1554,13 @@ size_t batch_smem_bytes(bool nsol) {   // NSOL stages its tile
 
 template <class S>
 cudaError_t op_batch_step(int kind, const void *recs, int ncases, const void *tiles, uint32_t ntiles, int grid, int cur,
-                          int toff, int want_moments, int pf, cudaStream_t st) {
+                          int toff, int want_moments, cudaStream_t st) {
     const size_t sm = batch_smem_bytes<S>(kind < 0 || kind % 4 == NSOL);
     const auto *c = (const BatchCase<S> *)recs + (size_t)((want_moments ? 2 : 0) + cur) * ncases;
     const auto *t = (const BatchTile *)tiles;
 #define LBM_BATCH_LAUNCH(S_, L_, A_)                                                       \
     if (kind == ((L_) < 0 ? -1 : (L_) * 4 + (A_)))                                        \
-        return launch_update(sizeof(S) < 8, k_batch<S_, L_, A_>, dim3(grid), dim3(kBatchThreads), sm, st, c, t, ntiles, toff, pf);
+        return launch_update(sizeof(S) < 8, k_batch<S_, L_, A_>, dim3(grid), dim3(kBatchThreads), sm, st, c, t, ntiles, toff);
     LBM_BATCH_KINDS(LBM_BATCH_LAUNCH, S)
 #undef LBM_BATCH_LAUNCH
     return cudaErrorInvalidValue;
@@ -1590,13 +1591,14 @@ int op_batch_grid(int kind) {
 // Host: the device record of one case for a lattice parity, with or without
 // moments (pointers from its HostArgs).
 template <class S>
-void op_batch_case(const HostArgs &h, int parity, int moments, void *out) {
+void op_batch_case(const HostArgs &h, int parity, int moments, int pf, void *out) {
     BatchCase<S> c;
     memset(&c, 0, sizeof(c));
     c.st = make_step<S>(h, StepCall{h.pop[1] ? parity : 0, parity, 0, moments});
     c.ntx_magic = h.ntx > 1 ? (~0ull / (unsigned long long)h.ntx) + 1ull : 0ull;
     c.layout = h.layout;
     c.algo = h.algo;
+    c.pf = pf;
     memcpy(out, &c, sizeof(c));
 }
 

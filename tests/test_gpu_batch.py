@@ -83,3 +83,29 @@ def test_autotuned_batch_equals_single_runs():
     with pytest.raises(lbm.LbmError):
         b.init(0)
     b.close()
+
+
+def test_each_case_declines_the_prefetch_for_itself():
+    """Device records of batches beyond the L2 cache: LBM_FLAG_NO_PREFETCH of a case changes its own
+    records (one per parity and moments flag) and no other's, whichever case sets it."""
+    nx, ny, n = 2048, 1024, 3
+    masks = [np.zeros(nx * ny, np.uint8)] * n
+    base = [lbm.make_params(nx, ny, 0.8, layout="bundle", algo="lptl", storage="f32") for _ in range(n)]
+    nbytes = lbm.lbm_batch_workspace_bytes(base)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+
+    def records(declining):
+        ws[: 1 << 16].zero_()
+        ps = [lbm.make_params(nx, ny, 0.8, layout="bundle", algo="lptl", storage="f32",
+                              flags=lbm.LBM_FLAG_NO_PREFETCH if c in declining else 0) for c in range(n)]
+        h = lbm.lbm_batch_create(ps, masks, ws, nbytes, torch.cuda.current_stream().cuda_stream)[0]
+        torch.cuda.synchronize()
+        out = ws[: 1 << 14].cpu().numpy().view(np.int32).copy()   # 12 records and the first work items
+        lbm.lbm_batch_destroy(h)
+        return out
+
+    none = records(())
+    where = [np.nonzero(records((c,)) != none)[0] for c in range(n)]
+    assert all(len(w) == 4 for w in where)
+    assert len(set(np.concatenate(where))) == 4 * n
+    assert np.array_equal(np.sort(np.concatenate(where[:2])), np.nonzero(records((0, 1)) != none)[0])
