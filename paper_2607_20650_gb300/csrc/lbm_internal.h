@@ -35,6 +35,8 @@ inline bool spread_evenly(dim3 grid, dim3 block, int sms) {
     return blocks * block.x * block.y * block.z >= (int64_t)sms * 1536 || blocks <= sms / 4;
 }
 
+// (A failure also stands as the runtime's last error, as after <<< >>>; the entry
+// points of Ops and Ops3 take it from there, so that no later call reports it.)
 template <class... P, class... A>
 inline cudaError_t launch_update(bool chained, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                                  cudaStream_t st, A &&...a) {

@@ -1558,12 +1558,14 @@ cudaError_t op_batch_step(int kind, const void *recs, int ncases, const void *ti
     const size_t sm = batch_smem_bytes<S>(kind < 0 || kind % 4 == NSOL);
     const auto *c = (const BatchCase<S> *)recs + (size_t)((want_moments ? 2 : 0) + cur) * ncases;
     const auto *t = (const BatchTile *)tiles;
+    cudaError_t e = cudaErrorInvalidValue;
 #define LBM_BATCH_LAUNCH(S_, L_, A_)                                                       \
     if (kind == ((L_) < 0 ? -1 : (L_) * 4 + (A_)))                                        \
-        return launch_update(sizeof(S) < 8, k_batch<S_, L_, A_>, dim3(grid), dim3(kBatchThreads), sm, st, c, t, ntiles, toff);
+        e = launch_update(sizeof(S) < 8, k_batch<S_, L_, A_>, dim3(grid), dim3(kBatchThreads), sm, st, c, t, ntiles, toff);
     LBM_BATCH_KINDS(LBM_BATCH_LAUNCH, S)
 #undef LBM_BATCH_LAUNCH
-    return cudaErrorInvalidValue;
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
 }
 
 template <class S, int LK, int AK>
@@ -1901,12 +1903,14 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
 template <class S>
 cudaError_t op_step(const HostArgs &h, const StepCall &c, cudaStream_t st) {
     const Step<S> a = make_step<S>(h, c);
+    cudaError_t e = cudaErrorInvalidValue;
     switch (h.layout) {
-        case STREAM: return step_layout<S, STREAM>(h, a, c.rd_parity, st);
-        case BUNDLE: return step_layout<S, BUNDLE>(h, a, c.rd_parity, st);
-        case COLLISION: return step_layout<S, COLLISION>(h, a, c.rd_parity, st);
+        case STREAM: e = step_layout<S, STREAM>(h, a, c.rd_parity, st); break;
+        case BUNDLE: e = step_layout<S, BUNDLE>(h, a, c.rd_parity, st); break;
+        case COLLISION: e = step_layout<S, COLLISION>(h, a, c.rd_parity, st); break;
     }
-    return cudaErrorInvalidValue;
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
 }
 
 #define LBM_LAYOUT_SWITCH(h, CALL)                          \
