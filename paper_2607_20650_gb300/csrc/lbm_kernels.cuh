@@ -592,10 +592,8 @@ __global__ void __launch_bounds__(kMaxTileThreads, sizeof(S) == 8 ? 1 : 4) k_two
 // shares what one node per thread repeats: one 16-bit load brings both link
 // bytes, the collision runs on packed FP32 pairs (collide2: each lane is the
 // scalar collide() bit for bit), two results are rounded to 16 bits by one
-// packed conversion, and the stores are 32-bit words. A pair's values of
-// one direction are adjacent in the stream layout (i N + n, n even); in the
-// bundle layout a pair's bundle is six adjacent values (3n even), stored as
-// three words. A solid node of a pair holding a fluid one stores its zeros in
+// packed conversion, and the stores are 32-bit words: in the bundle layout a
+// pair's bundle is six adjacent values (3n even), three words. A solid node of a pair holding a fluid one stores its zeros in
 // the same words, so the pair's sector is written whole. Pairs touching the
 // domain edge take the per-node path.
 template <class S>
@@ -642,32 +640,24 @@ __device__ __forceinline__ void encode_pair(const Step<S> &a, uint32_t n, const 
     }
 }
 
-// Store the pair words of nodes n, n + 1 (n even) in layout L (STREAM or BUNDLE).
-template <class S, int L>
+// Store the pair words of nodes n, n + 1 (n even).
+template <class S>
 __device__ __forceinline__ void store_pair(S *dst, uint32_t N, uint32_t n, const uint32_t *w) {
-    if (L == STREAM) {
 #pragma unroll
-        for (int i = 0; i < 9; ++i) *reinterpret_cast<uint32_t *>(dst + (uint32_t)i * N + n) = w[i];
-    } else {
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            uint32_t *p = reinterpret_cast<uint32_t *>(dst + (uint32_t)b * 3u * N + 3u * n);
-            const uint32_t w0 = w[3 * b], w1 = w[3 * b + 1], w2 = w[3 * b + 2];
-            p[0] = (w0 & 0xFFFFu) | (w1 << 16);            // (a, 3b), (a, 3b+1)
-            p[1] = (w2 & 0xFFFFu) | (w0 & 0xFFFF0000u);    // (a, 3b+2), (b, 3b)
-            p[2] = (w1 >> 16) | (w2 & 0xFFFF0000u);        // (b, 3b+1), (b, 3b+2)
-        }
+    for (int b = 0; b < 3; ++b) {
+        uint32_t *p = reinterpret_cast<uint32_t *>(dst + (uint32_t)b * 3u * N + 3u * n);
+        const uint32_t w0 = w[3 * b], w1 = w[3 * b + 1], w2 = w[3 * b + 2];
+        p[0] = (w0 & 0xFFFFu) | (w1 << 16);            // (a, 3b), (a, 3b+1)
+        p[1] = (w2 & 0xFFFFu) | (w0 & 0xFFFF0000u);    // (a, 3b+2), (b, 3b)
+        p[2] = (w1 >> 16) | (w2 & 0xFFFF0000u);        // (b, 3b+1), (b, 3b+2)
     }
 }
 
-// L2 prefetch of a pair's source records (both nodes): one address per
-// bundle, or per direction in the stream layout.
-template <class S, int L>
+// L2 prefetch of a pair's source records (both nodes): one address per bundle.
+template <class S>
 __device__ __forceinline__ void prefetch_pair(const S *src, uint32_t N, uint32_t n) {
 #pragma unroll
-    for (int i = 0; i < 9; ++i)
-        if (L == STREAM || i % 3 == 0)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(src + addr<L>(N, n, i)));
+    for (int i = 0; i < 9; i += 3) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + addr<BUNDLE>(N, n, i)));
 }
 
 // The lower / upper 16-bit value of a word.
@@ -738,35 +728,19 @@ __device__ __forceinline__ void pull_pair(const Step<S> &a, uint32_t n, uint32_t
 }
 
 // One pair: both link bytes in lk2 (node n in the low byte).
-template <class S, int L>
-__device__ __forceinline__ void pair_update(const Step<S> &a, uint32_t x, uint32_t y, uint32_t n, uint32_t lk2,
-                                            int lane) {
+template <class S>
+__device__ __forceinline__ void pair_update(const Step<S> &a, uint32_t x, uint32_t y, uint32_t n, uint32_t lk2) {
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     const uint32_t lka = lk2 & 0xFFu, lkb = lk2 >> 8;
     const bool fa = lka != SOLID_LINKS, fb = lkb != SOLID_LINKS;
-    const unsigned F = __ballot_sync(__activemask(), fa || fb);
-    if (!fa && !fb) {
-        // Stream layout: rewrite the zeros of a solid pair whose 32-byte
-        // sector (16 nodes = 8 pairs) also holds fluid nodes.
-        if (L == STREAM) {
-            const unsigned m = 0xFFu << (lane & ~7);
-            if (F & m) {
-                const uint32_t z[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-                store_pair<S, L>(a.dst, a.N, n, z);
-            }
-        }
-        return;
-    }
+    if (!fa && !fb) return;
     const bool interior = (x - 1u < nx - 3u) && (y - 1u < ny - 2u);
     if (!interior || !a.off32) {
-        if (fa) two_lattice_fluid<S, L>(a, x, y, n, lka);
-        else if (L == STREAM) store_zero<S, L>(a.dst, a.N, n, a.off32);
-        if (fb) two_lattice_fluid<S, L>(a, x + 1u, y, n + 1u, lkb);
-        else if (L == STREAM) store_zero<S, L>(a.dst, a.N, n + 1u, a.off32);
+        if (fa) two_lattice_fluid<S, BUNDLE>(a, x, y, n, lka);
+        if (fb) two_lattice_fluid<S, BUNDLE>(a, x + 1u, y, n + 1u, lkb);
         return;
     }
     f2 g[9];
-    static_assert(L == BUNDLE, "pairs are used in the bundle layout");
     pull_pair<S>(a, n, lka, lkb, g);
     f2 drho2, ux2, uy2;
     collide2(a.k2, a.k.force, g, drho2, ux2, uy2);
@@ -790,7 +764,7 @@ __device__ __forceinline__ void pair_update(const Step<S> &a, uint32_t x, uint32
             a.mom[2 * a.N + m] = fa ? v0 : v1;
         }
     }
-    if (L == BUNDLE && fa && fb && !a.sr) {
+    if (fa && fb && !a.sr) {
         // both fluid, nearest rounding: each 32-bit word of a bundle pair is
         // one packed conversion of the two values it holds
 #pragma unroll
@@ -808,7 +782,7 @@ __device__ __forceinline__ void pair_update(const Step<S> &a, uint32_t x, uint32
     }
     uint32_t w[9];
     encode_pair<S>(a, n, g, fa, fb, w);
-    store_pair<S, L>(a.dst, a.N, n, w);
+    store_pair<S>(a.dst, a.N, n, w);
 }
 
 // a.pf: L2 prefetch distance as for the 32-bit kernel (pairs of nodes for
@@ -821,7 +795,7 @@ __device__ __forceinline__ void pair_update(const Step<S> &a, uint32_t x, uint32
 #ifndef LBM_PAIR_MINB
 #define LBM_PAIR_MINB 5
 #endif
-template <class S, int L, bool LINEAR>
+template <class S, bool LINEAR>
 __global__ void __launch_bounds__(kMaxTileThreads / 2, LBM_PAIR_MINB) k_two_lattice_pair(const Step<S> a) {
     const uint32_t nx = (uint32_t)a.geo.nx, ny = (uint32_t)a.geo.ny;
     uint32_t x, y, n, np;
@@ -845,8 +819,8 @@ __global__ void __launch_bounds__(kMaxTileThreads / 2, LBM_PAIR_MINB) k_two_latt
     const uint32_t lkp = ahead ? (uint32_t)*reinterpret_cast<const unsigned short *>(a.links + np) : 0xFFFFu;
     const uint32_t lk2 = *reinterpret_cast<const unsigned short *>(a.links + n);
     chain_wait();
-    pair_update<S, L>(a, x, y, n, lk2, (int)((threadIdx.y * blockDim.x + threadIdx.x) & 31u));
-    if (lkp != 0xFFFFu) prefetch_pair<S, L>(a.src, a.N, np);
+    pair_update<S>(a, x, y, n, lk2);
+    if (lkp != 0xFFFFu) prefetch_pair<S>(a.src, a.N, np);
 }
 
 // ------------------------------------------------------------ buffer grid
@@ -1836,7 +1810,7 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h)) {
                 const dim3 b(128), g((unsigned)((h.N / 2 + 127) / 128));
-                return launch_update(chain && spread_evenly(g, b, h.sms), k_two_lattice_pair<S, L, true>, g, b, 0, st, a);
+                return launch_update(chain && spread_evenly(g, b, h.sms), k_two_lattice_pair<S, true>, g, b, 0, st, a);
             }
         }
         const int b = h.block_1d;
@@ -1874,7 +1848,7 @@ cudaError_t step_layout(const HostArgs &h, const Step<S> &a0, int phase, cudaStr
         if constexpr (sizeof(S) == 2 && L == BUNDLE) {
             if (pairs_ok<S, L>(h) && !(h.tile_x & 1))
                 return launch_update(chain && spread_evenly(grid, dim3(h.tile_x / 2, h.tile_y), h.sms),
-                                     k_two_lattice_pair<S, L, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st, a);
+                                     k_two_lattice_pair<S, false>, grid, dim3(h.tile_x / 2, h.tile_y), 0, st, a);
         }
         // Two nodes per thread on request (4- and 8-byte storage): one node
         // per thread at 32 registers keeps full occupancy and measured faster.
