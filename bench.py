@@ -177,23 +177,35 @@ def max_over_ranks(value: float, device: str) -> float:
     return float(t.item())
 
 
-def kernel_name(args, tile=(32, 4)) -> str:
-    """The update kernel as ncu lists it (layout as its enum value: stream 0,
-    bundle 1, collision 2)."""
-    t = {"f32": "float", "f64": "double", "f16s": "__half", "bf16s": "__nv_bfloat16"}[args.storage]
+def kernel_name(args, tile=(32, 4), aux: int = 0, l2: int = 0) -> str:
+    """The update kernel's instantiation, template arguments in the order of
+    csrc/lbm_kernels.cuh (layout as its enum value: stream 0, bundle 1,
+    collision 2). aux: what the lattice reports (its L2 prefetch distance;
+    NSOL: staging by tensor copies); l2: bytes of the L2 cache."""
+    t, elem = {"f32": ("float", 4), "f64": ("double", 8), "f16s": ("__half", 2),
+               "bf16s": ("__nv_bfloat16", 2)}[args.storage]
     lay = {"stream": 0, "bundle": 1, "collision": 2}[args.layout]
-    pairs = (args.storage in ("f16s", "bf16s") and args.layout == "bundle" and args.nx % 2 == 0
-             and not (getattr(args, "flags", 0) & 0x20))
+    flags, n = getattr(args, "flags", 0), args.nx * args.ny
+    pairs = elem == 2 and lay == 1 and args.nx % 2 == 0 and not flags & 0x20 and 9 * n < 1 << 32
+    # above 4M nodes (AA in the bundle layout: 128K) a kernel is compiled without the chained launches' wait
+    chain = str(n <= 4 << 20).lower()
     if args.algo == "lptl":
-        return f"k_two_lattice_pair<{t}, {lay}, true>" if pairs else f"k_two_lattice<{t}, {lay}, true>"
+        return f"k_two_lattice_pair<{t}, true>" if pairs else f"k_two_lattice<{t}, {lay}, true, {chain}>"
     if args.algo == "nptl":
+        if lay == 2 and tile[0] % 32 == 0 and not flags & 4:
+            return f"k_two_lattice_aos<{t}, {chain}>"
         if pairs and tile[0] % 2 == 0:
-            return f"k_two_lattice_pair<{t}, {lay}, false>"
-        if args.layout == "collision" and tile[0] % 32 == 0:
-            return f"k_two_lattice_aos<{t}>"
-        return f"k_two_lattice<{t}, {lay}, false>"
-    return {"npol": f"k_npol<{t}, {lay}>", "nsol": f"k_nsol<{t}, {lay}>",
-            "aa": f"k_aa<{t}, {lay}, 0|1> (two phases)"}[args.algo]
+            return f"k_two_lattice_pair<{t}, false>"
+        if flags & 2 and elem >= 4 and tile[1] >= 2 and tile[1] % 2 == 0:
+            return f"k_two_lattice2<{t}, {lay}>"
+        return f"k_two_lattice<{t}, {lay}, false, {chain}>"
+    if args.algo == "npol":
+        large = elem == 4 and (aux > 0 if lay == 1 else lay == 0 and 0 < l2 < 9 * n * elem)
+        return f"k_npol<{t}, {lay}, {str(large).lower()}>"
+    if args.algo == "nsol":
+        return f"k_nsol_tma<{t}, {lay}>" if aux else f"k_nsol<{t}, {lay}>"
+    chain = str(n <= (4 << 20 if lay != 1 else 1 << 17)).lower()
+    return f"k_aa<{t}, {lay}, 0|1, {chain}> (two phases)"
 
 
 def launches_for(k: int, graph_block: int = 64, counter: bool = True) -> int:
@@ -381,7 +393,8 @@ def run_ours(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm, "traffic": traffic, "peak_kind": peak_kind,
                      "algorithmic_bytes_per_launch": info["bytes_per_update"],
-                     "kernel": kernel_name(args, tile)},
+                     "kernel": kernel_name(args, tile, info["aux"],
+                                            torch.cuda.get_device_properties(local).L2_cache_size)},
         "clocks": clocks,
         "mlups_fluid": info["fluid_cells"] * args.steps * world / dt / 1e6,
     }

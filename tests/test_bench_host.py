@@ -71,3 +71,29 @@ def test_reference_arm_json_line():
     assert d["config"]["workload"].startswith("porous 2048x1024") and "seed 33" in d["config"]["workload"]
     assert d["config"]["stands_in_for"] == bench.WORKLOAD
     assert d["e2e"] == {"value": d["value"], "unit": "MLUPS", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}
+
+
+@pytest.mark.parametrize("algo,layout,storage,nx,kw,name", [
+    ("nptl", "bundle", "f32", 16384, {}, "k_two_lattice<float, 1, false, false>"),
+    ("lptl", "stream", "f64", 512, {}, "k_two_lattice<double, 0, true, true>"),
+    ("nptl", "bundle", "f16s", 512, {}, "k_two_lattice_pair<__half, false>"),
+    ("nptl", "bundle", "bf16s", 511, {}, "k_two_lattice<__nv_bfloat16, 1, false, true>"),
+    ("nptl", "collision", "f32", 16384, {}, "k_two_lattice_aos<float, false>"),
+    ("npol", "bundle", "f32", 16384, {"aux": 24}, "k_npol<float, 1, true>"),
+    ("npol", "stream", "f32", 16384, {"l2": 1 << 27}, "k_npol<float, 0, true>"),
+    ("npol", "stream", "f16s", 16384, {"l2": 1 << 27}, "k_npol<__half, 0, false>"),
+    ("nsol", "bundle", "f32", 512, {"aux": 1}, "k_nsol_tma<float, 1>"),
+    ("aa", "bundle", "f32", 512, {}, "k_aa<float, 1, 0|1, false> (two phases)"),
+])
+def test_kernel_name_has_the_template_arguments_of_the_source(algo, layout, storage, nx, kw, name):
+    """The name's argument count is that of the kernel's template list in the source."""
+    import argparse
+    import re
+    args = argparse.Namespace(algo=algo, layout=layout, storage=storage, nx=nx, ny=1024, flags=0)
+    assert bench.kernel_name(args, **kw) == name
+    kernel, given = re.match(r"(\w+)<(.*)>", name).groups()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    with open(os.path.join(root, "paper_2607_20650_gb300", "csrc", "lbm_kernels.cuh")) as f:
+        src = f.read()
+    params = re.findall(r"template <([^<>]*)>\s*__global__[^;{]*?\b%s\(" % kernel, src)
+    assert len(params) == 1 and len(params[0].split(",")) == len(given.split(","))
