@@ -474,9 +474,11 @@ __device__ __forceinline__ void collide_ops(const Relax<float> &k, int force, fl
 //   cu_i (3 + 9/2 cu_i) = c (9/2 c + 3 sg),  cF_i (3 + 9 cu_i) = cF+ (9 c + 3 sg)
 // with cF+ = sg cF_i, so no operand is negated at run time and one node and a
 // packed pair perform the same rounded operations. 92 operations, 64 without a
-// force (NF). The force enters after the relaxation: with (1 - omega/2)/omega F in P,
-// 73 operations, the node pairs take the same time (8192 x 4096 porous nodes, 16
-// updates: 3.57 against 3.59 ms), and the form overflows where tau F does.
+// force (NF). The force enters after the relaxation: with (1 - omega/2)/omega F in P
+// and shared even parts, 73 operations, an update is 1 to 5 % faster (8192 x 4096 porous
+// nodes, FP16, us, this order / that: node pairs 32 x 8 205 / 203, LPTL 221 / 211, one
+// node 253 / 243, NPOL 367 / 352, AA 267 / 260), but that form moves stored 16-bit values to
+// their neighbours and overflows where tau F does.
 template <bool NF, class T>
 __device__ __forceinline__ void collide_narrow(const NarrowRelax<T> &q, T *g, T &drho, T &ux, T &uy) {
     using A = Op<T>;

@@ -678,8 +678,8 @@ __device__ __forceinline__ float upper(uint32_t w) {
 // bundle bring them; where a lane of the warp bounces, the pair's own nine words
 // (three of them are among the others) hold the values that replace them. No
 // address is selected per direction and node, and a solid node, all of whose
-// links bounce, yields the zeros it holds. FP16, 8192 x 4096 porous nodes: 213 ->
-// 209 us an update (eighteen 16-bit loads through selected addresses before).
+// links bounce, yields the zeros it holds. FP16, 8192 x 4096 porous nodes, 16
+// updates: 3.91 -> 3.59 ms (eighteen 16-bit loads through selected addresses before).
 template <class S>
 __device__ __forceinline__ void pull_pair(const Step<S> &a, uint32_t n, uint32_t lka, uint32_t lkb, f2 *g) {
     const uint32_t N3 = 3u * a.N, nx3 = 3u * (uint32_t)a.geo.nx;

@@ -4,8 +4,9 @@ On a lattice larger than L2, states after the same updates with and without
 the prefetch (LBM_FLAG_NO_PREFETCH) must be bit-identical for every kernel
 that carries it, and the distance the library reports must be the one it
 documents: 5/4 of the device's resident threads, in nodes (LPTL) or rows
-(NPTL, AA). Kernels without it (16-bit storage, the collision layout, FP64,
-NPOL) and lattices that fit in L2 report 0."""
+(NPTL, AA). Kernels without it (16-bit storage but for node pairs, the
+collision layout, FP64, NPOL off the bundle layout) and lattices that fit in
+L2 report 0."""
 import numpy as np
 import pytest
 

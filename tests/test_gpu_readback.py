@@ -1,13 +1,12 @@
 """Host read-back of the moments through the C ABI.
 
 lbm_read_moments takes one of four routes: FP64 moments are copied as they
-are; FP32 moments are widened to FP64 either by the device straight into a
-page-locked destination, or on the host for a pageable one: through an
-unpinned buffer for a field of up to 64 MB, through two page-locked staging
-chunks of 64 MB beyond that. Every route must give the device's moments
-exactly (widening FP32 to FP64 is exact), including a lattice whose fields
-span several staging chunks with a ragged tail, and a call that asks for one
-field only."""
+are; FP32 moments are widened to FP64 by the device straight into a
+page-locked destination, by the device into page-locked slots for other
+fields of 8 MB and more, and on the host for smaller ones. Every route must
+give the device's moments exactly (widening FP32 to FP64 is exact), including
+a lattice whose fields span many turns of the ring of slots with a ragged
+tail, and a call that asks for one field only."""
 import numpy as np
 import pytest
 
@@ -31,8 +30,8 @@ def _pinned(N):
     return [torch.empty(N, dtype=torch.float64, pin_memory=True).numpy() for _ in range(3)]
 
 
-# 96 x 40: one partial chunk; 6144 x 5600 = 34,406,400 values per field:
-# two full chunks of 16,777,216 FP32 values and a tail of 851,968.
+# 96 x 40: on the host; 6144 x 5600 = 34,406,400 values per field: 131 full
+# chunks of 262,144 doubles and a tail of 65,536.
 @pytest.mark.parametrize("nx,ny", [(96, 40), (6144, 5600)])
 @pytest.mark.parametrize("storage", ["f32", "f16s", "f64"])
 def test_read_moments_routes_agree(storage, nx, ny):

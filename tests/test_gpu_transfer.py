@@ -1,7 +1,8 @@
-"""State and moments between device and host: around the sizes from which
-pageable buffers are locked for the call (1 MB of populations, 8 MB of one
-moments field), page-locked and unaligned buffers, a read-only source, every
-layout, slot order and storage type."""
+"""State and moments between device and host: around the sizes from which they
+go through the thread's page-locked slots (1 MB of populations, 8 MB of one
+moments field), page-locked and unaligned buffers, an array that numpy holds
+read-only (read-only pages: test_gpu_shared_host.py), every layout, slot order
+and storage type."""
 import numpy as np
 import pytest
 
